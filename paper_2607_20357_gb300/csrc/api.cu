@@ -121,7 +121,7 @@ struct PreLayout {
   int n_pad, mt_max, qkv_cap, o_cap, gu_cap, dn_cap, attn_cap;
   int ss_slots, ks_units;
   int64_t aq_cols;  // e4m3: widest quantised activation row (0 for bf16)
-  size_t xn, q, k, v, ao, hmid, yl, ss_a, ss_b, ks_part, ks_ticket, ks_info, act, seg, qkv, o, gu, dn, attn, counts,
+  size_t xn, q, k, v, ao, hmid, yl, ss_a, ss_b, ks_part, ks_ticket, ks_info, qkv, o, gu, dn, attn, counts,
       aq, as, total;
 };
 
@@ -194,8 +194,6 @@ PreLayout pre_layout(const svl_model_desc& d, int B, int64_t t_cap) {
   const size_t nl = d.n_layers;
   L.ks_ticket = b.take(sizeof(int) * L.ks_units * 2 * nl);  // per layer and residual GEMM
   L.ks_info = b.take(sizeof(int) * 8 * nl);
-  L.act = b.take(nl * B);
-  L.seg = b.take(sizeof(int4) * nl * B);
   L.qkv = b.take(sizeof(int4) * nl * L.qkv_cap);
   L.o = b.take(sizeof(int4) * nl * L.o_cap);
   L.gu = b.take(sizeof(int4) * nl * L.gu_cap);
@@ -847,15 +845,10 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
   const int hq = d.n_heads * dh, dkv = d.n_kv_heads * dh;
   const int nl = d.n_layers;
   int* counts = at<int>(ws, L.counts);
-  if (kvx && kvx->decode) {
-    // the step's rows: embeddings of the fed tokens at their cache positions
-    Launch L0(m, SVL_TAG_PACK, s);
-    launch_decode_prep(B, d.d_model, d.vocab, kvx->tokens, kvx->cache_len, kvx->max_len,
-                       static_cast<const __nv_bfloat16*>(m->w.embed), static_cast<__nv_bfloat16*>(X),
-                       const_cast<int32_t*>(cu_seqlens), const_cast<int32_t*>(pos), m->d_status, s);
-  }
+  const bool decode = kvx && kvx->decode;
 
   ScheduleArgs sa;
+  std::memset(&sa, 0, sizeof(sa));
   sa.B = B;
   sa.L = nl;
   sa.G = d.n_groups;
@@ -877,8 +870,6 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
   sa.cu_seqlens = cu_seqlens;
   sa.layer_gate = layer_gate;
   sa.group_gate = group_gate;
-  sa.act = at<uint8_t>(ws, L.act);
-  sa.seg = at<int4>(ws, L.seg);
   sa.qkv_tiles = at<int4>(ws, L.qkv);
   sa.qkv_cap = L.qkv_cap;
   sa.qkv_count = counts;
@@ -906,10 +897,47 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
       return SVL_ERR_CUDA;
   }
   int* ks_ticket = at<int>(ws, L.ks_ticket);
-  if (cudaMemsetAsync(ks_ticket, 0, sizeof(int) * L.ks_units * 2 * nl, s) != cudaSuccess) return SVL_ERR_CUDA;
+  sa.ks_ticket = ks_ticket;
+  sa.ks_ticket_ld = L.ks_units;
+  // fused RMSNorm: per-row partial sums of squares of X (see GemmParams)
+  float* ss_a = at<float>(ws, L.ss_a);
+  float* ss_b = at<float>(ws, L.ss_b);
+  const int ss_ld = static_cast<int>(L.t_pad);
+  if (only) {
+    // a single stage needs its own list, and the sums of squares only where
+    // its input is normalised
+    static const int kind[5] = {kListQkv, kListAttn, kListO, kListGateUp, kListDown};
+    sa.n_lists = 1;
+    sa.list_kinds = static_cast<uint32_t>(kind[only->stage]);
+    sa.l0 = only->layer;
+    sa.n_layers = 1;
+    sa.ss = only->stage == SVL_LAYER_QKV ? ss_a : (only->stage == SVL_LAYER_GATEUP ? ss_b : nullptr);
+  } else {
+    sa.n_lists = decode ? 4 : 5;  // decode attends to the cache without items
+    sa.list_kinds = kListQkv | (kListO << 4) | (kListGateUp << 8) | (kListDown << 12) | (kListAttn << 16);
+    sa.n_layers = nl;
+    sa.ss = ss_a;
+    // (a single stage takes the caller's V^T as it is, decode reads none past its rows)
+    if (!decode) sa.vt = at<__nv_bfloat16>(ws, L.v);
+  }
+  sa.dkv = dkv;
+  sa.t_pad = static_cast<int>(L.t_pad);
+  sa.X = static_cast<__nv_bfloat16*>(X);
+  sa.t_cap = t_cap;
+  sa.ss_ld = ss_ld;
+  sa.ss_slots = L.ss_slots;
+  if (decode) {
+    sa.tokens = kvx->tokens;
+    sa.cache_len = kvx->cache_len;
+    sa.embed = static_cast<const __nv_bfloat16*>(m->w.embed);
+    sa.V = d.vocab;
+    sa.max_len = kvx->max_len;
+    sa.cu_out = const_cast<int32_t*>(cu_seqlens);
+    sa.pos_out = const_cast<int32_t*>(pos);
+  }
   {
     Launch L1(m, SVL_TAG_SCHEDULE, s);
-    launch_schedule(sa, s);
+    if (launch_setup(sa, s) != cudaSuccess) return SVL_ERR_CUDA;
   }
 
   __nv_bfloat16* xn = at<__nv_bfloat16>(ws, L.xn);
@@ -980,10 +1008,6 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
     p.a_scale = as;
   };
 
-  // fused RMSNorm: per-row partial sums of squares of X (see GemmParams)
-  float* ss_a = at<float>(ws, L.ss_a);
-  float* ss_b = at<float>(ws, L.ss_b);
-  const int ss_ld = static_cast<int>(L.t_pad);
   auto set_norm = [&](GemmParams& p, const float* in, float* out) {
     p.ss_in = in;
     p.ss_out = out;
@@ -1002,11 +1026,6 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
   na.Y = xn;
   na.cu_seqlens = cu_seqlens;
 
-  // V^T is read in 128-key tiles that may run past the rows written in this
-  // call; zero it once so those (masked) keys hold finite values (a single
-  // stage reads or writes the caller's V^T as it is)
-  if (!only && cudaMemsetAsync(vb, 0, sizeof(__nv_bfloat16) * static_cast<size_t>(L.t_pad) * dkv, s) != cudaSuccess)
-    return SVL_ERR_CUDA;
   AttnTcArgs aa;
   std::memset(&aa, 0, sizeof(aa));
   if (!make_map(&aa.mapQ, qb, t_cap, hq) || !make_map(&aa.mapVt, vb, dkv, L.t_pad, static_cast<uint32_t>(dh)) ||
@@ -1021,13 +1040,6 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
   aa.ldo = hq;
   aa.status = m->d_status;
 
-  {
-    // sums of squares of the input rows: for the first layer's attention
-    // norm, or for the MLP norm when a single gate/up stage runs
-    Launch L1(m, SVL_TAG_RMSNORM, s);
-    launch_norm_init(static_cast<const __nv_bfloat16*>(X), cu_seqlens, B, static_cast<int>(t_cap), d.d_model,
-                     only && only->stage == SVL_LAYER_GATEUP ? ss_b : ss_a, ss_ld, L.ss_slots, s);
-  }
   // a stage of the layer runs unless a single other stage was asked for
   auto want = [&](int l, int stage) { return !only || (only->layer == l && only->stage == stage); };
 
@@ -1048,7 +1060,12 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
       }
       {
         Launch L1(m, SVL_TAG_SCHEDULE, s);
-        launch_schedule(sa, s);
+        ScheduleArgs rest = sa;  // the lists of the layers still to run
+        rest.l0 = l;
+        rest.n_layers = nl - l;
+        rest.vt = nullptr;
+        rest.ss = nullptr;
+        if (launch_setup(rest, s) != cudaSuccess) return SVL_ERR_CUDA;
       }
     }
 
@@ -1099,7 +1116,7 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
 
     if (want(l, SVL_LAYER_ATTN)) {
     const size_t layer_kv = static_cast<size_t>(B) * (kvx ? kvx->max_len : 0) * dkv;
-    if (kvx && kvx->decode) {
+    if (decode) {
       DecAttnArgs da;
       std::memset(&da, 0, sizeof(da));
       da.B = B;
@@ -1280,7 +1297,7 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
     p.ld[0] = d.vocab;
     if ((st = launch(EPI_F32, m, SVL_TAG_LMHEAD, p, static_cast<int64_t>(p.grid_m) * p.grid_n, s)) != SVL_OK) return st;
   }
-  if (kvx && kvx->decode) {
+  if (decode) {
     Launch L1(m, SVL_TAG_LMHEAD, s);
     launch_decode_finish(B, d.vocab, logits, kvx->next_token, kvx->cache_len, kvx->max_len, s);
   } else if (kvx && kvx->cache_len) {

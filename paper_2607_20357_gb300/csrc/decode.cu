@@ -52,38 +52,6 @@ void launch_kv_store(const KvArgs& a, int t_cap, cudaStream_t s) {
   if (grid.x > 0) launch_pdl(kv_store_kernel, grid, 256, 0, s, a);
 }
 
-// Decode inputs: one row per sample (cu_seqlens = 0..B), its position is the
-// cache length, its row of X the embedding of the fed token.
-__global__ void decode_prep_kernel(int B, int D, int V, const int* tokens, const int* cache_len, int max_len,
-                                   const __nv_bfloat16* embed, __nv_bfloat16* X, int* cu_seqlens, int* pos,
-                                   uint32_t* status) {
-  pdl_trigger();
-  pdl_wait();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b = blockIdx.x * (blockDim.x >> 5) + warp;
-  if (blockIdx.x == 0 && threadIdx.x == 0) cu_seqlens[0] = 0;
-  if (b >= B) return;
-  int id = tokens[b];
-  const int len = cache_len[b];
-  if (lane == 0) {
-    cu_seqlens[b + 1] = b + 1;
-    pos[b] = len;
-    if (id < 0 || id >= V || len < 0 || len >= max_len) report(status, SVL_DEV_BAD_INDEX);
-  }
-  const bool bad = id < 0 || id >= V;
-  if (bad) id = 0;
-  const uint4* src = reinterpret_cast<const uint4*>(embed + static_cast<size_t>(id) * D);
-  uint4* dst = reinterpret_cast<uint4*>(X + static_cast<size_t>(b) * D);
-  for (int c = lane; c < D / 8; c += 32) dst[c] = bad ? make_uint4(0, 0, 0, 0) : src[c];
-}
-
-void launch_decode_prep(int B, int D, int V, const int* tokens, const int* cache_len, int max_len,
-                        const __nv_bfloat16* embed, __nv_bfloat16* X, int* cu_seqlens, int* pos, uint32_t* status,
-                        cudaStream_t s) {
-  launch_pdl(decode_prep_kernel, (B + 7) / 8, 256, 0, s, B, D, V, tokens, cache_len, max_len, embed, X, cu_seqlens,
-             pos, status);
-}
-
 // One block per (sample, query head) of an active group: the new token's
 // query against the cached keys 0..len-1 and its own key (position len),
 // softmax in float32, output row of O. The block of the first query head of
@@ -114,7 +82,7 @@ __global__ void __launch_bounds__(kDecWarps * 32, 4) decode_attn_kernel(DecAttnA
   const int kvh = h / (a.A / a.Akv);
   const int len = a.cache_len[b];
   if (len < 0 || len >= a.max_len) {
-    // full (or corrupt) cache, reported by decode_prep: the head's output is
+    // full (or corrupt) cache, reported by setup_kernel: the head's output is
     // zero, so the step's logits for this sample are defined, and nothing is
     // appended
     if (tid < DH) a.out[static_cast<size_t>(b) * a.ldo + h * DH + tid] = __float2bfloat16(0.f);

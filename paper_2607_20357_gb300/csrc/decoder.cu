@@ -1,7 +1,7 @@
 // Device-side schedule of the gated decoder (Sec. 3.2) and the row kernels
 // around the GEMMs: RMSNorm, final norm of the last rows, RoPE table.
 //
-// For every layer l the schedule kernel turns the gates into work lists, so
+// For every layer l the setup kernel turns the gates into work lists, so
 // that gated-off work is never issued and the host never learns k or T:
 //  * e_{b,l,j} = (l < P) or (layer_gate[b,l] and group_gate[b,l,j]);
 //  * consecutive samples with the same non-zero group mask form one row
@@ -19,60 +19,9 @@
 
 namespace svl {
 
-constexpr int kMaxNT = 512;
-
-struct NTile {
-  int n0, ncols, mat;
-};
-
-// Column runs of consecutive active groups, cut into tiles of `step`.
-SVL_DEVINL int build_runs(NTile* out, int cnt, int mask, int G, int width, int step, int mat) {
-  int j = 0;
-  while (j < G) {
-    if (!((mask >> j) & 1)) { ++j; continue; }
-    int j1 = j;
-    while (j1 + 1 < G && ((mask >> (j1 + 1)) & 1)) ++j1;
-    const int c0 = j * width, c1 = (j1 + 1) * width;
-    for (int n0 = c0; n0 < c1 && cnt < kMaxNT; n0 += step) out[cnt++] = {n0, min(step, c1 - n0), mat};
-    j = j1 + 1;
-  }
-  return cnt;
-}
-
-// Emits mt x nt tiles of one segment in raster bands. mband > 0: bands of
-// `mband` m-tiles, each sweeping all n-tiles while its input rows stay in L2
-// (the tiles of one n-tile follow each other, so concurrent CTAs share its
-// weights too). Otherwise bands of `nband` n-tiles, each sweeping all m-tiles
-// while its weight columns stay in L2.
-__device__ void emit_tiles(int4* tiles, int base, int cap, int r0, int r1, const NTile* nt, int n_nt, int kmask,
-                           uint32_t* status, int bm = kBM_SCHED, int nband = kNBand, int mband = 0) {
-  const int mt = (r1 - r0 + bm - 1) / bm;
-  const int total = mt * n_nt;
-  for (int t = threadIdx.x; t < total; t += blockDim.x) {
-    int mi, ni;
-    if (mband > 0) {
-      const int band = t / (mband * n_nt);
-      const int rem = t - band * mband * n_nt;
-      const int bh = min(mband, mt - band * mband);
-      ni = rem / bh;
-      mi = band * mband + rem % bh;
-    } else {
-      const int band = t / (mt * nband);
-      const int rem = t - band * mt * nband;
-      const int bw = min(nband, n_nt - band * nband);
-      mi = rem / bw;
-      ni = band * nband + rem % bw;
-    }
-    const int m0 = r0 + mi * bm;
-    const int idx = base + t;
-    if (idx >= cap) {
-      report(status, SVL_DEV_BAD_INDEX);
-      continue;
-    }
-    const NTile n = nt[ni];
-    tiles[idx] = make_int4(m0, min(m0 + bm, r1), n.n0, n.ncols | (n.mat << 16) | (kmask << 24));
-  }
-}
+constexpr int kSetupThreads = 512;
+constexpr int kSetupRows = kSetupThreads / 32;  // rows of X per block (one warp each)
+constexpr int kVtRows = 512;                    // rows of V^T per zeroing block
 
 // The persistent GEMM runs tiles in waves of num_sms. When the last wave is
 // at most half full, each of its tiles is cut into two half-width tiles
@@ -136,217 +85,333 @@ __device__ int split_k_tail(int4* tiles, int count, int cap, int num_sms, int un
   return count + r * (sp - 1);
 }
 
-// Shared-memory copies of the layer's per-sample inputs: row offsets
-// cu[0..B] and the effective group mask of every sample (bit j: group j
-// runs). Filled by the whole block, so the serial walks below read shared
-// memory only.
-struct SchedShared {
-  int* cu;
-  uint8_t* mask;
+// Shared memory of a list block: the non-empty samples of the batch in order
+// (rows [cu0, cu1), group mask: bit j set if group j runs) and the row runs of
+// the list being built with their first entry's index. Sized for B samples.
+struct ListShared {
+  int *cu0, *cu1, *r0, *r1, *off;
+  uint8_t *mask, *key;
+  int n;  // non-empty samples
+  SVL_DEVINL ListShared(int* base, int B)
+      : cu0(base), cu1(cu0 + B), r0(cu1 + B), r1(r0 + B), off(r1 + B), mask(reinterpret_cast<uint8_t*>(off + B + 1)),
+        key(mask + B), n(0) {}
+};
+size_t list_shared_bytes(int B) { return (5 * static_cast<size_t>(B) + 1) * sizeof(int) + 2 * static_cast<size_t>(B); }
+
+// Maximal runs of consecutive samples with the same non-zero key: the group
+// mask (bit < 0), or whether group `bit` runs. Fills r0, r1 and key of every
+// run; returns their number. Called by the whole block.
+__device__ int find_runs(ListShared& sh, int bit, int* s_scan) {
+  auto key = [&](int i) -> int { return bit < 0 ? sh.mask[i] : (sh.mask[i] >> bit) & 1; };
+  int nrun = 0;
+  for (int c0 = 0; c0 < sh.n; c0 += blockDim.x) {
+    const int i = c0 + static_cast<int>(threadIdx.x);
+    const int k = i < sh.n ? key(i) : 0;
+    const int start = (k && (i == 0 || key(i - 1) != k)) ? 1 : 0;
+    int total;
+    const int id = nrun + block_exclusive_scan(start, &total, s_scan) + start - 1;
+    if (start) {
+      sh.r0[id] = sh.cu0[i];
+      sh.key[id] = static_cast<uint8_t>(k);
+    }
+    if (k && (i == sh.n - 1 || key(i + 1) != k)) sh.r1[id] = sh.cu1[i];
+    nrun += total;
+  }
+  __syncthreads();
+  return nrun;
+}
+
+// off[i] = sum of count(0 .. i-1) over n entries, off[n] = the total (returned).
+template <class Count>
+__device__ int prefix_offsets(ListShared& sh, int n, int* s_scan, Count count) {
+  int acc = 0;
+  for (int c0 = 0; c0 < n; c0 += blockDim.x) {
+    const int i = c0 + static_cast<int>(threadIdx.x);
+    int total;
+    const int ex = block_exclusive_scan(i < n ? count(i) : 0, &total, s_scan);
+    if (i < n) sh.off[i] = acc + ex;
+    acc += total;
+  }
+  if (threadIdx.x == 0) sh.off[n] = acc;
+  __syncthreads();
+  return acc;
+}
+
+// The columns of a tile list's n-tiles: up to three matrices (Q, K, V), each
+// a run of columns [c0, c1) cut into tiles of `step`.
+struct ColSet {
+  int c0[3], c1[3], nt[3], step;
+  SVL_DEVINL int total() const { return nt[0] + nt[1] + nt[2]; }
+  SVL_DEVINL void set(int mat, int a, int b) {
+    c0[mat] = a;
+    c1[mat] = b;
+    nt[mat] = (b - a + step - 1) / step;
+  }
+  // n-tile ni as (n0, ncols | mat << 16)
+  SVL_DEVINL int2 tile(int ni) const {
+    const int mat = ni < nt[0] ? 0 : (ni < nt[0] + nt[1] ? 1 : 2);
+    const int k = ni - (mat > 0 ? nt[0] : 0) - (mat > 1 ? nt[1] : 0);
+    const int a = mat == 0 ? c0[0] : (mat == 1 ? c0[1] : c0[2]), b = mat == 0 ? c1[0] : (mat == 1 ? c1[1] : c1[2]);
+    const int n0 = a + k * step;
+    return make_int2(n0, min(step, b - n0) | (mat << 16));
+  }
 };
 
-SVL_DEVINL bool group_on(const SchedShared& sh, int b, int j) { return (sh.mask[b] >> j) & 1; }
-
-// Emits the tiles of an N-sparse GEMM list of layer l: for each block of
-// adjacent groups with the same on/off pattern over the non-empty samples,
-// the maximal row runs of samples where the block runs, times the block's
-// columns (`cols(j0, j1, nt)` fills the n-tiles). Returns the tile count.
-// Called by the whole block; thread 0 walks groups and samples.
-template <class Cols>
-__device__ int emit_group_runs(const ScheduleArgs& a, const SchedShared& sh, int4* tiles, int cap, NTile* nt,
-                               int* s_nnt, int* s_run, Cols cols) {
-  const int tid = threadIdx.x, B = a.B, G = a.G;
-  int off = 0;
-  int j0 = 0;
-  while (j0 < G) {
-    // the block [j0, j1]: following groups with the same pattern
-    if (tid == 0) {
-      int j1 = j0;
-      for (; j1 + 1 < G; ++j1) {
-        bool same = true;
-        for (int b = 0; b < B && same; ++b)
-          if (sh.cu[b + 1] > sh.cu[b]) same = group_on(sh, b, j1 + 1) == group_on(sh, b, j0);
-        if (!same) break;
-      }
-      s_run[2] = j1;
-      *s_nnt = cols(j0, j1, nt);
-      s_run[3] = 0;  // next sample to look at
+// Writes the tiles of the block's runs from list index `base` on, each run's
+// mt x nt tiles in raster bands. mband > 0: bands of `mband` m-tiles, each
+// sweeping all n-tiles while its input rows stay in L2 (the tiles of one n-tile
+// follow each other, so concurrent CTAs share its weights too). Otherwise bands
+// of `nband` n-tiles, each sweeping all m-tiles while its weight columns stay
+// in L2. `kmask`: tiles carry their run's key as the K mask. All tiles of all
+// runs are written by one flat loop over the block's threads (a binary search
+// finds a tile's run). Returns the number of tiles.
+__device__ int emit_runs(ListShared& sh, int nrun, int4* tiles, int base, int cap, const ColSet& cs, bool kmask,
+                         uint32_t* status, int* s_scan, int bm, int nband, int mband) {
+  const int n_nt = cs.total();
+  const int total =
+      prefix_offsets(sh, nrun, s_scan, [&](int i) { return ((sh.r1[i] - sh.r0[i] + bm - 1) / bm) * n_nt; });
+  for (int t = threadIdx.x; t < total; t += blockDim.x) {
+    int lo = 0, hi = nrun;
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (sh.off[mid] <= t) lo = mid; else hi = mid;
     }
-    __syncthreads();
-    const int j1 = s_run[2];
-    while (true) {
-      if (tid == 0) {
-        // next maximal run of non-empty samples (empty ones are transparent) where the block runs
-        int b = s_run[3], r0 = -1, r1 = -1;
-        for (; b < B; ++b) {
-          const int q0 = sh.cu[b], q1 = sh.cu[b + 1];
-          if (q1 <= q0) continue;
-          if (group_on(sh, b, j0)) {
-            if (r0 < 0) r0 = q0;
-            r1 = q1;
-          } else if (r0 >= 0) {
-            break;
-          }
-        }
-        s_run[0] = r0;
-        s_run[1] = r1;
-        s_run[3] = b;
-      }
-      __syncthreads();
-      const int r0 = s_run[0], r1 = s_run[1];
-      if (r0 < 0) break;
-      emit_tiles(tiles, off, cap, r0, r1, nt, *s_nnt, 0, a.status, a.nsparse_rows, 0, a.mband);
-      off += ((r1 - r0 + a.nsparse_rows - 1) / a.nsparse_rows) * *s_nnt;
-      __syncthreads();
+    const int u = t - sh.off[lo], r0 = sh.r0[lo], r1 = sh.r1[lo];
+    const int mt = (r1 - r0 + bm - 1) / bm;
+    int mi, ni;
+    if (mband > 0) {
+      const int band = u / (mband * n_nt);
+      const int rem = u - band * mband * n_nt;
+      const int bh = min(mband, mt - band * mband);
+      ni = rem / bh;
+      mi = band * mband + rem % bh;
+    } else {
+      const int band = u / (mt * nband);
+      const int rem = u - band * mt * nband;
+      const int bw = min(nband, n_nt - band * nband);
+      mi = rem / bw;
+      ni = band * nband + rem % bw;
     }
-    j0 = j1 + 1;
-    __syncthreads();
+    const int m0 = r0 + mi * bm;
+    const int idx = base + t;
+    if (idx >= cap) {
+      report(status, SVL_DEV_BAD_INDEX);
+      continue;
+    }
+    const int2 n = cs.tile(ni);
+    tiles[idx] = make_int4(m0, min(m0 + bm, r1), n.x, n.y | (kmask ? static_cast<int>(sh.key[lo]) << 24 : 0));
   }
-  return min(off, cap);
+  __syncthreads();  // off, r0, r1 and key are reused by the caller
+  return total;
 }
 
-__global__ void __launch_bounds__(256) schedule_kernel(ScheduleArgs a) {
-  __shared__ NTile nt[kMaxNT];
-  __shared__ int s_nseg, s_nnt;
-  __shared__ int s_heads[256];
-  __shared__ int s_run[4];
-  __shared__ int s_scan[8];  // per-warp counts of split_tail (256 threads)
+// One work list of layer l: kind kListQkv / kListGateUp (N-sparse), kListO /
+// kListDown (K-sparse) or kListAttn. Nothing here is walked by one thread:
+// runs and offsets come from block-wide scans and every entry from the flat
+// loops. (The walk by thread 0 with block barriers per run that this replaces
+// took 63 us for one layer of 16 samples with mixed masks, this 6 us; the
+// lists of a layer are built by separate blocks.)
+__device__ void build_list(const ScheduleArgs& a, int l, int kind, int* dyn) {
+  __shared__ int s_scan[32];
+  __shared__ unsigned s_neq;
+  const int tid = threadIdx.x, B = a.B, G = a.G;
+  ListShared sh(dyn, B);
+  if (tid == 0) s_neq = 0;
+  __syncthreads();
+  // the non-empty samples, and for every pair of adjacent groups whether
+  // their on/off patterns over the samples differ
+  unsigned neq = 0;
+  for (int c0 = 0; c0 < B; c0 += blockDim.x) {
+    const int b = c0 + tid;
+    int q0 = 0, q1 = 0, mask = 0;
+    if (b < B) {
+      q0 = a.tokens ? b : a.cu_seqlens[b];
+      q1 = a.tokens ? b + 1 : a.cu_seqlens[b + 1];
+      for (int j = 0; j < G; ++j) {
+        const bool e = (l < a.P) || (a.layer_gate[b * a.L + l] && a.group_gate[(b * a.L + l) * G + j]);
+        mask |= e ? (1 << j) : 0;
+      }
+    }
+    const int some = q1 > q0 ? 1 : 0;
+    int total;
+    const int i = sh.n + block_exclusive_scan(some, &total, s_scan);
+    if (some) {
+      sh.cu0[i] = q0;
+      sh.cu1[i] = q1;
+      sh.mask[i] = static_cast<uint8_t>(mask);
+      neq |= mask ^ (mask >> 1);
+    }
+    sh.n += total;
+  }
+  if (neq) atomicOr(&s_neq, neq);
+  __syncthreads();
+  neq = s_neq;
+
+  if (kind == kListQkv || kind == kListGateUp) {
+    // N-sparse: per block of adjacent groups with the same pattern, the
+    // maximal row runs of samples where the block runs times its columns
+    const bool qkv = kind == kListQkv;
+    int4* tiles = qkv ? a.qkv_tiles + static_cast<size_t>(l) * a.qkv_cap : a.gu_tiles + static_cast<size_t>(l) * a.gu_cap;
+    const int cap = qkv ? a.qkv_cap : a.gu_cap;
+    const int hq = (a.A / G) * a.dh, hk = (a.Akv / G) * a.dh;
+    int off = 0;
+    for (int j0 = 0; j0 < G;) {
+      int j1 = j0;
+      while (j1 + 1 < G && !((neq >> j1) & 1)) ++j1;
+      ColSet cs{};
+      cs.step = qkv ? 256 : 128;
+      if (qkv) {
+        cs.set(0, j0 * hq, (j1 + 1) * hq);
+        cs.set(1, j0 * hk, (j1 + 1) * hk);
+        cs.set(2, j0 * hk, (j1 + 1) * hk);
+      } else {
+        cs.set(0, j0 * (a.Di / G), (j1 + 1) * (a.Di / G));
+      }
+      const int nrun = find_runs(sh, j0, s_scan);
+      off += emit_runs(sh, nrun, tiles, off, cap, cs, false, a.status, s_scan, a.nsparse_rows, 0, a.mband);
+      j0 = j1 + 1;
+    }
+    off = min(off, cap);
+    if (qkv) off = split_tail(tiles, off, cap, a.nsparse_wave, a.dh, s_scan);
+    if (tid == 0) (qkv ? a.qkv_count : a.gu_count)[l] = off;
+  } else if (kind == kListO || kind == kListDown) {
+    // K-sparse: segments of consecutive samples with the same mask, all D
+    // columns; the tiles carry the mask
+    const bool o = kind == kListO;
+    int4* tiles = o ? a.o_tiles + static_cast<size_t>(l) * a.o_cap : a.dn_tiles + static_cast<size_t>(l) * a.dn_cap;
+    const int cap = o ? a.o_cap : a.dn_cap;
+    ColSet cs{};
+    cs.step = 256;
+    cs.set(0, 0, a.D);
+    const int nrun = find_runs(sh, -1, s_scan);
+    int off = emit_runs(sh, nrun, tiles, 0, cap, cs, true, a.status, s_scan, kBM_SCHED, o ? kNBandO : kNBand, 0);
+    off = split_k_tail(tiles, min(off, cap), cap, a.num_sms, a.ks_units,
+                       a.ks_info + static_cast<size_t>(l) * 8 + (o ? 0 : 4));
+    if (tid == 0) (o ? a.o_count : a.dn_count)[l] = off;
+    int* ticket = a.ks_ticket + (2 * static_cast<size_t>(l) + (o ? 0 : 1)) * a.ks_ticket_ld;
+    for (int i = tid; i < a.ks_ticket_ld; i += blockDim.x) ticket[i] = 0;
+  } else {
+    // attention items: per active sample and active head, blocks of kAttnQ
+    // queries, latest first (the kernel takes units from the front of the list,
+    // so one head's blocks run at about the same time and share its keys in L2)
+    int4* items = a.attn_items + static_cast<size_t>(l) * a.attn_cap;
+    const int hpg = a.A / G;
+    const int total = prefix_offsets(sh, sh.n, s_scan, [&](int i) {
+      return ((sh.cu1[i] - sh.cu0[i] + kAttnQ - 1) / kAttnQ) * __popc(sh.mask[i]) * hpg;
+    });
+    for (int t = tid; t < total; t += blockDim.x) {
+      int lo = 0, hi = sh.n;
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (sh.off[mid] <= t) lo = mid; else hi = mid;
+      }
+      const int u = t - sh.off[lo], r0 = sh.cu0[lo], r1 = sh.cu1[lo];
+      const int nq = (r1 - r0 + kAttnQ - 1) / kAttnQ;
+      const int hi_ = u / nq, qi = nq - 1 - (u - hi_ * nq);
+      int grp = hi_ / hpg;  // the grp-th active group
+      const int within = hi_ - grp * hpg;
+      int j = 0;
+      for (int m = sh.mask[lo]; j < G; ++j)
+        if (((m >> j) & 1) && grp-- == 0) break;
+      const int q0 = r0 + qi * kAttnQ;
+      if (t < a.attn_cap) items[t] = make_int4(q0, min(q0 + kAttnQ, r1), r0, j * hpg + within);
+      else report(a.status, SVL_DEV_BAD_INDEX);
+    }
+    if (tid == 0) {
+      a.attn_count[l] = min(total, a.attn_cap);
+      a.attn_next[l] = 0;
+    }
+  }
+}
+
+// Everything the first GEMM of a forward needs, in one launch:
+//   blocks [0, n_lists * n_layers): one work list of one layer each;
+//   then the V^T zeroing blocks (z_blocks per sample boundary) and the row
+//   blocks (kSetupRows rows each): sums of squares of the packed rows, and
+//   for a decode step first the rows themselves.
+// V^T: attention reads 64-key tiles that start up to 7 keys before a sample
+// and run up to 63 past its end. Those keys are masked (P = 0) but must be
+// finite, and a neighbouring sample whose group is off in a layer has none
+// written there, so the windows around every sample boundary are zeroed once
+// per call (at b = 1 and 16 samples 10 MB instead of the whole 84 MB of V^T).
+__global__ void __launch_bounds__(kSetupThreads) setup_kernel(ScheduleArgs a) {
+  extern __shared__ int setup_dyn[];
   pdl_trigger();
   pdl_wait();
-  extern __shared__ int sched_dyn[];
-  const int l = blockIdx.x, tid = threadIdx.x;
-  const int B = a.B, G = a.G;
-  int4* seg = a.seg + static_cast<size_t>(l) * B;
-  uint8_t* act = a.act + static_cast<size_t>(l) * B;
-  const SchedShared sh{sched_dyn, reinterpret_cast<uint8_t*>(sched_dyn + B + 1)};
-  for (int b = tid; b <= B; b += blockDim.x) sh.cu[b] = a.cu_seqlens[b];
-  for (int b = tid; b < B; b += blockDim.x) {
-    int mask = 0;
-    for (int j = 0; j < G; ++j) {
-      const bool e = (l < a.P) || (a.layer_gate[b * a.L + l] && a.group_gate[(b * a.L + l) * G + j]);
-      mask |= e ? (1 << j) : 0;
-    }
-    sh.mask[b] = static_cast<uint8_t>(mask);
+  int blk = blockIdx.x;
+  const int n_list_blocks = a.n_lists * a.n_layers;
+  if (blk < n_list_blocks) {
+    // layers vary fastest: the lists needed first are built first
+    const int li = blk / a.n_layers;
+    build_list(a, a.l0 + blk - li * a.n_layers, (a.list_kinds >> (4 * li)) & 15, setup_dyn);
+    return;
   }
-  __syncthreads();
-
-  if (tid == 0) {
-    int ns = 0;
-    for (int b = 0; b < B; ++b) {
-      const int mask = sh.mask[b];
-      const int r0 = sh.cu[b], r1 = sh.cu[b + 1];
-      act[b] = (mask != 0 && r1 > r0) ? 1 : 0;
-      if (mask == 0 || r1 <= r0) continue;
-      if (ns > 0 && seg[ns - 1].z == mask && seg[ns - 1].y == r0) {
-        seg[ns - 1].y = r1;
-      } else {
-        seg[ns] = make_int4(r0, r1, mask, 0);
-        ++ns;
+  blk -= n_list_blocks;
+  if (a.vt) {
+    const int zb = (a.dkv + kVtRows - 1) / kVtRows, n_z = zb * (a.B + 1);
+    if (blk < n_z) {
+      const int b = blk / zb, v0 = (blk - b * zb) * kVtRows, rows = min(kVtRows, a.dkv - v0);
+      const int c = a.cu_seqlens[b];
+      const int w0 = max(c - 8, 0) >> 3, w1 = min(c + 64 + 7, a.t_pad) >> 3, nw = w1 - w0;  // 16-byte words
+      for (int i = threadIdx.x; i < rows * nw; i += blockDim.x) {
+        const int r = i / nw, w = i - r * nw;
+        reinterpret_cast<uint4*>(a.vt + static_cast<size_t>(v0 + r) * a.t_pad)[w0 + w] = make_uint4(0, 0, 0, 0);
       }
+      return;
     }
-    s_nseg = ns;
+    blk -= n_z;
   }
-  __syncthreads();
-  const int nseg = s_nseg;
-  const int hq = (a.A / G) * a.dh, hk = (a.Akv / G) * a.dh;
-
-  // ---- QKV (N-sparse over active groups' Q, K, V columns, per group block)
-  auto qkv_cols = [&](int j0, int j1, NTile* out) {
-    const int mask = ((1 << (j1 + 1)) - 1) & ~((1 << j0) - 1);
-    int c = build_runs(out, 0, mask, G, hq, 256, 0);
-    c = build_runs(out, c, mask, G, hk, 256, 1);
-    return build_runs(out, c, mask, G, hk, 256, 2);
-  };
-  int off = emit_group_runs(a, sh, a.qkv_tiles + static_cast<size_t>(l) * a.qkv_cap, a.qkv_cap, nt, &s_nnt, s_run,
-                            qkv_cols);
-  __syncthreads();
-  off = split_tail(a.qkv_tiles + static_cast<size_t>(l) * a.qkv_cap, off, a.qkv_cap, a.nsparse_wave, a.dh, s_scan);
-  if (tid == 0) a.qkv_count[l] = off;
-
-  // ---- O projection (K-sparse: kmask = segment mask), all D columns
-  off = 0;
-  if (tid == 0) s_nnt = build_runs(nt, 0, 1, 1, a.D, 256, 0);
-  __syncthreads();
-  for (int s = 0; s < nseg; ++s) {
-    const int4 sg = seg[s];
-    emit_tiles(a.o_tiles + static_cast<size_t>(l) * a.o_cap, off, a.o_cap, sg.x, sg.y, nt, s_nnt, sg.z, a.status,
-               kBM_SCHED, kNBandO);
-    off += ((sg.y - sg.x + kBM_SCHED - 1) / kBM_SCHED) * s_nnt;
-  }
-  __syncthreads();
-  off = split_k_tail(a.o_tiles + static_cast<size_t>(l) * a.o_cap, min(off, a.o_cap), a.o_cap, a.num_sms, a.ks_units,
-                     a.ks_info + static_cast<size_t>(l) * 8);
-  if (tid == 0) a.o_count[l] = off;
-  // ---- down projection: same tiles shape as O
-  off = 0;
-  for (int s = 0; s < nseg; ++s) {
-    const int4 sg = seg[s];
-    emit_tiles(a.dn_tiles + static_cast<size_t>(l) * a.dn_cap, off, a.dn_cap, sg.x, sg.y, nt, s_nnt, sg.z, a.status);
-    off += ((sg.y - sg.x + kBM_SCHED - 1) / kBM_SCHED) * s_nnt;
-  }
-  __syncthreads();
-  off = split_k_tail(a.dn_tiles + static_cast<size_t>(l) * a.dn_cap, min(off, a.dn_cap), a.dn_cap, a.num_sms,
-                     a.ks_units, a.ks_info + static_cast<size_t>(l) * 8 + 4);
-  if (tid == 0) a.dn_count[l] = off;
-  __syncthreads();
-
-  // ---- gate/up (N-sparse over active FFN channels, 128 per tile, per group block)
-  auto gu_cols = [&](int j0, int j1, NTile* out) {
-    const int mask = ((1 << (j1 + 1)) - 1) & ~((1 << j0) - 1);
-    return build_runs(out, 0, mask, G, a.Di / G, 128, 0);
-  };
-  off = emit_group_runs(a, sh, a.gu_tiles + static_cast<size_t>(l) * a.gu_cap, a.gu_cap, nt, &s_nnt, s_run, gu_cols);
-  __syncthreads();
-  if (tid == 0) a.gu_count[l] = off;
-
-  // ---- attention items: per active sample and active head, blocks of kAttnQ
-  // queries, latest first (the kernel takes units from the front of the list,
-  // so one head's blocks run at about the same time and share its keys in L2)
-  off = 0;
-  int4* items = a.attn_items + static_cast<size_t>(l) * a.attn_cap;
-  const int hpg = a.A / G;
-  for (int s = 0; s < nseg; ++s) {
-    const int4 sg = seg[s];
-    if (tid == 0) {
-      int nh = 0;
-      for (int j = 0; j < G; ++j)
-        if ((sg.z >> j) & 1)
-          for (int h = 0; h < hpg && nh < 256; ++h) s_heads[nh++] = j * hpg + h;
-      s_nnt = nh;
+  if (!a.ss) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int r = blk * kSetupRows + warp;
+  __nv_bfloat16* x = a.X + static_cast<size_t>(r) * a.D;
+  const uint4* src = reinterpret_cast<const uint4*>(x);
+  bool bad = false;
+  if (a.tokens) {
+    // decode: row b is the embedding of the fed token at position cache_len[b]
+    if (blk == 0 && threadIdx.x == 0) a.cu_out[0] = 0;
+    if (r >= a.B) return;
+    const int id = a.tokens[r], len = a.cache_len[r];
+    bad = id < 0 || id >= a.V;
+    if (lane == 0) {
+      a.cu_out[r + 1] = r + 1;
+      a.pos_out[r] = len;
+      if (bad || len < 0 || len >= a.max_len) report(a.status, SVL_DEV_BAD_INDEX);
     }
-    __syncthreads();
-    const int nh = s_nnt;
-    // samples inside the segment
-    int lo = 0, hi = B;
-    while (hi - lo > 1) {  // first sample of the segment
-      const int mid = (lo + hi) >> 1;
-      if (sh.cu[mid] <= sg.x) lo = mid; else hi = mid;
-    }
-    for (int b = lo; b < B && sh.cu[b] < sg.y; ++b) {
-      const int r0 = sh.cu[b], r1 = sh.cu[b + 1];
-      if (r1 <= r0) continue;
-      const int nq = (r1 - r0 + kAttnQ - 1) / kAttnQ;
-      const int total = nq * nh;
-      for (int t = tid; t < total; t += blockDim.x) {
-        const int qi = nq - 1 - t % nq;
-        const int h = s_heads[t / nq];
-        const int q0 = r0 + qi * kAttnQ;
-        const int idx = off + t;
-        if (idx < a.attn_cap) items[idx] = make_int4(q0, min(q0 + kAttnQ, r1), r0, h);
-        else report(a.status, SVL_DEV_BAD_INDEX);
-      }
-      off += total;
-    }
-    __syncthreads();
+    src = reinterpret_cast<const uint4*>(a.embed + static_cast<size_t>(bad ? 0 : id) * a.D);
+  } else if (r >= a.cu_seqlens[a.B] || r >= a.t_cap) {
+    return;
   }
-  if (tid == 0) {
-    a.attn_count[l] = min(off, a.attn_cap);
-    a.attn_next[l] = 0;
+  // sum of squares of the row into slot 0 of ss ([slots][ss_ld]), the other
+  // slots zeroed: the first layer's fused RMSNorm reads these
+  float acc = 0.f;
+  for (int c = lane; c < a.D / 8; c += 32) {
+    const uint4 u = bad ? make_uint4(0, 0, 0, 0) : src[c];
+    if (a.tokens) reinterpret_cast<uint4*>(x)[c] = u;
+    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float2 f = unpack_bf16x2(w[i]);
+      acc = fmaf(f.x, f.x, fmaf(f.y, f.y, acc));
+    }
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  for (int i = lane; i < a.ss_slots; i += 32) a.ss[static_cast<size_t>(i) * a.ss_ld + r] = i == 0 ? acc : 0.f;
 }
 
-void launch_schedule(const ScheduleArgs& a, cudaStream_t s) {
-  launch_pdl(schedule_kernel, a.L, 256, static_cast<size_t>(a.B + 1) * sizeof(int) + a.B, s, a);
+cudaError_t launch_setup(const ScheduleArgs& a, cudaStream_t s) {
+  const size_t smem = list_shared_bytes(a.B);
+  if (smem > 48 * 1024) {
+    // per call: the attribute belongs to the current device's function
+    const cudaError_t e =
+        cudaFuncSetAttribute(setup_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+  }
+  const int zb = a.vt ? ((a.dkv + kVtRows - 1) / kVtRows) * (a.B + 1) : 0;
+  const int rows = a.ss ? ((a.tokens ? a.B : a.t_cap) + kSetupRows - 1) / kSetupRows : 0;
+  const int grid = a.n_lists * a.n_layers + zb + rows;
+  return grid > 0 ? launch_pdl(setup_kernel, grid, kSetupThreads, smem, s, a) : cudaSuccess;
 }
 
 // LLM-side compute controller (Sec. 3.2), one block per sample:
@@ -526,37 +591,6 @@ __global__ void final_rows_kernel(NormArgs a, int n_pad) {
     return;
   }
   norm_row(a.X + static_cast<size_t>(r1 - 1) * a.D, a.gain, y, a.D, a.eps, lane);
-}
-
-// Sum of squares of every packed row of X into slot 0 of ss ([slots][ss_ld]),
-// the other slots zeroed: the first layer's fused RMSNorm reads these.
-__global__ void norm_init_kernel(const __nv_bfloat16* X, const int* cu_seqlens, int B, int t_cap, int D, float* ss,
-                                 int ss_ld, int slots) {
-  pdl_trigger();
-  pdl_wait();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r = blockIdx.x * (blockDim.x >> 5) + warp;
-  if (r >= cu_seqlens[B] || r >= t_cap) return;
-  const uint4* xv = reinterpret_cast<const uint4*>(X + static_cast<size_t>(r) * D);
-  float acc = 0.f;
-  for (int c = lane; c < D / 8; c += 32) {
-    const uint4 u = xv[c];
-    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float2 f = unpack_bf16x2(w[i]);
-      acc = fmaf(f.x, f.x, fmaf(f.y, f.y, acc));
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  for (int i = lane; i < slots; i += 32) ss[static_cast<size_t>(i) * ss_ld + r] = i == 0 ? acc : 0.f;
-}
-
-void launch_norm_init(const __nv_bfloat16* X, const int* cu_seqlens, int B, int t_cap, int D, float* ss, int ss_ld,
-                      int slots, cudaStream_t s) {
-  const int grid = (t_cap + 7) / 8;
-  if (grid > 0) launch_pdl(norm_init_kernel, grid, 256, 0, s, X, cu_seqlens, B, t_cap, D, ss, ss_ld, slots);
 }
 
 // W'[r][c] = W[r][c] * g[c] (a norm gain folded into the projection after it)

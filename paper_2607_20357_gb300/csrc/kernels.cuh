@@ -91,6 +91,33 @@ SVL_DEVINL int find_sample(const int* cu, int B, int r) {
   return lo;
 }
 
+// Exclusive block-wide prefix sum of one int per thread (blockDim.x <= 1024).
+SVL_DEVINL int block_exclusive_scan(int v, int* total, int* warp_sums) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+  int x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) warp_sums[warp] = x;
+  __syncthreads();
+  if (warp == 0) {
+    int w = lane < nw ? warp_sums[lane] : 0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      int y = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += y;
+    }
+    if (lane < nw) warp_sums[lane] = w;  // inclusive
+  }
+  __syncthreads();
+  const int base = warp > 0 ? warp_sums[warp - 1] : 0;
+  *total = warp_sums[nw - 1];
+  __syncthreads();
+  return base + x - v;
+}
+
 // ---------------------------------------------------------------- e4m3 operands
 // Per-row e4m3 quantisation of bf16 rows (times a gain vector when given:
 // the input norm's gain of the QKV and gate/up projections). Row r of src holds G groups of kg
@@ -128,9 +155,6 @@ struct KvArgs {
   __nv_bfloat16* v_cache;
 };
 void launch_kv_store(const KvArgs& a, int t_cap, cudaStream_t s);
-void launch_decode_prep(int B, int D, int V, const int* tokens, const int* cache_len, int max_len,
-                        const __nv_bfloat16* embed, __nv_bfloat16* X, int* cu_seqlens, int* pos, uint32_t* status,
-                        cudaStream_t s);
 struct DecAttnArgs {
   int B, A, Akv, dh, dkv, G, L, P, l, max_len, t_pad, ldq, ldo;
   float scale;
@@ -149,6 +173,9 @@ void launch_decode_finish(int B, int V, const float* logits, int* next_token, in
                           cudaStream_t s);
 
 // ---------------------------------------------------------------- decoder
+// Work lists of a layer (setup_kernel).
+enum ListKind : int { kListQkv = 0, kListO = 1, kListDown = 2, kListGateUp = 3, kListAttn = 4 };
+
 struct ScheduleArgs {
   int B, L, G, P;
   int num_sms;              // CTAs of the persistent GEMM (one wave of tiles)
@@ -159,20 +186,40 @@ struct ScheduleArgs {
   const int* cu_seqlens;
   const uint8_t* layer_gate;
   const uint8_t* group_gate;
+  // lists to build: n_lists kinds (4 bits each, the first in the low bits)
+  // for layers l0 .. l0 + n_layers - 1
+  int n_lists, l0, n_layers;
+  uint32_t list_kinds;
   // per-layer outputs (layer l at offset l * cap)
-  uint8_t* act;             // [L, B] sample active in layer
-  int4* seg;                // [L, B] row segments {r0, r1, mask, 0}
   int4* qkv_tiles; int qkv_cap; int* qkv_count;
   int4* o_tiles; int o_cap; int* o_count;
   int4* gu_tiles; int gu_cap; int* gu_count;
   int4* dn_tiles; int dn_cap; int* dn_count;
   int4* attn_items; int attn_cap; int* attn_count;
-  int* attn_next;           // [L] attention unit counters, zeroed here
+  int* attn_next;           // [L] attention unit counters, zeroed with the items
   int* ks_info;             // [L][2][4]: K-split tail of the O (0) and down (1) lists, see GemmParams
   int ks_units;             // most tail shares the partial buffer holds
+  int* ks_ticket;           // [L][2][ks_ticket_ld] tickets of those tails, zeroed with the lists
+  int ks_ticket_ld;
+  // V^T [dkv][t_pad], zeroed around the sample boundaries (nullptr: not)
+  __nv_bfloat16* vt;
+  int dkv, t_pad;
+  // sums of squares of the rows of X into ss [ss_slots][ss_ld] (nullptr: not)
+  __nv_bfloat16* X;
+  int t_cap;
+  float* ss;
+  int ss_ld, ss_slots;
+  // decode step: the rows of X, cu_seqlens (0..B) and positions are written
+  // here from the fed tokens (nullptr: a packed batch)
+  const int* tokens;
+  const int* cache_len;
+  const __nv_bfloat16* embed;
+  int V, max_len;
+  int* cu_out;
+  int* pos_out;
   uint32_t* status;
 };
-void launch_schedule(const ScheduleArgs& a, cudaStream_t s);
+cudaError_t launch_setup(const ScheduleArgs& a, cudaStream_t s);
 
 // Number of K shares the last wave of a residual GEMM's `count` tiles is cut
 // into (1: no split). The persistent grid has num_sms CTAs, so the last wave
@@ -230,10 +277,8 @@ struct NormArgs {
 };
 void launch_rmsnorm(const NormArgs& a, cudaStream_t s);
 
-// Fused-RMSNorm support: sums of squares of the packed rows (slot 0), norm
-// gains folded into a projection's columns, and a check for unit gains.
-void launch_norm_init(const __nv_bfloat16* X, const int* cu_seqlens, int B, int t_cap, int D, float* ss, int ss_ld,
-                      int slots, cudaStream_t s);
+// Fused-RMSNorm support: norm gains folded into a projection's columns, and a
+// check for unit gains.
 cudaError_t fold_gain(const __nv_bfloat16* W, const __nv_bfloat16* g, __nv_bfloat16* out, int64_t rows, int cols,
                       cudaStream_t s);
 cudaError_t gain_is_one(const __nv_bfloat16* g, int n, int* flag, cudaStream_t s);

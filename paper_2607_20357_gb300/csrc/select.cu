@@ -53,33 +53,6 @@ SVL_DEVINL uint32_t order_key(float z) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// Exclusive block-wide prefix sum of one int per thread (blockDim.x <= 1024).
-SVL_DEVINL int block_exclusive_scan(int v, int* total, int* warp_sums) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  int x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) warp_sums[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    int w = lane < nw ? warp_sums[lane] : 0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      int y = __shfl_up_sync(0xffffffffu, w, o);
-      if (lane >= o) w += y;
-    }
-    if (lane < nw) warp_sums[lane] = w;  // inclusive
-  }
-  __syncthreads();
-  const int base = warp > 0 ? warp_sums[warp - 1] : 0;
-  *total = warp_sums[nw - 1];
-  __syncthreads();
-  return base + x - v;
-}
-
 // One block per sample: k from the budget (largest k with Eq. 8 cost within
 // b * C_full), then the k largest logits (ties: lower index), written in
 // ascending index order to kept_local[vis_off[b] ...].
