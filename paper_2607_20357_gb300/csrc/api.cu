@@ -625,6 +625,7 @@ svl_status score_select_impl(svl_model* m, int32_t B, int32_t n_vis_total, const
     p.w2 = static_cast<const __nv_bfloat16*>(m->w.ctrl_w2);
     p.c2 = m->w.ctrl_c2;
     p.b_box_rows = d.h_ctrl;
+    p.early = 3;  // only the epilogue reads what the launch before wrote (e_b)
     st = launch(d.h_ctrl <= 64 ? EPI_SCORE : EPI_SCORE_WIDE, m, SVL_TAG_SCORE, p, p.grid_m, s);
     if (st != SVL_OK) return st;
   }
@@ -748,6 +749,8 @@ svl_status pack_impl(svl_model* m, int32_t B, int32_t n_vis_total, int32_t n_tex
     GemmParams p = base_params(m);
     if (!make_map(&p.mapA, a.stage, n_vis_total, d.c_vis)) return SVL_ERR_CUDA;
     p.mapB[0] = m->tm_proj_w1;
+    p.early = 2;
+    p.late = true;
     p.grid_m = (n_vis_total + kBM - 1) / kBM;
     p.grid_n = (d.proj_hidden + 255) / 256;
     p.bn = 256;
@@ -764,6 +767,7 @@ svl_status pack_impl(svl_model* m, int32_t B, int32_t n_vis_total, int32_t n_tex
     GemmParams q = base_params(m);
     if (!make_map(&q.mapA, at<__nv_bfloat16>(ws, L.hp), n_vis_total, d.proj_hidden)) return SVL_ERR_CUDA;
     q.mapB[0] = m->tm_proj_w2;
+    q.early = 2;
     q.grid_m = p.grid_m;
     q.grid_n = (d.d_model + 255) / 256;
     q.bn = 256;
@@ -940,6 +944,17 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
     if (launch_setup(sa, s) != cudaSuccess) return SVL_ERR_CUDA;
   }
 
+  // The weights of a GEMM may load before its predecessor has finished when
+  // that predecessor was launched late and the setup kernel, whose lists the
+  // GEMM reads, is older than it.
+  bool fresh = true, prev_late = false;  // the last launch was the setup; was late
+  auto next_launch = [&](bool late) {
+    const int early = !fresh && prev_late ? 2 : 0;
+    fresh = false;
+    prev_late = late;
+    return early;
+  };
+
   __nv_bfloat16* xn = at<__nv_bfloat16>(ws, L.xn);
   __nv_bfloat16* qb = only ? only->q : at<__nv_bfloat16>(ws, L.q);
   __nv_bfloat16* kb = only ? only->k : at<__nv_bfloat16>(ws, L.k);
@@ -994,6 +1009,8 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
       qa.P = d.n_prefix;
     }
     Launch L1(m, SVL_TAG_QUANT, s);
+    qa.late = true;
+    next_launch(true);
     return launch_quant_rows(qa, s) == cudaSuccess ? SVL_OK : SVL_ERR_CUDA;
   };
   auto set_f8 = [&](GemmParams& p, const CUtensorMap& mapA, const CUtensorMap* tm8, const float* const* sc,
@@ -1066,6 +1083,8 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
         rest.vt = nullptr;
         rest.ss = nullptr;
         if (launch_setup(rest, s) != cudaSuccess) return SVL_ERR_CUDA;
+        fresh = true;
+        prev_late = false;
       }
     }
 
@@ -1109,6 +1128,8 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
     p.mapR = map_q32;
     p.mapR2 = map_k32;
     p.stage_tma = 1;
+    p.late = false;  // attention loads nothing early
+    p.early = next_launch(p.late);
     if ((st = pair ? launch_pair(EPI_QKV_ROPE, m, SVL_TAG_QKV, p, L.qkv_cap, s)
                    : launch(EPI_QKV_ROPE, m, SVL_TAG_QKV, p, L.qkv_cap, s, f8, thin)) != SVL_OK)
       return st;
@@ -1143,6 +1164,8 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
       da.v_cache = kvx->kv + static_cast<size_t>(nl + l) * layer_kv;
       da.out = ao;
       Launch L1(m, SVL_TAG_ATTENTION, s);
+      da.late = !f8;
+      next_launch(da.late);
       launch_decode_attn(da, s);
     } else {
       if (kvx) {
@@ -1158,12 +1181,15 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
         ka.k_cache = kvx->kv + static_cast<size_t>(l) * layer_kv;
         ka.v_cache = kvx->kv + static_cast<size_t>(nl + l) * layer_kv;
         Launch L1(m, SVL_TAG_COPY, s);
+        next_launch(false);
         launch_kv_store(ka, t_cap, s);
       }
       aa.items = sa.attn_items + static_cast<size_t>(l) * L.attn_cap;
       aa.count = counts + 4 * nl + l;
       aa.next_unit = counts + 5 * nl + l;
       Launch L1(m, SVL_TAG_ATTENTION, s);
+      aa.late = !only && !f8;
+      next_launch(aa.late);
       if (launch_attention_tc(aa, gemm_grid(m, L.attn_cap), s) != cudaSuccess) return SVL_ERR_CUDA;
     }
     }
@@ -1188,6 +1214,8 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
     p.mapR = map_xr;
     p.stage_tma = 1;
     p.a_evict_first = 1;  // n-band list: the weights stay in L2, the input rows stream
+    p.late = !only && !f8;
+    p.early = next_launch(p.late);
     p.ks_info = sa.ks_info + static_cast<size_t>(l) * 8;
     p.ks_part = at<float>(ws, L.ks_part);
     p.ks_ticket = ks_ticket + static_cast<size_t>(2 * l) * L.ks_units;
@@ -1221,6 +1249,8 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
     p.ld[0] = d.d_ffn;
     p.mapR = map_hmo;
     p.stage_tma = 1;
+    p.late = !only && !f8;
+    p.early = next_launch(p.late);
     if ((st = pair ? launch_pair(EPI_SWIGLU, m, SVL_TAG_GATEUP, p, L.gu_cap, s)
                    : launch(EPI_SWIGLU, m, SVL_TAG_GATEUP, p, L.gu_cap, s, f8, thin)) != SVL_OK)
       return st;
@@ -1246,6 +1276,8 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
     p.mapR = map_xr;
     p.stage_tma = 1;
     p.a_evict_first = 1;  // n-band list: the weights stay in L2, the input rows stream
+    p.late = !only && !f8 && l + 1 < nl;
+    p.early = next_launch(p.late);
     p.ks_info = sa.ks_info + static_cast<size_t>(l) * 8 + 4;
     p.ks_part = at<float>(ws, L.ks_part);
     p.ks_ticket = ks_ticket + static_cast<size_t>(2 * l + 1) * L.ks_units;
@@ -1267,6 +1299,7 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
       launch_final_last_rows(na, n_pad, s);
     }
     p.mapA = m->tm_lm_head;
+    p.early = 1;  // the weights are A here
     if (!make_map(&p.mapB[0], na.Y, n_pad, d.d_model)) return SVL_ERR_CUDA;
     p.grid_m = (d.vocab + kBM - 1) / kBM;
     p.grid_n = (n_pad + 255) / 256;
@@ -1285,6 +1318,7 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
     }
     p.mapA = map_xn;
     p.mapB[0] = m->tm_lm_head;
+    p.early = 2;
     p.grid_m = (t_cap + kBM - 1) / kBM;
     p.grid_n = (d.vocab + 255) / 256;
     p.bn = 256;
@@ -1716,6 +1750,7 @@ extern "C" svl_status svl_score_select_noalloc(svl_model* m, int32_t B, int32_t 
     p.w2 = static_cast<const __nv_bfloat16*>(m->w.ctrl_w2);
     p.c2 = m->w.ctrl_c2;
     p.b_box_rows = d.h_ctrl;
+    p.early = 3;  // only the epilogue reads what the launch before wrote (e_b)
     st = launch(d.h_ctrl <= 64 ? EPI_SCORE : EPI_SCORE_WIDE, m, SVL_TAG_SCORE, p, p.grid_m, s);
     if (st != SVL_OK) return st;
   }

@@ -215,8 +215,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) attn_tc_kernel(const __grid_c
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  pdl_trigger();
-  pdl_wait();
+  pdl_begin(a.late);
   const int n_items = min(*a.count, a.cap);
   const int n_units = 2 * n_items;
   const int group = a.A / a.Akv;

@@ -15,12 +15,25 @@
 namespace svl {
 
 // ---------------------------------------------------------------- dependent launch
-// Every kernel is launched with programmatic stream serialization: it lets
-// its successor launch right away (pdl_trigger) and waits for its
-// predecessor's completion and memory (pdl_wait) before reading anything the
-// predecessor wrote. Work before pdl_wait touches no shared global data.
+// Every kernel is launched with programmatic stream serialization and waits
+// for its predecessor's completion and memory (pdl_wait) before reading
+// anything the predecessor wrote. Where it lets its successor launch
+// (pdl_trigger) decides what that successor may read before its own wait:
+//  - at once (the default): nothing. The launch latency of both is hidden.
+//  - `late`, after its own wait: everything up to the launch before it is
+//    then complete and visible when the successor starts, so the successor may
+//    read what was written two or more launches before itself (work lists) and
+//    what no kernel of the call writes (weights). Only kernels in front of one
+//    that does so pay for it: in chains of kernels of a few microseconds a
+//    late trigger exposes about 3 us of launch latency per kernel.
 SVL_DEVINL void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 SVL_DEVINL void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+SVL_DEVINL void pdl_begin(bool late) {
+  if (!late) pdl_trigger();
+  pdl_wait();
+  if (late) pdl_trigger();
+}
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,

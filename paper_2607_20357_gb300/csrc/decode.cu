@@ -16,8 +16,7 @@ namespace svl {
 // memory so that both the V^T reads and the cache writes are coalesced.
 __global__ void kv_store_kernel(KvArgs a) {
   __shared__ __nv_bfloat16 tile[32][33];
-  pdl_trigger();
-  pdl_wait();
+  pdl_begin(false);
   const int T = a.cu_seqlens[a.B];
   const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;  // packed rows, kv columns
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8 threads
@@ -72,8 +71,7 @@ __global__ void __launch_bounds__(kDecWarps * 32, 4) decode_attn_kernel(DecAttnA
   __shared__ float sm_m[kDecWarps], sm_l[kDecWarps];
   __shared__ float sm_o[kDecWarps][DH];
   __shared__ float sp[kDecWarps][32];
-  pdl_trigger();
-  pdl_wait();
+  pdl_begin(a.late);
   const int b = blockIdx.x, h = blockIdx.y;
   const int G = a.G, hpg = a.A / G, g = h / hpg;
   if (!(a.layer_gate[b * a.L + a.l] && a.group_gate[(static_cast<size_t>(b) * a.L + a.l) * G + g]) && a.l >= a.P)
@@ -223,8 +221,7 @@ __global__ void __launch_bounds__(kFinThreads) decode_finish_kernel(int B, int V
                                                                     int* cache_len, int max_len) {
   __shared__ float bv[kFinThreads / 32];
   __shared__ int bi[kFinThreads / 32];
-  pdl_trigger();
-  pdl_wait();
+  pdl_begin(false);
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float* row = logits + static_cast<size_t>(b) * V;
   float best = -INFINITY;

@@ -336,8 +336,7 @@ __device__ void build_list(const ScheduleArgs& a, int l, int kind, int* dyn) {
 // per call (at b = 1 and 16 samples 10 MB instead of the whole 84 MB of V^T).
 __global__ void __launch_bounds__(kSetupThreads) setup_kernel(ScheduleArgs a) {
   extern __shared__ int setup_dyn[];
-  pdl_trigger();
-  pdl_wait();
+  pdl_begin(false);
   int blk = blockIdx.x;
   const int n_list_blocks = a.n_lists * a.n_layers;
   if (blk < n_list_blocks) {
@@ -431,8 +430,7 @@ __global__ void __launch_bounds__(kCtlThreads) controller_kernel(CtlArgs a) {
   __shared__ double pe[256], hid[256];
   __shared__ int keep_groups;
   __shared__ long long n_on_sh;
-  pdl_trigger();
-  pdl_wait();
+  pdl_begin(false);
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int L = a.L, G = a.G, P = min(a.P, a.L), H = a.H, D = a.D;
   const int ng = (L - P) * G;
@@ -568,8 +566,7 @@ SVL_DEVINL void norm_row(const __nv_bfloat16* x, const __nv_bfloat16* g, __nv_bf
 }
 
 __global__ void rmsnorm_kernel(NormArgs a) {
-  pdl_trigger();
-  pdl_wait();
+  pdl_begin(true);  // the LM head loads weights before it waits
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r = blockIdx.x * (blockDim.x >> 5) + warp;
   const int T = a.cu_seqlens[a.B];
@@ -579,8 +576,7 @@ __global__ void rmsnorm_kernel(NormArgs a) {
 }
 
 __global__ void final_rows_kernel(NormArgs a, int n_pad) {
-  pdl_trigger();
-  pdl_wait();
+  pdl_begin(true);  // the LM head loads weights before it waits
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int b = blockIdx.x * (blockDim.x >> 5) + warp;
   if (b >= n_pad) return;

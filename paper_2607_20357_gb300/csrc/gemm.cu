@@ -1,8 +1,8 @@
 // Persistent warp-specialised tcgen05 GEMM with fused epilogues (sm_103a).
 //
-//   warp 0      one thread issues TMA loads of A (128 rows x 128 bytes) and B
-//               (up to 2 x 128 rows x 128 bytes) per stage into a 4-stage
-//               shared-memory ring: 64 K of bf16 or 128 K of e4m3;
+//   warps 6, 0  one thread each issues the TMA loads of A (128 rows x 128
+//               bytes) and of B (up to 2 x 128 rows x 128 bytes) per stage into
+//               a 4-stage shared-memory ring: 64 K of bf16 or 128 K of e4m3;
 //   warp 1      allocates 512 TMEM columns; one thread issues
 //               tcgen05.mma (M = 128, N <= 256, K = 16 per bf16 instruction,
 //               32 per e4m3 one) and commits stage releases and
@@ -24,18 +24,49 @@ struct TileInfo {
   bool valid;
 };
 
-SVL_DEVINL int num_tiles(const GemmParams& p) {
-  if (p.tiles) {
-    int n = *p.tile_count;
-    return n < 0 ? 0 : (n > p.max_tiles ? p.max_tiles : n);
-  }
-  return p.grid_m * p.grid_n;
+// What a role reads about the launch's work once, before its tile loop. The
+// loads go to the L2: the lists may be read before the predecessor has
+// completed, when lines of an earlier call's lists could still sit in the L1.
+struct Work {
+  int n;             // tiles
+  int ks0, kr, ks;   // K-split tail: first copy, tail tiles, shares (see GemmParams)
+  int mlim;          // dense grid: rows
+  int4 next;         // the list entry of the CTA's next tile, fetched one ahead
+};
+
+SVL_DEVINL void fetch_tile(const GemmParams& p, Work& w, int t) {
+  if (p.tiles && t < w.n) w.next = __ldcg(p.tiles + t);
 }
 
-SVL_DEVINL TileInfo get_tile(const GemmParams& p, int t) {
+SVL_DEVINL Work load_work(const GemmParams& p, int first) {
+  Work w;
+  w.ks0 = 0x7fffffff;
+  w.kr = w.ks = 0;
+  w.mlim = p.m_limit;
+  w.next = make_int4(0, 0, 0, 0);
+  if (p.tiles) {
+    const int n = __ldcg(p.tile_count);
+    if (p.ks_info) {
+      w.ks0 = __ldcg(p.ks_info);
+      w.kr = __ldcg(p.ks_info + 1);
+      w.ks = __ldcg(p.ks_info + 2);
+      if (w.kr <= 0 || w.ks < 2) w.ks0 = 0x7fffffff;
+    }
+    w.n = n < 0 ? 0 : (n > p.max_tiles ? p.max_tiles : n);
+    fetch_tile(p, w, first);
+  } else {
+    if (p.m_limit_dev) w.mlim = min(w.mlim, __ldcg(p.m_limit_dev));
+    w.n = p.grid_m * p.grid_n;
+  }
+  return w;
+}
+
+// Tile t (the one fetched last) and, `step` further, the fetch of the next.
+SVL_DEVINL TileInfo get_tile(const GemmParams& p, Work& w, int t, int step) {
   TileInfo ti;
   if (p.tiles) {
-    int4 v = p.tiles[t];
+    const int4 v = w.next;
+    fetch_tile(p, w, t + step);
     ti.m0 = v.x;
     ti.m_end = v.y;
     ti.n0 = v.z;
@@ -44,28 +75,23 @@ SVL_DEVINL TileInfo get_tile(const GemmParams& p, int t) {
     ti.kmask = tile_kmask(v.w);
     ti.valid = ti.ncols > 0 && ti.m_end > ti.m0 && ti.mat < 3;
   } else {
-    int mi = t % p.grid_m, ni = t / p.grid_m;
-    int mlim = p.m_limit;
-    if (p.m_limit_dev) mlim = min(mlim, *p.m_limit_dev);
+    const int mi = t % p.grid_m, ni = t / p.grid_m;
     ti.m0 = mi * kBM;
-    ti.m_end = min(ti.m0 + kBM, mlim);
+    ti.m_end = min(ti.m0 + kBM, w.mlim);
     ti.n0 = ni * p.bn;
     ti.ncols = min(p.bn, p.n_limit - ti.n0);
     ti.mat = 0;
     ti.kmask = 0;
-    ti.valid = ti.m0 < mlim && ti.ncols > 0;
+    ti.valid = ti.m0 < w.mlim && ti.ncols > 0;
   }
   ti.part = 0;
   ti.nsplit = 1;
   ti.slot = 0;
-  if (p.ks_info && t >= p.ks_info[0]) {
-    const int r = p.ks_info[1], sp = p.ks_info[2];
-    if (r > 0 && sp > 1) {
-      const int u = t - p.ks_info[0];
-      ti.slot = u % r;
-      ti.part = u / r;
-      ti.nsplit = sp;
-    }
+  if (t >= w.ks0) {
+    const int u = t - w.ks0;
+    ti.part = u / w.kr;
+    ti.slot = u - ti.part * w.kr;
+    ti.nsplit = w.ks;
   }
   return ti;
 }
@@ -84,6 +110,23 @@ struct KWalk {
   int kb, grp, kin;
   const int nkb, kgb, kmask;
   SVL_DEVINL KWalk(int nkb_, int kgb_, int kmask_) : kb(-1), grp(0), kin(-1), nkb(nkb_), kgb(kgb_), kmask(kmask_) {}
+  // Moves to the n-th active block (n >= 1), as n calls of next() would. The
+  // shares of a K-split tile start here: stepping took 0.1 us a block, 8 us
+  // for the last of eight shares of an 11,008-deep product.
+  SVL_DEVINL void skip(int n) {
+    if (n <= 0) return;
+    const int g = (n - 1) / kgb, r = (n - 1) - g * kgb;
+    if (kmask == 0) {
+      kb = n - 1;
+      grp = g;
+    } else {
+      int m = kmask;
+      for (int i = 0; i < g; ++i) m &= m - 1;  // drop the g lowest active groups
+      grp = __ffs(m) - 1;
+      kb = grp * kgb + r;
+    }
+    kin = r;
+  }
   // advances to the next active K block; false when the tile is done
   SVL_DEVINL bool next() {
     while (true) {
@@ -136,44 +179,52 @@ struct StageCfg<EPI_SCORE_WIDE, false> {
   static constexpr int bytes = kABytes + kBHalfBytes;
 };
 
-// ------------------------------------------------------------------ producer
-template <int NST, int SBYTES, int ABYTES, bool F8>
+// ------------------------------------------------------------------ producers
+// One thread loads A, one loads B, each on its own walk over the CTA's K
+// steps: the ring of four 48 KB stages covers the load latency only just, so
+// the path from a released stage to its loads is kept short (a stage's three
+// loads issued by one thread in turn made the gate/up GEMM 3 % slower). A
+// producer whose operand is in p.early starts without waiting for the
+// predecessor; the ring and the other operand hold it back.
+template <int OP, int NST, int SBYTES, int ABYTES, bool F8>  // OP 0: A, 1: B
 SVL_DEVINL void producer_loop(const GemmParams& p, uint8_t* stages, uint64_t* full,
                               uint64_t* empty, volatile int* abort) {
   constexpr int BK = F8 ? kBK8 : kBK;
-  const int ntiles = num_tiles(p);
+  Work wk = load_work(p, blockIdx.x);
   const int nkb = p.K / BK, kgb = p.kgroup / BK;
   const uint64_t pol = l2_evict_first_policy();
   int s = 0;
-  uint32_t ph = 0;
-  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    TileInfo ti = get_tile(p, t);
+  uint32_t ph = 1;
+  for (int t = blockIdx.x; t < wk.n; t += gridDim.x) {
+    const TileInfo ti = get_tile(p, wk, t, gridDim.x);
     if (!ti.valid) continue;
     const int halves = p.b_split ? 2 : (ti.ncols > kBHalf ? 2 : 1);
     const CUtensorMap* mb0 = p.b_split ? &p.mapB[0] : &p.mapB[ti.mat];
     const CUtensorMap* mb1 = p.b_split ? &p.mapB[1] : &p.mapB[ti.mat];
     const int y1 = p.b_split ? ti.n0 : ti.n0 + kBHalf;
-    const uint32_t bytes = ABYTES + halves * (p.b_box_rows ? p.b_box_rows * 128 : kBHalfBytes);
+    const uint32_t bytes = OP == 0 ? ABYTES : halves * (p.b_box_rows ? p.b_box_rows * 128 : kBHalfBytes);
     KWalk w(nkb, kgb, ti.kmask);
     int i0, i1;
     k_share(ti, nkb, kgb, i0, i1);
-    for (int i = 0; i < i0; ++i) w.next();
+    w.skip(i0);
+    w.next();
     for (int i = i0; i < i1; ++i) {
-      w.next();
-      const int kb = w.kb;
-      if (!mbar_wait(&empty[s], ph ^ 1, abort)) {
+      uint8_t* dst = stages + s * SBYTES + (OP == 0 ? 0 : ABYTES);
+      if (!mbar_wait(&empty[s], ph, abort)) {
         set_abort(abort, p.status);
         return;
       }
-      uint8_t* sa = stages + s * SBYTES;
-      uint8_t* sb = sa + ABYTES;
       mbar_arrive_expect_tx(&full[s], bytes);
-      if (p.a_evict_first)
-        tma_load_2d_hint(sa, &p.mapA, &full[s], kb * BK, ti.m0, pol);
-      else
-        tma_load_2d(sa, &p.mapA, &full[s], kb * BK, ti.m0);
-      tma_load_2d(sb, mb0, &full[s], kb * BK, ti.n0);
-      if (halves == 2) tma_load_2d(sb + kBHalfBytes, mb1, &full[s], kb * BK, y1);
+      if constexpr (OP == 0) {
+        if (p.a_evict_first)
+          tma_load_2d_hint(dst, &p.mapA, &full[s], w.kb * BK, ti.m0, pol);
+        else
+          tma_load_2d(dst, &p.mapA, &full[s], w.kb * BK, ti.m0);
+      } else {
+        tma_load_2d(dst, mb0, &full[s], w.kb * BK, ti.n0);
+        if (halves == 2) tma_load_2d(dst + kBHalfBytes, mb1, &full[s], w.kb * BK, y1);
+      }
+      w.next();
       if (++s == NST) {
         s = 0;
         ph ^= 1;
@@ -187,12 +238,12 @@ template <int NST, int SBYTES, int ABYTES, bool F8>
 SVL_DEVINL void mma_loop(const GemmParams& p, uint8_t* stages, uint64_t* full, uint64_t* empty,
                          uint64_t* tfull, uint64_t* tempty, uint32_t tmem, volatile int* abort) {
   constexpr int BK = F8 ? kBK8 : kBK;
-  const int ntiles = num_tiles(p);
+  Work wk = load_work(p, blockIdx.x);
   const int nkb = p.K / BK, kgb = p.kgroup / BK;
   int s = 0, it = 0;
   uint32_t ph = 0;
-  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    TileInfo ti = get_tile(p, t);
+  for (int t = blockIdx.x; t < wk.n; t += gridDim.x) {
+    const TileInfo ti = get_tile(p, wk, t, gridDim.x);
     if (!ti.valid) continue;
     const int acc = it & 1;
     const uint32_t aph = (it >> 1) & 1;
@@ -822,7 +873,7 @@ SVL_DEVINL void qkv_tile_tma(const GemmParams& p, const TileInfo& ti, int q, uin
 template <int KIND, bool F8, bool THIN>
 SVL_DEVINL void epilogue_loop(const GemmParams& p, uint64_t* tfull, uint64_t* tempty, uint32_t tmem,
                               volatile int* abort, KsSync& ks, uint8_t* rstage, uint64_t* rbar) {
-  const int ntiles = num_tiles(p);
+  Work wk = load_work(p, blockIdx.x);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = warp & 3;  // TMEM lane quarter this warp may access
   // residual (EPI_RESID) or outputs (EPI_SWIGLU, EPI_QKV_ROPE) through shared memory
@@ -832,8 +883,8 @@ SVL_DEVINL void epilogue_loop(const GemmParams& p, uint64_t* tfull, uint64_t* te
   uint32_t rpar = 0;  // EPI_RESID: parity of each buffer's next wait
   uint32_t sbuf = 0;  // EPI_SWIGLU: chunks stored so far (buffer = sbuf & 1)
   int it = 0;
-  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    TileInfo ti = get_tile(p, t);
+  for (int t = blockIdx.x; t < wk.n; t += gridDim.x) {
+    const TileInfo ti = get_tile(p, wk, t, gridDim.x);
     if (!ti.valid) continue;
     const int acc = it & 1;
     const uint32_t aph = (it >> 1) & 1;
@@ -925,7 +976,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int i = 0; i < NST; ++i) {
-      mbar_init(&full[i], 1);
+      mbar_init(&full[i], 2);  // the A and the B producer
       mbar_init(&empty[i], 1);
     }
     for (int i = 0; i < 2; ++i) {
@@ -950,13 +1001,20 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  // set-up above touches no global data; from here on the predecessor's
-  // outputs are read
-  pdl_trigger();
-  pdl_wait();
+  // The set-up above touches no global data. With early operands the lists
+  // are old enough to be read before the predecessor has completed, so only
+  // the roles that read its outputs wait for it.
+  if (!p.late) pdl_trigger();
+  const bool waits = warp == 0 ? !(p.early & 2) : warp == 6 ? !(p.early & 1) : warp == 1 ? !p.early : true;
+  if (waits) {
+    pdl_wait();
+    if (p.late) pdl_trigger();
+  }
 
   if (warp == 0) {
-    if (lane == 0) producer_loop<NST, SBYTES, ABYTES, F8>(p, stages, full, empty, abort);
+    if (lane == 0) producer_loop<1, NST, SBYTES, ABYTES, F8>(p, stages, full, empty, abort);
+  } else if (warp == 6) {
+    if (lane == 0) producer_loop<0, NST, SBYTES, ABYTES, F8>(p, stages, full, empty, abort);
   } else if (warp == 1) {
     if (lane == 0) mma_loop<NST, SBYTES, ABYTES, F8>(p, stages, full, empty, tfull, tempty, tmem, abort);
   } else {
@@ -1017,8 +1075,8 @@ SVL_DEVINL int pair_n(const GemmParams& p, const TileInfo& ti) {
 
 SVL_DEVINL void pair_producer(const GemmParams& p, uint8_t* stages, uint64_t* full, uint64_t* empty, uint32_t rank,
                               volatile int* abort) {
-  const int ntiles = num_tiles(p);
   const int npairs = gridDim.x >> 1, pair = blockIdx.x >> 1;
+  Work wk = load_work(p, pair);
   const int nkb = p.K / kBK, kgb = p.kgroup / kBK;
   int s = 0;
   uint32_t ph = 0;
@@ -1028,8 +1086,8 @@ SVL_DEVINL void pair_producer(const GemmParams& p, uint8_t* stages, uint64_t* fu
       ph ^= 1;
     }
   };
-  for (int t = pair; t < ntiles; t += npairs) {
-    const TileInfo ti = get_tile(p, t);
+  for (int t = pair; t < wk.n; t += npairs) {
+    const TileInfo ti = get_tile(p, wk, t, npairs);
     if (!ti.valid) continue;
     const int brows = pair_n(p, ti) / 2;
     const CUtensorMap* mb = p.b_split ? &p.mapB[rank] : &p.mapB[ti.mat];
@@ -1062,13 +1120,13 @@ SVL_DEVINL void pair_producer(const GemmParams& p, uint8_t* stages, uint64_t* fu
 
 SVL_DEVINL void pair_mma(const GemmParams& p, uint8_t* stages, uint64_t* full, uint64_t* empty, uint64_t* tfull,
                          uint64_t* tempty, uint32_t tmem, volatile int* abort) {
-  const int ntiles = num_tiles(p);
   const int npairs = gridDim.x >> 1, pair = blockIdx.x >> 1;
+  Work wk = load_work(p, pair);
   const int nkb = p.K / kBK, kgb = p.kgroup / kBK;
   int s = 0, it = 0;
   uint32_t ph = 0;
-  for (int t = pair; t < ntiles; t += npairs) {
-    const TileInfo ti = get_tile(p, t);
+  for (int t = pair; t < wk.n; t += npairs) {
+    const TileInfo ti = get_tile(p, wk, t, npairs);
     if (!ti.valid) continue;
     const int acc = it & 1;
     const uint32_t aph = (it >> 1) & 1;
@@ -1108,13 +1166,13 @@ SVL_DEVINL void pair_mma(const GemmParams& p, uint8_t* stages, uint64_t* full, u
 template <int KIND>
 SVL_DEVINL void pair_epilogue(const GemmParams& p, uint64_t* tfull, uint64_t* tempty, uint32_t tmem, uint32_t rank,
                               volatile int* abort) {
-  const int ntiles = num_tiles(p);
   const int npairs = gridDim.x >> 1, pair = blockIdx.x >> 1;
+  Work wk = load_work(p, pair);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = warp & 3;  // TMEM lane quarter this warp may access
   int it = 0;
-  for (int t = pair; t < ntiles; t += npairs) {
-    const TileInfo ti = get_tile(p, t);
+  for (int t = pair; t < wk.n; t += npairs) {
+    const TileInfo ti = get_tile(p, wk, t, npairs);
     if (!ti.valid) continue;
     const int acc = it & 1;
     const uint32_t aph = (it >> 1) & 1;
@@ -1138,7 +1196,7 @@ SVL_DEVINL void pair_epilogue(const GemmParams& p, uint64_t* tfull, uint64_t* te
 }
 
 template <int KIND>
-__global__ void __launch_bounds__(kGemmThreads, 1) gemm_pair_kernel(const __grid_constant__ GemmParams p) {
+__global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid_constant__ GemmParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(stages + kPairStages * kPairStageBytes);
@@ -1174,8 +1232,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_pair_kernel(const __grid
   tc_fence_after();
   cluster_sync();  // both CTAs' barriers exist before any TMA or arrive reaches them
   const uint32_t tmem = *tmem_slot;
-  pdl_trigger();
-  pdl_wait();
+  pdl_begin(p.late);
 
   if (warp == 0) {
     if (lane == 0) pair_producer(p, stages, full, empty, rank, abort);
@@ -1211,7 +1268,7 @@ static cudaError_t launch_pair_kind(const GemmParams& p, int pairs, cudaStream_t
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(2 * pairs));
-  cfg.blockDim = dim3(kGemmThreads);
+  cfg.blockDim = dim3(kPairThreads);
   cfg.dynamicSmemBytes = kPairSmem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
@@ -1238,7 +1295,7 @@ cudaError_t launch_gemm_pair(EpiKind kind, const GemmParams& p, int pairs, cudaS
 int gemm_pair_max_clusters(EpiKind kind) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2);
-  cfg.blockDim = dim3(kGemmThreads);
+  cfg.blockDim = dim3(kPairThreads);
   cfg.dynamicSmemBytes = kPairSmem;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;

@@ -20,7 +20,8 @@ constexpr int kThinRows = 32;      // A rows of a THIN launch (see launch_gemm)
 constexpr int kABytes = kBM * kBK * 2;
 constexpr int kBHalfBytes = kBHalf * kBK * 2;
 constexpr int kStageBytes = kABytes + 2 * kBHalfBytes;
-constexpr int kGemmThreads = 192;  // warp 0 TMA, warp 1 MMA + TMEM, warps 2-5 epilogue
+constexpr int kGemmThreads = 224;  // warp 0 TMA of B, warp 1 MMA + TMEM, warps 2-5 epilogue, warp 6 TMA of A
+constexpr int kPairThreads = 192;  // CTA pairs: one TMA warp
 constexpr int kAccCols = 256;      // fp32 columns per accumulator
 constexpr int kTmemCols = 512;     // two accumulators (epilogue overlaps the next tile)
 constexpr int kGemmSmem = kStages * kStageBytes + 1024 /*align*/ + 256 /*barriers*/;
@@ -113,6 +114,13 @@ struct GemmParams {
   // residual GEMMs keep a band of weights in L2 while the input rows stream
   // through; this keeps the rows from pushing the band out.
   int a_evict_first;
+  // Operands (bit 0: A, bit 1: B) whose first stages may be loaded before the
+  // kernel waits for its predecessor: weights, and anything written at least
+  // two launches ago. Needs the tile list (or m_limit_dev) to be that old as
+  // well; 0 otherwise. The weights of the next GEMM then stream in while its
+  // predecessor finishes. The predecessor must have been launched `late`.
+  int early;
+  bool late;  // the successor may launch only after this kernel's wait (see pdl_trigger)
   uint32_t* status;
 };
 

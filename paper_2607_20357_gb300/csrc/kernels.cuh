@@ -140,6 +140,7 @@ struct QuantArgs {
   const uint8_t* layer_gate;  // [B, L] or nullptr
   const uint8_t* group_gate;  // [B, L, G] or nullptr
   int L, l, P;
+  bool late;  // successor may launch only after this kernel's wait (see pdl_trigger)
 };
 cudaError_t launch_quant_rows(const QuantArgs& a, cudaStream_t s);
 
@@ -167,6 +168,7 @@ struct DecAttnArgs {
   __nv_bfloat16* k_cache;   // this layer's [B][max_len][dkv]
   __nv_bfloat16* v_cache;
   __nv_bfloat16* out;       // [B, A*dh]
+  bool late;                // see QuantArgs
 };
 void launch_decode_attn(const DecAttnArgs& a, cudaStream_t s);
 void launch_decode_finish(int B, int V, const float* logits, int* next_token, int* cache_len, int max_len,
@@ -299,6 +301,7 @@ struct AttnTcArgs {
   float scale_log2;         // log2(e) / sqrt(dh)
   __nv_bfloat16* O;         // [T_cap, A*dh]
   int ldo;
+  bool late;                // see QuantArgs
   uint32_t* status;
 };
 cudaError_t launch_attention_tc(const AttnTcArgs& a, int grid, cudaStream_t s);

@@ -8,8 +8,7 @@
 namespace svl {
 
 __global__ void pack_offsets_kernel(PackArgs a) {
-  pdl_trigger();
-  pdl_wait();
+  pdl_begin(false);
   if (threadIdx.x != 0) return;
   int t = 0;
   a.cu_seqlens[0] = 0;
@@ -28,8 +27,7 @@ __global__ void pack_offsets_kernel(PackArgs a) {
 
 // One warp per output row.
 __global__ void pack_gather_kernel(PackArgs a) {
-  pdl_trigger();
-  pdl_wait();
+  pdl_begin(a.use_projector);  // the projector GEMM loads weights before it waits
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r = blockIdx.x * (blockDim.x >> 5) + warp;
   const int T = *a.t_total;
@@ -76,8 +74,7 @@ __global__ void pack_gather_kernel(PackArgs a) {
 }
 
 __global__ void offsets_diff_kernel(const int* off, int* len, int B) {
-  pdl_trigger();
-  pdl_wait();
+  pdl_begin(false);
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b < B) len[b] = off[b + 1] - off[b];
 }
@@ -94,8 +91,7 @@ __global__ void llm_budget_embed_kernel(const float* __restrict__ budget, const 
                                         __nv_bfloat16* __restrict__ out) {
   __shared__ double pe[256];
   __shared__ double hid[256];
-  pdl_trigger();
-  pdl_wait();
+  pdl_begin(false);
   const int b = blockIdx.x, i = threadIdx.x;
   const double bv = static_cast<double>(budget[b]);
   if (i < H) {

@@ -49,8 +49,7 @@ SVL_DEVINL uint2 codes8(const float f[8], float inv) {
 
 // One warp per row, two passes (rows wider than 16,384 codes).
 __global__ void __launch_bounds__(kQuantWarps * 32) quant_rows_kernel(QuantArgs a) {
-  pdl_trigger();
-  pdl_wait();
+  pdl_begin(a.late);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t r = static_cast<int64_t>(blockIdx.x) * kQuantWarps + warp;
   int64_t rows = a.rows;
@@ -109,8 +108,7 @@ template <int NCH, bool GAIN>
 __global__ void __launch_bounds__(kQuantThreads) quant_row_cta_kernel(QuantArgs a) {
   __shared__ float red[2][kQuantThreads / 32];
   __shared__ int s_mask[2];
-  pdl_trigger();
-  pdl_wait();
+  pdl_begin(a.late);
   int64_t rows = a.rows;
   if (a.cu_seqlens) rows = min(rows, static_cast<int64_t>(a.cu_seqlens[a.B]));
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;

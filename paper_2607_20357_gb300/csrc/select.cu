@@ -29,8 +29,7 @@ __global__ void budget_embed_kernel(const float* __restrict__ budget, const __nv
                                     const __nv_bfloat16* __restrict__ w2, int H, float* __restrict__ e_b) {
   __shared__ float pe[256];
   __shared__ float hid[256];
-  pdl_trigger();
-  pdl_wait();
+  pdl_begin(true);  // the score GEMM loads its operands before it waits
   const int b = blockIdx.x, i = threadIdx.x;
   if (i < H) {
     const int half = H / 2;
@@ -71,8 +70,7 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectArgs a) {
   __shared__ long long n_on_sum;  // updated with 64-bit atomics
   __shared__ int n_pos, keep_groups;
   __shared__ double kappa_sum;
-  pdl_trigger();
-  pdl_wait();
+  pdl_begin(false);
 
   const int b = blockIdx.x, tid = threadIdx.x;
   const int v0 = a.vis_off[b], v1 = a.vis_off[b + 1];
@@ -278,8 +276,7 @@ __global__ void compact_kernel(int B, const int* __restrict__ vis_off, const int
                                const int* __restrict__ kept_local, int* __restrict__ kept_idx,
                                int* __restrict__ kept_off, int* __restrict__ kept_total) {
   __shared__ int off;
-  pdl_trigger();
-  pdl_wait();
+  pdl_begin(false);
   const int b = blockIdx.x;
   if (threadIdx.x == 0) off = 0;
   __syncthreads();
