@@ -1300,7 +1300,9 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
     }
     p.mapA = m->tm_lm_head;
     p.early = 1;  // the weights are A here
-    if (!make_map(&p.mapB[0], na.Y, n_pad, d.d_model)) return SVL_ERR_CUDA;
+    const bool few = n_pad <= kThinRows;
+    if (!make_map(&p.mapB[0], na.Y, n_pad, d.d_model, few ? kThinRows : 128)) return SVL_ERR_CUDA;
+    p.b_box_rows = few ? kThinRows : 0;
     p.grid_m = (d.vocab + kBM - 1) / kBM;
     p.grid_n = (n_pad + 255) / 256;
     p.bn = std::min(n_pad, 256);
@@ -1310,7 +1312,9 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
     p.kgroup = d.d_model;
     p.out[0] = logits;
     p.ld[0] = d.vocab;
-    if ((st = launch(EPI_LOGITS_T, m, SVL_TAG_LMHEAD, p, static_cast<int64_t>(p.grid_m) * p.grid_n, s)) != SVL_OK) return st;
+    if ((st = launch(EPI_LOGITS_T, m, SVL_TAG_LMHEAD, p, static_cast<int64_t>(p.grid_m) * p.grid_n, s, false, few)) !=
+        SVL_OK)
+      return st;
   } else {
     {
       Launch L1(m, SVL_TAG_RMSNORM, s);

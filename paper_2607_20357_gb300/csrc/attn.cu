@@ -59,12 +59,6 @@ SVL_DEVINL void attn_abort(volatile int* abort, uint32_t* status) {
   report(status, SVL_DEV_TIMEOUT);
 }
 
-SVL_DEVINL float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 SVL_DEVINL float max3(float a, float b, float c) {
   float d;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));

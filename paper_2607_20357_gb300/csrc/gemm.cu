@@ -166,6 +166,16 @@ struct StageCfg<KIND, true> {
   static constexpr int abytes = kThinRows * 128;
   static constexpr int bytes = abytes + 2 * kBHalfBytes;
 };
+// LM head of at most kThinRows samples: a stage is 16 KB of weights (A) and
+// the samples' rows in a box of kThinRows, so ten stages keep 160 KB of
+// weights in flight per SM (four 48 KB stages held 64 KB: 3.9 TB/s for a
+// 1.1 GB head).
+template <>
+struct StageCfg<EPI_LOGITS_T, true> {
+  static constexpr int stages = 10;
+  static constexpr int abytes = kABytes;
+  static constexpr int bytes = kABytes + kThinRows * 128;
+};
 template <>
 struct StageCfg<EPI_SCORE, false> {
   static constexpr int stages = 9;
@@ -561,6 +571,7 @@ struct KsSync {
   uint64_t* gather;  // 128 arrivals: every row of this share is stored
   uint64_t* done;    // 1 arrival: every share of the tile is stored (*flag = 1) or a wait gave up (0)
   volatile int* flag;
+  uint64_t* load;    // the bulk copies of this share's slice
   uint32_t phase;
 };
 
@@ -570,20 +581,183 @@ SVL_DEVINL int ld_acquire(const int* p) {
   return v;
 }
 
+// One 128-column slot of one row of a K-split tile, by a whole warp: the sum
+// over its shares in share order (from the partials at `base`) goes onto the
+// residual row, four columns per lane. The squares of the stored values, summed
+// in column order within 32 columns (eight lanes, the chain handed from lane to
+// lane) and then over the four chunks pairwise, are the norm's partial.
+template <bool F8>
+SVL_DEVINL void ksplit_slot(const GemmParams& p, const TileInfo& ti, const float* base, int row, int slot) {
+  const int lane = threadIdx.x & 31, col = slot * 128 + lane * 4;
+  uint2* xr = reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out[0]) +
+                                       static_cast<size_t>(ti.m0 + row) * p.ld[0] + ti.n0 + col);
+  float2 oa = make_float2(0.f, 0.f), ob = oa;  // the stored values
+  if (col < ti.ncols) {
+    const uint2 x = *xr;
+    float4 f[8], v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      if (q < ti.nsplit)
+        f[q] = __ldcg(reinterpret_cast<const float4*>(base + (static_cast<size_t>(q) * kBM + row) * kAccCols + col));
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      if (q < ti.nsplit) {
+        v.x += f[q].x;
+        v.y += f[q].y;
+        v.z += f[q].z;
+        v.w += f[q].w;
+      }
+    }
+    if constexpr (F8) {
+      const float4 cs = __ldg(reinterpret_cast<const float4*>(p.b_scale[0] + ti.n0 + col));
+      const float rs = p.a_scale[ti.m0 + row];
+      v.x *= rs * cs.x;
+      v.y *= rs * cs.y;
+      v.z *= rs * cs.z;
+      v.w *= rs * cs.w;
+    }
+    const float2 x0 = unpack_bf16x2(x.x), x1 = unpack_bf16x2(x.y);
+    const uint2 o = make_uint2(pack_bf16x2(v.x + x0.x, v.y + x0.y), pack_bf16x2(v.z + x1.x, v.w + x1.y));
+    *xr = o;
+    oa = unpack_bf16x2(o.x);
+    ob = unpack_bf16x2(o.y);
+  }
+  if (!p.ss_out) return;
+  float ss = 0.f;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const float prev = __shfl_up_sync(0xffffffffu, ss, 1);
+    if ((lane & 7) == j) {
+      ss = fmaf(oa.x, oa.x, fmaf(oa.y, oa.y, j ? prev : 0.f));
+      ss = fmaf(ob.x, ob.x, fmaf(ob.y, ob.y, ss));
+    }
+  }
+  ss += __shfl_xor_sync(0xffffffffu, ss, 8);
+  ss += __shfl_xor_sync(0xffffffffu, ss, 16);
+  if (lane == 7) p.ss_out[static_cast<size_t>((ti.n0 >> 7) + slot) * p.ss_ld + ti.m0 + row] = ss;
+}
+
+// The same for rows [r0, r1) whose shares and residual lie in the ring (see
+// ksplit_tile): each warp takes a run of rows, first forms and stores the sums
+// (also over the residual in the ring), then one lane per 32 columns adds up
+// the squares of four rows at a time.
+constexpr int kKsResid = 136 * 1024;  // ring offset of the residual rows (past nsplit slices of 1 KB rows)
+static_assert(kKsResid + 64 * 512 <= kStages * kStageBytes, "K-split slices in the stage ring");
+
+template <bool F8>
+SVL_DEVINL void ksplit_rows(const GemmParams& p, const TileInfo& ti, uint8_t* ring, int r0, int r1) {
+  const int lane = threadIdx.x & 31, wrp = (threadIdx.x >> 5) - 2;
+  const int n = r1 - r0, a0 = n * wrp / 4, a1 = n * (wrp + 1) / 4;  // this warp's rows of the slice
+  __nv_bfloat16* X =
+      reinterpret_cast<__nv_bfloat16*>(p.out[0]) + static_cast<size_t>(ti.m0 + r0) * p.ld[0] + ti.n0;
+  for (int c = lane * 8; c < ti.ncols; c += 256) {  // eight columns per lane
+    float cs[8];
+    if constexpr (F8) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) cs[i] = __ldg(p.b_scale[0] + ti.n0 + c + i);
+    }
+#pragma unroll 2
+    for (int r = a0; r < a1; ++r) {
+      uint4* xr = reinterpret_cast<uint4*>(ring + kKsResid + r * 512 + c * 2);
+      const int sw = (r0 + r) & 7, u0 = (c >> 2) & 7;
+      const uint8_t* src = ring + static_cast<size_t>(r) * (kAccCols * 4) + (c >> 5) * 128;
+      float v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = 0.f;
+      for (int q = 0; q < ti.nsplit; ++q, src += static_cast<size_t>(n) * (kAccCols * 4)) {
+        const float4 f = *reinterpret_cast<const float4*>(src + ((u0 ^ sw) << 4));
+        const float4 g = *reinterpret_cast<const float4*>(src + (((u0 + 1) ^ sw) << 4));
+        v[0] += f.x;
+        v[1] += f.y;
+        v[2] += f.z;
+        v[3] += f.w;
+        v[4] += g.x;
+        v[5] += g.y;
+        v[6] += g.z;
+        v[7] += g.w;
+      }
+      if constexpr (F8) {
+        const float rs = p.a_scale[ti.m0 + r0 + r];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] *= rs * cs[i];
+      }
+      const uint4 x = *xr;
+      const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
+      uint32_t o[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 f = unpack_bf16x2(xw[i]);
+        o[i] = pack_bf16x2(v[2 * i] + f.x, v[2 * i + 1] + f.y);
+      }
+      *xr = make_uint4(o[0], o[1], o[2], o[3]);
+      *reinterpret_cast<uint4*>(X + static_cast<size_t>(r) * p.ld[0] + c) = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+  }
+  if (!p.ss_out) return;
+  __syncwarp();
+  const int c = (lane & 7) * 32;
+  for (int rb = a0; rb < a1; rb += 4) {  // uniform over the warp
+    const int r = rb + (lane >> 3);
+    float ss = 0.f;
+    if (r < a1 && c < ti.ncols) {
+      const uint4* xr = reinterpret_cast<const uint4*>(ring + kKsResid + r * 512 + c * 2);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint4 u = xr[i];
+        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float2 f = unpack_bf16x2(w[k]);
+          ss = fmaf(f.x, f.x, fmaf(f.y, f.y, ss));
+        }
+      }
+    }
+    ss += __shfl_xor_sync(0xffffffffu, ss, 1);
+    ss += __shfl_xor_sync(0xffffffffu, ss, 2);
+    if (r < a1 && c < ti.ncols && (lane & 3) == 0)
+      p.ss_out[static_cast<size_t>((ti.n0 + c) >> 7) * p.ss_ld + ti.m0 + r0 + r] = ss;
+  }
+}
+
 // Residual epilogue of one K-split share. The share's accumulator goes to
 // ks_part; once every share of the tile is stored (the shares run side by
 // side in the last wave of the persistent grid, whose CTAs are all resident),
-// this CTA sums all shares in order for its 1/nsplit of the tile's rows, adds
-// them to the residual rows and writes their norm partial sums. Every wait is
-// bounded; returns false on a time-out.
-template <bool F8>
+// this CTA sums all shares in order for its part of the tile, adds them to the
+// residual rows and writes their norm partial sums. Every wait is bounded;
+// returns false on a time-out.
+//
+// THIN tiles have a few rows: plain stores and loads, the (row, 128-column
+// slot) pairs dealt out over the shares. Otherwise a share reduces a slice of
+// rows and everything moves in bulk copies through the stage ring, which is
+// free (a share is its CTA's last tile and all its MMAs are done): the
+// accumulator rows are staged there and stored 32 rows at a time, the residual
+// rows of the slice load while the shares meet, and the slice of every share
+// follows. At 309 rows (O projection, three shares) the epilogue threads'
+// own stores took 5.4 us and their loads 14 us; the bulk copies take 3 and 4.
+template <bool F8, bool THIN>
 SVL_DEVINL bool ksplit_tile(const GemmParams& p, const TileInfo& ti, int lrow, uint32_t taddr, bool empty, KsSync& ks,
-                            volatile int* abort) {
+                            volatile int* abort, uint8_t* ring) {
+  const int lane = threadIdx.x & 31, wrp = (threadIdx.x >> 5) - 2;
+  const int nr = ti.m_end - ti.m0, nsl = (ti.ncols + 127) / 128;
+  const int r0 = nr * ti.part / ti.nsplit, r1 = nr * (ti.part + 1) / ti.nsplit;  // this share's slice (not THIN)
   const size_t unit = static_cast<size_t>(ti.slot) * ti.nsplit;
+  const __nv_bfloat16* X =
+      reinterpret_cast<const __nv_bfloat16*>(p.out[0]) + static_cast<size_t>(ti.m0) * p.ld[0] + ti.n0;
   float* mine = p.ks_part + ((unit + ti.part) * kBM + lrow) * kAccCols;
+  if constexpr (!THIN) {
+    if (wrp == 0 && r1 > r0) {
+      const uint32_t xb = static_cast<uint32_t>(ti.ncols) * 2;
+      if (lane == 0)
+        mbar_arrive_expect_tx(ks.load, static_cast<uint32_t>(r1 - r0) * (xb + ti.nsplit * kAccCols * 4));
+      __syncwarp();
+      for (int r = r0 + lane; r < r1; r += 32)
+        bulk_load(ring + kKsResid + (r - r0) * 512, X + static_cast<size_t>(r) * p.ld[0], xb, ks.load);
+    }
+  }
   // rows past the tile's end are never reduced: no partial for them
-  const bool stored = ti.m0 + lrow < ti.m_end;
+  const bool stored = lrow < nr;
   float v[32];
+  uint8_t* stage = ring + lrow * (kAccCols * 4);
   for (int c = 0; c < ti.ncols; c += 32) {
     if (!empty) {
       tmem_ld32(taddr + c, v);  // warp-collective: every lane loads
@@ -591,11 +765,31 @@ SVL_DEVINL bool ksplit_tile(const GemmParams& p, const TileInfo& ti, int lrow, u
 #pragma unroll
       for (int j = 0; j < 32; ++j) v[j] = 0.f;
     }
-    if (stored) {
-      float4* d = reinterpret_cast<float4*>(mine + c);
+    if constexpr (THIN) {
+      if (stored) {
+        float4* d = reinterpret_cast<float4*>(mine + c);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) d[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+        for (int i = 0; i < 8; ++i) d[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+      }
+    } else {
+      // 16-byte unit i of each 32 columns at i ^ (row & 7): conflict-free, and kept in ks_part
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        *reinterpret_cast<float4*>(stage + c * 4 + ((i ^ (lane & 7)) << 4)) =
+            make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
     }
+  }
+  if constexpr (!THIN) {
+    fence_proxy_async();
+    __syncwarp();
+    const int rows = min(32, nr - (lrow & ~31));
+    if (lane == 0 && rows > 0) {
+      bulk_store(mine, stage, static_cast<uint32_t>(rows) * kAccCols * 4);
+      bulk_commit();
+      bulk_wait0();
+      asm volatile("fence.proxy.async;" ::: "memory");
+    }
+    __syncwarp();
   }
   __threadfence();
   mbar_arrive(ks.gather);
@@ -620,68 +814,23 @@ SVL_DEVINL bool ksplit_tile(const GemmParams& p, const TileInfo& ti, int lrow, u
   ks.phase ^= 1;
   __syncwarp();
   if (!__all_sync(0xffffffffu, got) || !*ks.flag) return false;
-  // The tile's valid rows x 128-column slots form the groups of the
-  // reduction; the shares take every nsplit-th group, so the work is spread
-  // over all of them even when only a few rows are valid (one row per
-  // sample in decode). Four adjacent lanes take the four 32-column chunks of
-  // a group and combine their sums of squares for the norm slot.
-  const int nr = ti.m_end - ti.m0;
-  const int nsl = (ti.ncols + 127) / 128;
-  const int ngroups = nr * nsl;
-  const int n_mine = ti.part < ngroups ? (ngroups - ti.part + ti.nsplit - 1) / ti.nsplit : 0;
-  const int et = threadIdx.x - 2 * 32;  // 0..127
-  const int chunk = et & 3;
-  const float* base = p.ks_part + unit * kBM * kAccCols;
-  for (int k0 = 0; k0 < n_mine; k0 += 32) {  // uniform over the CTA
-    const int i = k0 + (et >> 2);
-    const bool act = i < n_mine;
-    const int g = ti.part + i * ti.nsplit;
-    const int lr = act ? g / nsl : 0, sl = act ? g - lr * nsl : 0;
-    const int row = ti.m0 + lr;
-    const int c = sl * 128 + chunk * 32;
-    float hss = 0.f;
-    if (act && c < ti.ncols) {
-      const int n = min(32, ti.ncols - c);
-#pragma unroll
-      for (int j = 0; j < 32; ++j) v[j] = 0.f;
-      for (int q = 0; q < ti.nsplit; ++q) {
-        const float4* src = reinterpret_cast<const float4*>(base + (static_cast<size_t>(q) * kBM + lr) * kAccCols + c);
-        float4 f[8];
-#pragma unroll
-        for (int i4 = 0; i4 < 8; ++i4) f[i4] = __ldcg(src + i4);
-#pragma unroll
-        for (int i4 = 0; i4 < 8; ++i4) {
-          v[4 * i4] += f[i4].x;
-          v[4 * i4 + 1] += f[i4].y;
-          v[4 * i4 + 2] += f[i4].z;
-          v[4 * i4 + 3] += f[i4].w;
-        }
-      }
-      if constexpr (F8) scale_cols(v, p.b_scale[0] + ti.n0 + c, p.a_scale[row]);
-      __nv_bfloat16* orow = reinterpret_cast<__nv_bfloat16*>(p.out[0]) + static_cast<size_t>(row) * p.ld[0] + ti.n0;
-      const uint4* xs = reinterpret_cast<const uint4*>(orow + c);
-#pragma unroll
-      for (int i4 = 0; i4 < 4; ++i4) {
-        if (i4 * 8 < n) {
-          const uint4 x = xs[i4];
-          const uint32_t wd[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const float2 f = unpack_bf16x2(wd[k]);
-            v[8 * i4 + 2 * k] += f.x;
-            v[8 * i4 + 2 * k + 1] += f.y;
-          }
-        }
-      }
-      if (p.ss_out) hss = store_bf16_ss(orow + c, v, n);
-      else store_bf16(orow + c, v, n);
+  if constexpr (THIN) {
+    const float* base = p.ks_part + unit * kBM * kAccCols;
+    for (int g = ti.part + wrp * ti.nsplit; g < nr * nsl; g += 4 * ti.nsplit) {  // uniform over the warp
+      const int row = nsl == 2 ? g >> 1 : g;
+      ksplit_slot<F8>(p, ti, base, row, g - row * nsl);
     }
-    if (p.ss_out) {
-      // the group's four chunks sit in four adjacent lanes: chunk order kept
-      hss += __shfl_xor_sync(0xffffffffu, hss, 1);
-      hss += __shfl_xor_sync(0xffffffffu, hss, 2);
-      if (act && chunk == 0) p.ss_out[static_cast<size_t>((ti.n0 >> 7) + sl) * p.ss_ld + row] = hss;
+  } else if (r1 > r0) {
+    if (threadIdx.x == 2 * 32) {
+      asm volatile("fence.proxy.async;" ::: "memory");
+      const uint32_t bytes = static_cast<uint32_t>(r1 - r0) * kAccCols * 4;
+      for (int q = 0; q < ti.nsplit; ++q)
+        bulk_load(ring + static_cast<size_t>(q) * bytes, p.ks_part + ((unit + q) * kBM + r0) * kAccCols, bytes, ks.load);
     }
+    const bool in = mbar_wait(ks.load, ks.phase ^ 1, abort);
+    __syncwarp();
+    if (!__all_sync(0xffffffffu, in)) return false;
+    ksplit_rows<F8>(p, ti, ring, r0, r1);
   }
   return true;
 }
@@ -872,7 +1021,7 @@ SVL_DEVINL void qkv_tile_tma(const GemmParams& p, const TileInfo& ti, int q, uin
 
 template <int KIND, bool F8, bool THIN>
 SVL_DEVINL void epilogue_loop(const GemmParams& p, uint64_t* tfull, uint64_t* tempty, uint32_t tmem,
-                              volatile int* abort, KsSync& ks, uint8_t* rstage, uint64_t* rbar) {
+                              volatile int* abort, KsSync& ks, uint8_t* rstage, uint64_t* rbar, uint8_t* ring) {
   Work wk = load_work(p, blockIdx.x);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = warp & 3;  // TMEM lane quarter this warp may access
@@ -925,7 +1074,7 @@ SVL_DEVINL void epilogue_loop(const GemmParams& p, uint64_t* tfull, uint64_t* te
         int i0, i1;
         constexpr int BK = F8 ? kBK8 : kBK;
         k_share(ti, p.K / BK, p.kgroup / BK, i0, i1);
-        if (!ksplit_tile<F8>(p, ti, q * 32 + lane, taddr, i0 == i1, ks, abort)) {
+        if (!ksplit_tile<F8, THIN>(p, ti, q * 32 + lane, taddr, i0 == i1, ks, abort, ring)) {
           set_abort(abort, p.status);
           return;
         }
@@ -965,13 +1114,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
   uint64_t* tempty = bars + 2 * NST + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * NST + 4);
   volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  KsSync ks{bars + 2 * NST + 5, bars + 2 * NST + 6, reinterpret_cast<volatile int*>(bars + 2 * NST + 7), 0};
+  KsSync ks{bars + 2 * NST + 5, bars + 2 * NST + 6, reinterpret_cast<volatile int*>(bars + 2 * NST + 7), bars + 31, 0};
   // EPI_RESID / EPI_SWIGLU / EPI_QKV_ROPE: the epilogue warps' chunk buffers
   // (and, for the residual loads, their barriers)
   constexpr bool kStaged = (KIND == EPI_RESID || KIND == EPI_SWIGLU || KIND == EPI_QKV_ROPE) && !THIN;
   uint64_t* rbar = bars + 2 * NST + 8;
   uint8_t* rstage = stages + NST * SBYTES + 1024;
-  static_assert(!kStaged || (2 * NST + 16) * 8 <= 256, "barriers of the staged residual epilogue");
+  static_assert(2 * NST + (kStaged ? 16 : 8) <= 31, "barriers");
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -985,6 +1134,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
     }
     mbar_init(ks.gather, 4 * 32);
     mbar_init(ks.done, 1);
+    mbar_init(ks.load, 1);
     if (kStaged)
       for (int i = 0; i < 8; ++i) mbar_init(&rbar[i], 1);
     *abort = 0;
@@ -1018,7 +1168,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
   } else if (warp == 1) {
     if (lane == 0) mma_loop<NST, SBYTES, ABYTES, F8>(p, stages, full, empty, tfull, tempty, tmem, abort);
   } else {
-    epilogue_loop<KIND, F8, THIN>(p, tfull, tempty, tmem, abort, ks, rstage, rbar);
+    epilogue_loop<KIND, F8, THIN>(p, tfull, tempty, tmem, abort, ks, rstage, rbar, stages);
   }
 
   __syncwarp();
@@ -1371,6 +1521,7 @@ cudaError_t launch_gemm(EpiKind kind, const GemmParams& p, int grid, cudaStream_
       case EPI_SWIGLU:
         return e4m3 ? launch_kind<EPI_SWIGLU, true, true>(p, grid, stream)
                     : launch_kind<EPI_SWIGLU, false, true>(p, grid, stream);
+      case EPI_LOGITS_T: return launch_kind<EPI_LOGITS_T, false, true>(p, grid, stream);
       default: return cudaErrorInvalidValue;
     }
   }

@@ -125,8 +125,9 @@ struct GemmParams {
 };
 
 // `thin`: every tile has at most kThinRows rows and mapA has boxes of
-// kThinRows rows (QKV, residual and SwiGLU epilogues): deeper weight
-// pipeline for decode-sized batches.
+// kThinRows rows (QKV, residual and SwiGLU epilogues), or at most kThinRows
+// columns and mapB such boxes (EPI_LOGITS_T, whose weights are A): deeper
+// weight pipeline for decode-sized batches.
 cudaError_t launch_gemm(EpiKind kind, const GemmParams& p, int grid, cudaStream_t stream, bool e4m3 = false,
                         bool thin = false);
 
