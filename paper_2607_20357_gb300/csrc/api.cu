@@ -1166,7 +1166,7 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
       Launch L1(m, SVL_TAG_ATTENTION, s);
       da.late = !f8;
       next_launch(da.late);
-      launch_decode_attn(da, s);
+      if (launch_decode_attn(da, s) != cudaSuccess) return SVL_ERR_CUDA;
     } else {
       if (kvx) {
         KvArgs ka;
@@ -1337,7 +1337,8 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
   }
   if (decode) {
     Launch L1(m, SVL_TAG_LMHEAD, s);
-    launch_decode_finish(B, d.vocab, logits, kvx->next_token, kvx->cache_len, kvx->max_len, s);
+    if (launch_decode_finish(B, d.vocab, logits, kvx->next_token, kvx->cache_len, kvx->max_len, s) != cudaSuccess)
+      return SVL_ERR_CUDA;
   } else if (kvx && kvx->cache_len) {
     launch_offsets_diff(cu_seqlens, kvx->cache_len, B, s);  // cache length = prompt length
     g_launches++;

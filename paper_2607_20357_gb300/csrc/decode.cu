@@ -51,33 +51,124 @@ void launch_kv_store(const KvArgs& a, int t_cap, cudaStream_t s) {
   if (grid.x > 0) launch_pdl(kv_store_kernel, grid, 256, 0, s, a);
 }
 
-// One block per (sample, query head) of an active group: the new token's
-// query against the cached keys 0..len-1 and its own key (position len),
-// softmax in float32, output row of O. The block of the first query head of
-// each KV head also appends the new key and value to the cache. Each of the
-// 8 warps takes a contiguous run of positions, 32 at a time: lane j scores
-// key j on its own (its whole K row as 16-byte loads against q in shared
-// memory, no shuffles per key), the warp folds the 32 scores into its online
+// Attention of the new tokens: each query head of an active group against the
+// cached keys 0..len-1 and the token's own key (position len), softmax in
+// float32, output row of O. The positions form kRuns contiguous runs, each
+// walked by one warp 32 at a time: lane j scores key j on its own (one chain
+// over the head's dimensions), the warp folds the 32 scores into its online
 // softmax, then every lane accumulates its d_head / 32 output dimensions over
-// the 32 V rows (independent loads). The warps are merged at the end.
-// Memory-bound on the cache (2 * (len + 1) * d_head * 2 bytes per head).
-constexpr int kDecWarps = 8;
+// the 32 V rows in order. The runs are merged in order at the end.
+// Memory-bound on the cache (2 * (len + 1) * d_head * 2 bytes per KV head), so
+// what matters is that rows are read whole and many at a time:
+//  - d_head / 8 lanes copy a K row with 16 bytes each into a swizzled tile in
+//    shared memory, from which the lanes read their own rows (a lane reading
+//    its row straight from global memory touches 32 lines per instruction);
+//  - one query head per KV head: a block per head, a warp per run, and the V
+//    rows are requested into registers before the scores are formed;
+//  - several (GQA): a cluster of kRuns blocks per KV head, a block per run, a
+//    warp per query head, so the cache is read once for all of them; the tiles
+//    of the next 32 positions load while these are worked on, and the runs meet
+//    through distributed shared memory.
+constexpr int kRuns = 8;
+constexpr int kDecThreads = kRuns * 32;
 
-template <int DH>  // d_head: 64 or 128
-__global__ void __launch_bounds__(kDecWarps * 32, 4) decode_attn_kernel(DecAttnArgs a) {
-  constexpr int PER = DH / 32;
-  __shared__ __align__(16) float sq[DH];  // q * scale
-  __shared__ __align__(16) float snv[DH];  // the new value row
-  __shared__ float sm_m[kDecWarps], sm_l[kDecWarps];
-  __shared__ float sm_o[kDecWarps][DH];
-  __shared__ float sp[kDecWarps][32];
+SVL_DEVINL void cp_async16(void* smem, const void* gmem) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem)), "l"(gmem) : "memory");
+}
+SVL_DEVINL void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+SVL_DEVINL void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Whether head group g of sample b runs in this layer.
+SVL_DEVINL bool dec_group_on(const DecAttnArgs& a, int b, int g) {
+  return a.l < a.P || (a.layer_gate[b * a.L + a.l] && a.group_gate[(static_cast<size_t>(b) * a.L + a.l) * a.G + g]);
+}
+
+// One run's softmax state: the running max, the row sum and this lane's
+// d_head / 32 output dimensions.
+template <int PER>
+struct RunState {
+  float m = -INFINITY, l = 0.f, o[PER];
+};
+
+// Score of key `lane` of a K tile against sq (q * scale).
+template <int DH>
+SVL_DEVINL float tile_score(const uint8_t* ktile, const float* sq, int lane) {
+  float acc = 0.f;
+#pragma unroll
+  for (int c = 0; c < DH / 8; ++c) {
+    const uint4 u = *reinterpret_cast<const uint4*>(ktile + lane * DH * 2 + ((c ^ (lane & 7)) << 4));
+    const float4 q0 = *reinterpret_cast<const float4*>(sq + 8 * c);
+    const float4 q1 = *reinterpret_cast<const float4*>(sq + 8 * c + 4);
+    const float2 k0 = unpack_bf16x2(u.x), k1 = unpack_bf16x2(u.y), k2 = unpack_bf16x2(u.z), k3 = unpack_bf16x2(u.w);
+    acc = fmaf(q0.x, k0.x, acc);
+    acc = fmaf(q0.y, k0.y, acc);
+    acc = fmaf(q0.z, k1.x, acc);
+    acc = fmaf(q0.w, k1.y, acc);
+    acc = fmaf(q1.x, k2.x, acc);
+    acc = fmaf(q1.y, k2.y, acc);
+    acc = fmaf(q1.z, k3.x, acc);
+    acc = fmaf(q1.w, k3.y, acc);
+  }
+  return acc;
+}
+
+// Folds 32 scores (valid where `in`) into the run's max and row sum; returns
+// this lane's probability.
+template <int PER>
+SVL_DEVINL float fold_scores(RunState<PER>& r, float sc, bool in) {
+  float mx = sc;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+  const float mn = fmaxf(r.m, mx);
+  const float e = in ? __expf(sc - mn) : 0.f;
+  float es = e;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) es += __shfl_xor_sync(0xffffffffu, es, off);
+  const float corr = __expf(r.m - mn);  // 0 while m is -inf
+  r.l = r.l * corr + es;
+#pragma unroll
+  for (int i = 0; i < PER; ++i) r.o[i] *= corr;
+  r.m = mn;
+  return e;
+}
+
+// O += probability of row j times this lane's dimensions of it (packed bf16).
+template <int PER>
+SVL_DEVINL void fold_row(RunState<PER>& r, float e, int j, const uint2 w) {
+  const float ej = __shfl_sync(0xffffffffu, e, j);
+  const float2 v0 = unpack_bf16x2(w.x);
+  r.o[0] = fmaf(ej, v0.x, r.o[0]);
+  r.o[1] = fmaf(ej, v0.y, r.o[1]);
+  if constexpr (PER == 4) {
+    const float2 v1 = unpack_bf16x2(w.y);
+    r.o[2] = fmaf(ej, v1.x, r.o[2]);
+    r.o[3] = fmaf(ej, v1.y, r.o[3]);
+  }
+}
+
+// PER packed bf16 values of a row.
+template <int PER>
+SVL_DEVINL uint2 row_part(const void* p) {
+  if constexpr (PER == 4) return *reinterpret_cast<const uint2*>(p);
+  else return make_uint2(*reinterpret_cast<const uint32_t*>(p), 0u);
+}
+
+// One query head per KV head: block (b, head), warp = run.
+template <int DH>
+__global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(DecAttnArgs a) {
+  constexpr int PER = DH / 32, CH = DH / 8;  // dimensions per lane, 16-byte chunks per row
+  extern __shared__ __align__(128) uint8_t dec_smem[];  // K tiles [kRuns][32 rows]
+  __shared__ __align__(16) float sq[DH];                // q * scale
+  __shared__ __align__(16) __nv_bfloat16 snv[DH];       // the new value row
+  __shared__ float sm_m[kRuns], sm_l[kRuns];
+  __shared__ float sm_o[kRuns][DH];
   pdl_begin(a.late);
   const int b = blockIdx.x, h = blockIdx.y;
-  const int G = a.G, hpg = a.A / G, g = h / hpg;
-  if (!(a.layer_gate[b * a.L + a.l] && a.group_gate[(static_cast<size_t>(b) * a.L + a.l) * G + g]) && a.l >= a.P)
-    return;  // gated off: no keys, no values, no output
+  if (!dec_group_on(a, b, h / (a.A / a.G))) return;  // gated off: no keys, no values, no output
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
-  const int kvh = h / (a.A / a.Akv);
   const int len = a.cache_len[b];
   if (len < 0 || len >= a.max_len) {
     // full (or corrupt) cache, reported by setup_kernel: the head's output is
@@ -86,129 +177,227 @@ __global__ void __launch_bounds__(kDecWarps * 32, 4) decode_attn_kernel(DecAttnA
     if (tid < DH) a.out[static_cast<size_t>(b) * a.ldo + h * DH + tid] = __float2bfloat16(0.f);
     return;
   }
-  const __nv_bfloat16* knew = a.k + static_cast<size_t>(b) * a.dkv + kvh * DH;
+  const __nv_bfloat16* knew = a.k + static_cast<size_t>(b) * a.dkv + h * DH;
+  const size_t cbase = static_cast<size_t>(b) * a.max_len * a.dkv + static_cast<size_t>(h) * DH;
+  const int n = len + 1, per_run = (n + kRuns - 1) / kRuns;
+  const int p_begin = warp * per_run, p_end = min(n, p_begin + per_run);
+  uint8_t* ktile = dec_smem + warp * 32 * DH * 2;
+  uint2 vv[32];
+  // requests the K tile and this lane's part of the V rows of positions
+  // [p0, p0 + 32) of the run (the new token's V row comes from snv), eight V
+  // rows at a time as far as the run goes
+  const __nv_bfloat16* kc = a.k_cache + cbase + (lane % CH) * 8;
+  const __nv_bfloat16* vc = a.v_cache + cbase + lane * PER;
+  auto request = [&](int p0) {
+    constexpr int RI = 32 / CH;  // rows per instruction
+#pragma unroll
+    for (int it = 0; it < CH; ++it) {
+      const int row = it * RI + lane / CH, p = p0 + row;
+      if (p < p_end)
+        cp_async16(ktile + row * DH * 2 + (((lane % CH) ^ (row & 7)) << 4),
+                   p < len ? kc + static_cast<size_t>(p) * a.dkv : knew + (lane % CH) * 8);
+    }
+    cp_async_commit();
+    const int cached = min(p_end, len) - p0;
+#pragma unroll
+    for (int j0 = 0; j0 < 32; j0 += 8) {
+      if (j0 >= cached) break;
+#pragma unroll
+      for (int j = j0; j < j0 + 8; ++j)  // rows past the cached ones repeat the last: never used
+        vv[j] = row_part<PER>(vc + static_cast<size_t>(p0 + min(j, cached - 1)) * a.dkv);
+    }
+  };
+  request(p_begin);
   if (tid < DH) {
     sq[tid] = __bfloat162float(a.q[static_cast<size_t>(b) * a.ldq + h * DH + tid]) * a.scale;
-    const __nv_bfloat16 vnew = a.vt[static_cast<size_t>(kvh * DH + tid) * a.t_pad + b];
-    snv[tid] = __bfloat162float(vnew);
-    if (h % (a.A / a.Akv) == 0) {  // append the new key and value to the cache
-      const size_t at = (static_cast<size_t>(b) * a.max_len + len) * a.dkv + kvh * DH + tid;
-      a.k_cache[at] = knew[tid];
-      a.v_cache[at] = vnew;
-    }
+    const __nv_bfloat16 vnew = a.vt[static_cast<size_t>(h * DH + tid) * a.t_pad + b];
+    snv[tid] = vnew;
+    // append the new key and value to the cache
+    const size_t at = (static_cast<size_t>(b) * a.max_len + len) * a.dkv + h * DH + tid;
+    a.k_cache[at] = knew[tid];
+    a.v_cache[at] = vnew;
   }
   __syncthreads();
-  const size_t cbase = static_cast<size_t>(b) * a.max_len * a.dkv + static_cast<size_t>(kvh) * DH;
-  const int n = len + 1, per_warp = (n + kDecWarps - 1) / kDecWarps;
-  const int p_begin = warp * per_warp, p_end = min(n, p_begin + per_warp);
-  float m = -INFINITY, l = 0.f, o[PER];
+  RunState<PER> r;
 #pragma unroll
-  for (int i = 0; i < PER; ++i) o[i] = 0.f;
+  for (int i = 0; i < PER; ++i) r.o[i] = 0.f;
   for (int p0 = p_begin; p0 < p_end; p0 += 32) {
-    const int p = p0 + lane;
-    float sc = -INFINITY;
-    if (p < p_end) {
-      const uint4* kr = reinterpret_cast<const uint4*>(p < len ? a.k_cache + cbase + static_cast<size_t>(p) * a.dkv
-                                                               : knew);
-      uint4 u[DH / 8];
-#pragma unroll
-      for (int c = 0; c < DH / 8; ++c) u[c] = kr[c];
-      float acc = 0.f;
-#pragma unroll
-      for (int c = 0; c < DH / 8; ++c) {
-        const float4 q0 = *reinterpret_cast<const float4*>(sq + 8 * c);
-        const float4 q1 = *reinterpret_cast<const float4*>(sq + 8 * c + 4);
-        const float2 k0 = unpack_bf16x2(u[c].x), k1 = unpack_bf16x2(u[c].y), k2 = unpack_bf16x2(u[c].z),
-                     k3 = unpack_bf16x2(u[c].w);
-        acc = fmaf(q0.x, k0.x, acc);
-        acc = fmaf(q0.y, k0.y, acc);
-        acc = fmaf(q0.z, k1.x, acc);
-        acc = fmaf(q0.w, k1.y, acc);
-        acc = fmaf(q1.x, k2.x, acc);
-        acc = fmaf(q1.y, k2.y, acc);
-        acc = fmaf(q1.z, k3.x, acc);
-        acc = fmaf(q1.w, k3.y, acc);
-      }
-      sc = acc;
-    }
-    float mx = sc;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    const float mn = fmaxf(m, mx);
-    const float e = p < p_end ? __expf(sc - mn) : 0.f;
-    float es = e;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) es += __shfl_xor_sync(0xffffffffu, es, off);
-    const float corr = __expf(m - mn);  // 0 while m is -inf
-    l = l * corr + es;
-#pragma unroll
-    for (int i = 0; i < PER; ++i) o[i] *= corr;
-    m = mn;
-    sp[warp][lane] = e;
+    if (p0 > p_begin) request(p0);
+    cp_async_wait<0>();
     __syncwarp();
-    const int nk = min(32, p_end - p0);
-#pragma unroll 8
-    for (int j = 0; j < nk; ++j) {
-      const int pj = p0 + j;
-      const float ej = sp[warp][j];
-      float vv[PER];
-      if (pj < len) {
-        const __nv_bfloat16* vr = a.v_cache + cbase + static_cast<size_t>(pj) * a.dkv + lane * PER;
-        if constexpr (PER == 4) {
-          const uint2 w = *reinterpret_cast<const uint2*>(vr);
-          const float2 v0 = unpack_bf16x2(w.x), v1 = unpack_bf16x2(w.y);
-          vv[0] = v0.x; vv[1] = v0.y; vv[2] = v1.x; vv[3] = v1.y;
-        } else {
-          const float2 v0 = unpack_bf16x2(*reinterpret_cast<const uint32_t*>(vr));
-          vv[0] = v0.x; vv[1] = v0.y;
-        }
-      } else {
+    const bool in = p0 + lane < p_end;
+    const float sc = tile_score<DH>(ktile, sq, lane);
+    const float e = fold_scores<PER>(r, in ? sc : -INFINITY, in);
+    const int cached = min(p_end, len) - p0;
 #pragma unroll
-        for (int i = 0; i < PER; ++i) vv[i] = snv[lane * PER + i];
-      }
+    for (int j0 = 0; j0 < 32; j0 += 8) {
+      if (j0 >= cached) break;
 #pragma unroll
-      for (int i = 0; i < PER; ++i) o[i] = fmaf(ej, vv[i], o[i]);
+      for (int j = j0; j < j0 + 8; ++j)
+        if (j < cached) fold_row<PER>(r, e, j, vv[j]);
     }
-    __syncwarp();
+    if (len >= p0 && len < p0 + 32 && len < p_end) fold_row<PER>(r, e, len - p0, row_part<PER>(snv + lane * PER));
+    __syncwarp();  // the tile is read before it is filled again
   }
   if (lane == 0) {
-    sm_m[warp] = m;
-    sm_l[warp] = l;
+    sm_m[warp] = r.m;
+    sm_l[warp] = r.l;
   }
 #pragma unroll
-  for (int i = 0; i < PER; ++i) sm_o[warp][lane * PER + i] = o[i];
+  for (int i = 0; i < PER; ++i) sm_o[warp][lane * PER + i] = r.o[i];
   __syncthreads();
-  if (warp == 0) {
+  if (tid < DH) {
     float M = -INFINITY;
-    for (int w = 0; w < kDecWarps; ++w) M = fmaxf(M, sm_m[w]);
-    float L = 0.f, acc[PER];
-#pragma unroll
-    for (int i = 0; i < PER; ++i) acc[i] = 0.f;
-    for (int w = 0; w < kDecWarps; ++w) {
+    for (int w = 0; w < kRuns; ++w) M = fmaxf(M, sm_m[w]);
+    float L = 0.f, acc = 0.f;
+    for (int w = 0; w < kRuns; ++w) {
       const float f = sm_m[w] == -INFINITY ? 0.f : __expf(sm_m[w] - M);
       L += sm_l[w] * f;
-#pragma unroll
-      for (int i = 0; i < PER; ++i) acc[i] += sm_o[w][lane * PER + i] * f;
+      acc += sm_o[w][tid] * f;
     }
     const float inv = L > 0.f ? 1.f / L : 0.f;
-#pragma unroll
-    for (int i = 0; i < PER; ++i)
-      a.out[static_cast<size_t>(b) * a.ldo + h * DH + lane * PER + i] = __float2bfloat16_rn(acc[i] * inv);
+    a.out[static_cast<size_t>(b) * a.ldo + h * DH + tid] = __float2bfloat16_rn(acc * inv);
   }
 }
 
-void launch_decode_attn(const DecAttnArgs& a, cudaStream_t s) {
-  if (a.dh == 128)
-    launch_pdl(decode_attn_kernel<128>, dim3(a.B, a.A), kDecWarps * 32, 0, s, a);
-  else
-    launch_pdl(decode_attn_kernel<64>, dim3(a.B, a.A), kDecWarps * 32, 0, s, a);
+constexpr int kGqaRing = 5;  // tiles in flight per run (16 KB each at d_head 128)
+
+// Several query heads per KV head: cluster of kRuns blocks, block = run, warp
+// = query head; blockIdx.y = KV head times passes of kRuns query heads.
+template <int DH>
+__global__ void __launch_bounds__(kDecThreads) decode_attn_gqa_kernel(DecAttnArgs a) {
+  constexpr int PER = DH / 32, CH = DH / 8, TB = 32 * DH * 2;
+  extern __shared__ __align__(128) uint8_t dec_smem[];  // kGqaRing tiles of 32 K rows and 32 V rows
+  __shared__ __align__(16) float sq[kRuns][DH];
+  __shared__ float sm_m[kRuns], sm_l[kRuns];  // per query head, read by the cluster
+  __shared__ float sm_o[kRuns][DH];
+  pdl_begin(a.late);
+  const int run = blockIdx.x, b = blockIdx.z;
+  const int grp = a.A / a.Akv, npass = (grp + kRuns - 1) / kRuns;
+  const int kvh = blockIdx.y / npass, h0 = kvh * grp + (blockIdx.y - kvh * npass) * kRuns;
+  const int nh = min(kRuns, (kvh + 1) * grp - h0);
+  if (!dec_group_on(a, b, h0 / (a.A / a.G))) return;  // the whole cluster
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
+  const int len = a.cache_len[b];
+  __nv_bfloat16* out = a.out + static_cast<size_t>(b) * a.ldo + h0 * DH;
+  if (len < 0 || len >= a.max_len) {  // the whole cluster; see decode_attn_kernel
+    if (run == 0)
+      for (int i = tid; i < nh * DH; i += kDecThreads) out[i] = __float2bfloat16(0.f);
+    return;
+  }
+  const __nv_bfloat16* knew = a.k + static_cast<size_t>(b) * a.dkv + kvh * DH;
+  const __nv_bfloat16* vnew = a.vt + static_cast<size_t>(kvh) * DH * a.t_pad + b;
+  const size_t cbase = static_cast<size_t>(b) * a.max_len * a.dkv + static_cast<size_t>(kvh) * DH;
+  const int n = len + 1, per_run = (n + kRuns - 1) / kRuns;
+  const int p_begin = run * per_run, p_end = min(n, p_begin + per_run);
+  auto request = [&](int p0, int buf) {
+    uint8_t *kt = dec_smem + buf * 2 * TB, *vt = kt + TB;
+    for (int idx = tid; idx < 32 * CH; idx += kDecThreads) {
+      const int row = idx / CH, c = idx % CH, p = p0 + row;
+      if (p < p_end) {
+        const size_t at = cbase + static_cast<size_t>(p) * a.dkv + c * 8;
+        cp_async16(kt + row * DH * 2 + ((c ^ (row & 7)) << 4), p < len ? a.k_cache + at : knew + c * 8);
+        if (p < len) cp_async16(vt + row * DH * 2 + c * 16, a.v_cache + at);
+      }
+    }
+    cp_async_commit();
+    const int jn = len - p0;  // the new token's V row (transposed in this step's V^T)
+    if (jn >= 0 && jn < 32 && len < p_end && tid < DH)
+      reinterpret_cast<__nv_bfloat16*>(vt)[jn * DH + tid] = vnew[static_cast<size_t>(tid) * a.t_pad];
+  };
+  for (int i = 0; i < kGqaRing - 1; ++i) request(p_begin + 32 * i, i);
+  for (int i = tid; i < nh * DH; i += kDecThreads)
+    sq[i / DH][i % DH] = __bfloat162float(a.q[static_cast<size_t>(b) * a.ldq + h0 * DH + i]) * a.scale;
+  if (run == 0 && h0 == kvh * grp && tid < DH) {  // append the new key and value to the cache
+    const size_t at = (static_cast<size_t>(b) * a.max_len + len) * a.dkv + kvh * DH + tid;
+    a.k_cache[at] = knew[tid];
+    a.v_cache[at] = vnew[static_cast<size_t>(tid) * a.t_pad];
+  }
+  RunState<PER> r;
+#pragma unroll
+  for (int i = 0; i < PER; ++i) r.o[i] = 0.f;
+  int buf = 0;
+  for (int p0 = p_begin; p0 < p_end; p0 += 32) {
+    cp_async_wait<kGqaRing - 2>();
+    __syncthreads();  // this tile has landed, and the previous one is read
+    request(p0 + 32 * (kGqaRing - 1), buf == 0 ? kGqaRing - 1 : buf - 1);
+    if (warp < nh) {
+      const bool in = p0 + lane < p_end;
+      const uint8_t* kt = dec_smem + buf * 2 * TB;
+      const float e = fold_scores<PER>(r, in ? tile_score<DH>(kt, sq[warp], lane) : -INFINITY, in);
+      const uint8_t* vrows = kt + TB + lane * PER * 2;
+      const int nk = min(32, p_end - p0);
+#pragma unroll
+      for (int j0 = 0; j0 < 32; j0 += 8) {
+        if (j0 >= nk) break;
+#pragma unroll
+        for (int j = j0; j < j0 + 8; ++j)
+          if (j < nk) fold_row<PER>(r, e, j, row_part<PER>(vrows + j * DH * 2));
+      }
+    }
+    if (++buf == kGqaRing) buf = 0;
+  }
+  cp_async_wait<0>();
+  if (warp < nh) {
+    if (lane == 0) {
+      sm_m[warp] = r.m;
+      sm_l[warp] = r.l;
+    }
+#pragma unroll
+    for (int i = 0; i < PER; ++i) sm_o[warp][lane * PER + i] = r.o[i];
+  }
+  // merge the runs in order: every block writes d_head / kRuns dimensions
+  cluster_sync();
+  constexpr int DW = DH / kRuns;
+  for (int i = tid; i < nh * DW; i += kDecThreads) {
+    const int h = i / DW, d = run * DW + i % DW;
+    float mw[kRuns], M = -INFINITY;
+#pragma unroll
+    for (int w = 0; w < kRuns; ++w) {
+      mw[w] = ld_cluster(mapa_shared(&sm_m[h], w));
+      M = fmaxf(M, mw[w]);
+    }
+    float L = 0.f, acc = 0.f;
+#pragma unroll
+    for (int w = 0; w < kRuns; ++w) {
+      const float f = mw[w] == -INFINITY ? 0.f : __expf(mw[w] - M);
+      L += ld_cluster(mapa_shared(&sm_l[h], w)) * f;
+      acc += ld_cluster(mapa_shared(&sm_o[h][d], w)) * f;
+    }
+    const float inv = L > 0.f ? 1.f / L : 0.f;
+    out[h * DH + d] = __float2bfloat16_rn(acc * inv);
+  }
+  cluster_sync();  // the others have read this block's run
+}
+
+template <int DH>
+static cudaError_t launch_dec(const DecAttnArgs& a, cudaStream_t s) {
+  const int grp = a.A / a.Akv;
+  if (grp > 1) {
+    constexpr int ring = kGqaRing * 2 * 32 * DH * 2;
+    const cudaError_t e =
+        cudaFuncSetAttribute(decode_attn_gqa_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, ring);
+    if (e != cudaSuccess) return e;
+    return launch_pdl_cluster(decode_attn_gqa_kernel<DH>, dim3(kRuns, a.Akv * ((grp + kRuns - 1) / kRuns), a.B),
+                              kDecThreads, ring, kRuns, s, a);
+  }
+  constexpr int smem = kRuns * 32 * DH * 2;
+  const cudaError_t e =
+      cudaFuncSetAttribute(decode_attn_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(decode_attn_kernel<DH>, dim3(a.B, a.A), kDecThreads, smem, s, a);
+}
+
+cudaError_t launch_decode_attn(const DecAttnArgs& a, cudaStream_t s) {
+  return a.dh == 128 ? launch_dec<128>(a, s) : launch_dec<64>(a, s);
 }
 
 // Greedy next token per sample (largest logit; equal logits: lower id) and
-// the cache length advanced by the fed token. One 1024-thread block per
-// sample; with V a multiple of 4 each thread reads float4s (4 consecutive ids,
-// kept in id order, so the tie rule holds).
-constexpr int kFinThreads = 1024;
+// the cache length advanced by the fed token. A cluster of kFinSplit CTAs
+// scans a sample's logits in contiguous parts (one block took 11 us for
+// 152,064 logits); with V a multiple of 4 each thread reads float4s (4
+// consecutive ids, kept in id order, so the tie rule holds).
+constexpr int kFinThreads = 512, kFinSplit = 8;
 
 SVL_DEVINL void arg_better(float x, int v, float& best, int& idx) {
   if (x > best || (x == best && v < idx)) {
@@ -221,14 +410,18 @@ __global__ void __launch_bounds__(kFinThreads) decode_finish_kernel(int B, int V
                                                                     int* cache_len, int max_len) {
   __shared__ float bv[kFinThreads / 32];
   __shared__ int bi[kFinThreads / 32];
+  __shared__ float cta_v;
+  __shared__ int cta_i;
   pdl_begin(false);
-  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int b = blockIdx.y, part = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float* row = logits + static_cast<size_t>(b) * V;
   float best = -INFINITY;
   int idx = 0x7fffffff;
   if ((V & 3) == 0) {
     const float4* r4 = reinterpret_cast<const float4*>(row);
-    for (int c = tid; c < V / 4; c += kFinThreads) {
+    const int n4 = V / 4, per = (n4 + kFinSplit - 1) / kFinSplit, c1 = min(n4, (part + 1) * per);
+#pragma unroll 4
+    for (int c = part * per + tid; c < c1; c += kFinThreads) {
       const float4 x = r4[c];
       arg_better(x.x, 4 * c, best, idx);
       arg_better(x.y, 4 * c + 1, best, idx);
@@ -236,7 +429,8 @@ __global__ void __launch_bounds__(kFinThreads) decode_finish_kernel(int B, int V
       arg_better(x.w, 4 * c + 3, best, idx);
     }
   } else {
-    for (int v = tid; v < V; v += kFinThreads) arg_better(row[v], v, best, idx);
+    const int per = (V + kFinSplit - 1) / kFinSplit, v1 = min(V, (part + 1) * per);
+    for (int v = part * per + tid; v < v1; v += kFinThreads) arg_better(row[v], v, best, idx);
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
@@ -251,6 +445,14 @@ __global__ void __launch_bounds__(kFinThreads) decode_finish_kernel(int B, int V
   __syncthreads();
   if (tid == 0) {
     for (int w = 1; w < kFinThreads / 32; ++w) arg_better(bv[w], bi[w], best, idx);
+    cta_v = best;
+    cta_i = idx;
+  }
+  cluster_sync();
+  if (part == 0 && tid == 0) {
+    for (int c = 1; c < kFinSplit; ++c)
+      arg_better(ld_cluster(mapa_shared(&cta_v, c)),
+                 __float_as_int(ld_cluster(mapa_shared(&cta_i, c))), best, idx);
     // a sample whose cache was already full took no step: its length stays
     // and it has no next token
     const int len = cache_len[b];
@@ -258,11 +460,13 @@ __global__ void __launch_bounds__(kFinThreads) decode_finish_kernel(int B, int V
     if (next_token) next_token[b] = !stepped ? -1 : (idx == 0x7fffffff ? 0 : idx);
     if (stepped) cache_len[b] = len + 1;
   }
+  cluster_sync();  // the first CTA has read the others' results
 }
 
-void launch_decode_finish(int B, int V, const float* logits, int* next_token, int* cache_len, int max_len,
-                          cudaStream_t s) {
-  launch_pdl(decode_finish_kernel, B, kFinThreads, 0, s, B, V, logits, next_token, cache_len, max_len);
+cudaError_t launch_decode_finish(int B, int V, const float* logits, int* next_token, int* cache_len, int max_len,
+                                 cudaStream_t s) {
+  return launch_pdl_cluster(decode_finish_kernel, dim3(kFinSplit, B), kFinThreads, 0, kFinSplit, s, B, V, logits,
+                            next_token, cache_len, max_len);
 }
 
 }  // namespace svl

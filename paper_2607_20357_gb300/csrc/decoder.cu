@@ -533,11 +533,8 @@ void launch_controller(const CtlArgs& a, cudaStream_t s) {
 
 // ---------------------------------------------------------------- RMSNorm
 
-SVL_DEVINL void norm_row(const __nv_bfloat16* x, const __nv_bfloat16* g, __nv_bfloat16* y, int D, float eps,
-                         int lane) {
-  const uint4* xv = reinterpret_cast<const uint4*>(x);
-  const uint4* gv = reinterpret_cast<const uint4*>(g);
-  uint4* yv = reinterpret_cast<uint4*>(y);
+// 1 / rms of a row of D values, by one warp.
+SVL_DEVINL float row_inv_rms(const uint4* xv, int D, float eps, int lane) {
   float ss = 0.f;
   for (int c = lane; c < D / 8; c += 32) {
     const uint4 u = xv[c];
@@ -550,19 +547,28 @@ SVL_DEVINL void norm_row(const __nv_bfloat16* x, const __nv_bfloat16* g, __nv_bf
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-  const float inv = rsqrtf(ss / static_cast<float>(D) + eps);
-  for (int c = lane; c < D / 8; c += 32) {
-    const uint4 u = xv[c], gg = gv[c];
-    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-    const uint32_t q[4] = {gg.x, gg.y, gg.z, gg.w};
-    uint32_t o[4];
+  return rsqrtf(ss / static_cast<float>(D) + eps);
+}
+
+// Eight values times inv times their gains, rounded to bf16.
+SVL_DEVINL uint4 norm8(const uint4 u, const uint4 gg, float inv) {
+  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+  const uint32_t q[4] = {gg.x, gg.y, gg.z, gg.w};
+  uint32_t o[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float2 f = unpack_bf16x2(w[i]), h = unpack_bf16x2(q[i]);
-      o[i] = pack_bf16x2(f.x * inv * h.x, f.y * inv * h.y);
-    }
-    yv[c] = make_uint4(o[0], o[1], o[2], o[3]);
+  for (int i = 0; i < 4; ++i) {
+    const float2 f = unpack_bf16x2(w[i]), h = unpack_bf16x2(q[i]);
+    o[i] = pack_bf16x2(f.x * inv * h.x, f.y * inv * h.y);
   }
+  return make_uint4(o[0], o[1], o[2], o[3]);
+}
+
+SVL_DEVINL void norm_row(const __nv_bfloat16* x, const __nv_bfloat16* g, __nv_bfloat16* y, int D, float eps,
+                         int lane) {
+  const uint4* xv = reinterpret_cast<const uint4*>(x);
+  const float inv = row_inv_rms(xv, D, eps, lane);
+  for (int c = lane; c < D / 8; c += 32)
+    reinterpret_cast<uint4*>(y)[c] = norm8(xv[c], reinterpret_cast<const uint4*>(g)[c], inv);
 }
 
 __global__ void rmsnorm_kernel(NormArgs a) {
@@ -575,18 +581,27 @@ __global__ void rmsnorm_kernel(NormArgs a) {
   norm_row(a.X + static_cast<size_t>(r) * a.D, a.gain, a.Y + static_cast<size_t>(r) * a.D, a.D, a.eps, lane);
 }
 
-__global__ void final_rows_kernel(NormArgs a, int n_pad) {
+// One block per sample: the final norm of its last row, staged in shared
+// memory by the whole block; every warp then sums the squares in the order of
+// a single warp (a warp per row reading global memory took 10 us, all of it
+// load latency). Rows B .. n_pad - 1 are zeroed.
+constexpr int kFinalThreads = 256;
+__global__ void __launch_bounds__(kFinalThreads) final_rows_kernel(NormArgs a) {
+  extern __shared__ uint4 final_row[];  // [D / 8]
   pdl_begin(true);  // the LM head loads weights before it waits
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b = blockIdx.x * (blockDim.x >> 5) + warp;
-  if (b >= n_pad) return;
-  __nv_bfloat16* y = a.Y + static_cast<size_t>(b) * a.D;
+  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+  uint4* y = reinterpret_cast<uint4*>(a.Y + static_cast<size_t>(b) * a.D);
   const int r1 = b < a.B ? a.cu_seqlens[b + 1] : 0, r0 = b < a.B ? a.cu_seqlens[b] : 0;
-  if (b >= a.B || r1 <= r0) {
-    for (int c = lane; c < a.D / 8; c += 32) reinterpret_cast<uint4*>(y)[c] = make_uint4(0, 0, 0, 0);
+  if (r1 <= r0) {
+    for (int c = tid; c < a.D / 8; c += kFinalThreads) y[c] = make_uint4(0, 0, 0, 0);
     return;
   }
-  norm_row(a.X + static_cast<size_t>(r1 - 1) * a.D, a.gain, y, a.D, a.eps, lane);
+  const uint4* x = reinterpret_cast<const uint4*>(a.X + static_cast<size_t>(r1 - 1) * a.D);
+  const uint4* g = reinterpret_cast<const uint4*>(a.gain);
+  for (int c = tid; c < a.D / 8; c += kFinalThreads) final_row[c] = x[c];
+  __syncthreads();
+  const float inv = row_inv_rms(final_row, a.D, a.eps, lane);
+  for (int c = tid; c < a.D / 8; c += kFinalThreads) y[c] = norm8(final_row[c], g[c], inv);
 }
 
 // W'[r][c] = W[r][c] * g[c] (a norm gain folded into the projection after it)
@@ -622,7 +637,10 @@ void launch_rmsnorm(const NormArgs& a, cudaStream_t s) {
 }
 
 void launch_final_last_rows(const NormArgs& a, int n_pad, cudaStream_t s) {
-  launch_pdl(final_rows_kernel, (n_pad + 7) / 8, 256, 0, s, a, n_pad);
+  const size_t smem = 2 * static_cast<size_t>(a.D);
+  if (smem > 48 * 1024)
+    cudaFuncSetAttribute(final_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  launch_pdl(final_rows_kernel, n_pad, kFinalThreads, smem, s, a);
 }
 
 __global__ void selftest_wait_kernel(uint32_t* status, long long cycles) {

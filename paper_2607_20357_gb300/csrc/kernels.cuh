@@ -170,9 +170,9 @@ struct DecAttnArgs {
   __nv_bfloat16* out;       // [B, A*dh]
   bool late;                // see QuantArgs
 };
-void launch_decode_attn(const DecAttnArgs& a, cudaStream_t s);
-void launch_decode_finish(int B, int V, const float* logits, int* next_token, int* cache_len, int max_len,
-                          cudaStream_t s);
+cudaError_t launch_decode_attn(const DecAttnArgs& a, cudaStream_t s);
+cudaError_t launch_decode_finish(int B, int V, const float* logits, int* next_token, int* cache_len, int max_len,
+                                 cudaStream_t s);
 
 // ---------------------------------------------------------------- decoder
 // Work lists of a layer (setup_kernel).
