@@ -93,24 +93,34 @@ struct RunState {
   float m = -INFINITY, l = 0.f, o[PER];
 };
 
-// Score of key `lane` of a K tile against sq (q * scale).
+// Score of key `lane` of a K tile against sq (q * scale): one chain over the
+// dimensions, its operands read eight 16-byte chunks at a time so that only
+// the first read's latency is exposed.
 template <int DH>
 SVL_DEVINL float tile_score(const uint8_t* ktile, const float* sq, int lane) {
+  const uint8_t* row = ktile + lane * DH * 2;
+  const int sw = (lane & 7) << 4;
   float acc = 0.f;
 #pragma unroll
-  for (int c = 0; c < DH / 8; ++c) {
-    const uint4 u = *reinterpret_cast<const uint4*>(ktile + lane * DH * 2 + ((c ^ (lane & 7)) << 4));
-    const float4 q0 = *reinterpret_cast<const float4*>(sq + 8 * c);
-    const float4 q1 = *reinterpret_cast<const float4*>(sq + 8 * c + 4);
-    const float2 k0 = unpack_bf16x2(u.x), k1 = unpack_bf16x2(u.y), k2 = unpack_bf16x2(u.z), k3 = unpack_bf16x2(u.w);
-    acc = fmaf(q0.x, k0.x, acc);
-    acc = fmaf(q0.y, k0.y, acc);
-    acc = fmaf(q0.z, k1.x, acc);
-    acc = fmaf(q0.w, k1.y, acc);
-    acc = fmaf(q1.x, k2.x, acc);
-    acc = fmaf(q1.y, k2.y, acc);
-    acc = fmaf(q1.z, k3.x, acc);
-    acc = fmaf(q1.w, k3.y, acc);
+  for (int c0 = 0; c0 < DH / 8; c0 += 8) {
+    uint4 u[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) u[c] = *reinterpret_cast<const uint4*>(row + (((c0 + c) << 4) ^ sw));
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const float4 q0 = *reinterpret_cast<const float4*>(sq + 8 * (c0 + c));
+      const float4 q1 = *reinterpret_cast<const float4*>(sq + 8 * (c0 + c) + 4);
+      const float2 k0 = unpack_bf16x2(u[c].x), k1 = unpack_bf16x2(u[c].y), k2 = unpack_bf16x2(u[c].z),
+                   k3 = unpack_bf16x2(u[c].w);
+      acc = fmaf(q0.x, k0.x, acc);
+      acc = fmaf(q0.y, k0.y, acc);
+      acc = fmaf(q0.z, k1.x, acc);
+      acc = fmaf(q0.w, k1.y, acc);
+      acc = fmaf(q1.x, k2.x, acc);
+      acc = fmaf(q1.y, k2.y, acc);
+      acc = fmaf(q1.z, k3.x, acc);
+      acc = fmaf(q1.w, k3.y, acc);
+    }
   }
   return acc;
 }
@@ -135,25 +145,44 @@ SVL_DEVINL float fold_scores(RunState<PER>& r, float sc, bool in) {
   return e;
 }
 
-// O += probability of row j times this lane's dimensions of it (packed bf16).
-template <int PER>
-SVL_DEVINL void fold_row(RunState<PER>& r, float e, int j, const uint2 w) {
-  const float ej = __shfl_sync(0xffffffffu, e, j);
-  const float2 v0 = unpack_bf16x2(w.x);
-  r.o[0] = fmaf(ej, v0.x, r.o[0]);
-  r.o[1] = fmaf(ej, v0.y, r.o[1]);
-  if constexpr (PER == 4) {
-    const float2 v1 = unpack_bf16x2(w.y);
-    r.o[2] = fmaf(ej, v1.x, r.o[2]);
-    r.o[3] = fmaf(ej, v1.y, r.o[3]);
-  }
-}
-
 // PER packed bf16 values of a row.
 template <int PER>
 SVL_DEVINL uint2 row_part(const void* p) {
   if constexpr (PER == 4) return *reinterpret_cast<const uint2*>(p);
   else return make_uint2(*reinterpret_cast<const uint32_t*>(p), 0u);
+}
+
+// O += probability times this lane's dimensions (packed bf16, from row(j)) for
+// the rows j < n of a tile, eight at a time without branches between them: the
+// rows past n of the last eight count as zeros.
+template <int PER, class Row>
+SVL_DEVINL void fold_rows(RunState<PER>& r, float e, int n, Row row) {
+#pragma unroll
+  for (int j0 = 0; j0 < 32; j0 += 8) {
+    if (j0 >= n) break;
+    float ej[8];
+    uint2 w[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      ej[j] = __shfl_sync(0xffffffffu, e, j0 + j);
+      w[j] = row(j0 + j);
+      if (j0 + j >= n) {
+        ej[j] = 0.f;
+        w[j] = make_uint2(0, 0);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const float2 v0 = unpack_bf16x2(w[j].x);
+      r.o[0] = fmaf(ej[j], v0.x, r.o[0]);
+      r.o[1] = fmaf(ej[j], v0.y, r.o[1]);
+      if constexpr (PER == 4) {
+        const float2 v1 = unpack_bf16x2(w[j].y);
+        r.o[2] = fmaf(ej[j], v1.x, r.o[2]);
+        r.o[3] = fmaf(ej[j], v1.y, r.o[3]);
+      }
+    }
+  }
 }
 
 // One query head per KV head: block (b, head), warp = run.
@@ -228,15 +257,18 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(DecAttnArgs
     const bool in = p0 + lane < p_end;
     const float sc = tile_score<DH>(ktile, sq, lane);
     const float e = fold_scores<PER>(r, in ? sc : -INFINITY, in);
-    const int cached = min(p_end, len) - p0;
-#pragma unroll
-    for (int j0 = 0; j0 < 32; j0 += 8) {
-      if (j0 >= cached) break;
-#pragma unroll
-      for (int j = j0; j < j0 + 8; ++j)
-        if (j < cached) fold_row<PER>(r, e, j, vv[j]);
+    fold_rows<PER>(r, e, min(p_end, len) - p0, [&](int j) { return vv[j]; });
+    if (len >= p0 && len < p0 + 32 && len < p_end) {  // the new token, last of the last run
+      const float en = __shfl_sync(0xffffffffu, e, len - p0);
+      const uint2 w = row_part<PER>(snv + lane * PER);
+      const float2 v0 = unpack_bf16x2(w.x), v1 = unpack_bf16x2(w.y);
+      r.o[0] = fmaf(en, v0.x, r.o[0]);
+      r.o[1] = fmaf(en, v0.y, r.o[1]);
+      if constexpr (PER == 4) {
+        r.o[2] = fmaf(en, v1.x, r.o[2]);
+        r.o[3] = fmaf(en, v1.y, r.o[3]);
+      }
     }
-    if (len >= p0 && len < p0 + 32 && len < p_end) fold_row<PER>(r, e, len - p0, row_part<PER>(snv + lane * PER));
     __syncwarp();  // the tile is read before it is filled again
   }
   if (lane == 0) {
@@ -326,14 +358,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_attn_gqa_kernel(DecAttnArg
       const uint8_t* kt = dec_smem + buf * 2 * TB;
       const float e = fold_scores<PER>(r, in ? tile_score<DH>(kt, sq[warp], lane) : -INFINITY, in);
       const uint8_t* vrows = kt + TB + lane * PER * 2;
-      const int nk = min(32, p_end - p0);
-#pragma unroll
-      for (int j0 = 0; j0 < 32; j0 += 8) {
-        if (j0 >= nk) break;
-#pragma unroll
-        for (int j = j0; j < j0 + 8; ++j)
-          if (j < nk) fold_row<PER>(r, e, j, row_part<PER>(vrows + j * DH * 2));
-      }
+      fold_rows<PER>(r, e, min(32, p_end - p0), [&](int j) { return row_part<PER>(vrows + j * DH * 2); });
     }
     if (++buf == kGqaRing) buf = 0;
   }
