@@ -30,6 +30,7 @@ struct svl_model {
   std::vector<CUtensorMap> tm_pair;
   uint32_t* d_status = nullptr;
   float2* rope_cs = nullptr;
+  double* omega = nullptr;  // [h_ctrl / 2] frequencies of the budget encoding (Eq. 5)
   // B-operand tensor maps of the weights: per layer q, k, v, o, g, u, d
   std::vector<CUtensorMap> tm_layer;
   // norm gains folded into the projections after them (allocated only for
@@ -111,10 +112,10 @@ constexpr int kMaxPrefillBatch = 4096;  // samples per prefill call
 // between calls through the workspace, so the three layouts overlap and the
 // workspace size is the largest of them.
 struct SelLayout {
-  size_t e_b, scalars, kept_local, total;
+  size_t e_b, kept_local, total;
 };
 struct PackLayout {
-  size_t scalars, stage, hp, row_map, tok, total;
+  size_t stage, hp, row_map, tok, total;
 };
 struct PreLayout {
   int64_t t_cap, t_pad;
@@ -138,7 +139,6 @@ SelLayout sel_layout(const svl_model_desc& d, int B, int64_t nv) {
   SelLayout L{};
   Bump b;
   L.e_b = b.take(sizeof(float) * B * d.h_ctrl);
-  L.scalars = b.take(64);
   L.kept_local = b.take(sizeof(int) * std::max<int64_t>(nv, 1));
   L.total = b.off;
   return L;
@@ -147,7 +147,6 @@ SelLayout sel_layout(const svl_model_desc& d, int B, int64_t nv) {
 PackLayout pack_layout(const svl_model_desc& d, int B, int64_t nv) {
   PackLayout L{};
   Bump b;
-  L.scalars = b.take(64);
   L.tok = b.take(2 * static_cast<size_t>(B) * d.d_model);  // budget-token rows (compute controller)
   if (d.proj_hidden) {
     L.stage = b.take(2 * nv * d.c_vis);
@@ -534,13 +533,15 @@ svl_status svl_model_create(const svl_model_desc* desc, const svl_weights* w, sv
     }
   }
   if (cudaMalloc(&m->d_status, sizeof(uint32_t)) != cudaSuccess ||
+      cudaMalloc(&m->omega, sizeof(double) * d.h_ctrl) != cudaSuccess ||
       cudaMalloc(&m->rope_cs, sizeof(float2) * static_cast<size_t>(d.max_seq) * (dh / 2)) != cudaSuccess) {
     svl_model_destroy(m);
     return SVL_ERR_CUDA;
   }
   cudaMemset(m->d_status, 0, sizeof(uint32_t));
   launch_rope_table(m->rope_cs, d.max_seq, dh, static_cast<double>(d.rope_theta), 0);
-  g_launches++;
+  launch_budget_omega(m->omega, d.h_ctrl, 0);
+  g_launches += 2;
   if (cudaDeviceSynchronize() != cudaSuccess) {
     svl_model_destroy(m);
     return SVL_ERR_CUDA;
@@ -554,6 +555,7 @@ void svl_model_destroy(svl_model* m) {
   for (cudaEvent_t e : m->ev_pool) cudaEventDestroy(e);
   if (m->d_status) cudaFree(m->d_status);
   if (m->rope_cs) cudaFree(m->rope_cs);
+  if (m->omega) cudaFree(m->omega);
   for (void* f : m->folded)
     if (f) cudaFree(f);
   for (void* f : m->f8_mem)
@@ -581,64 +583,67 @@ namespace {
 // Token controller: scores, k and the kept lists. Gates are given
 // (layer_gate, group_gate) or, under the paper's rule, derived from the
 // compute controller's logits and projected (gate_logits, *_out).
-svl_status score_select_impl(svl_model* m, int32_t B, int32_t n_vis_total, const void* vis_feats,
-                             const int32_t* vis_off, const int32_t* text_len, const float* budget,
-                             const int32_t* keep_count, const uint8_t* layer_gate, const uint8_t* group_gate,
-                             int rule, const float* gate_logits, uint8_t* layer_gate_out, uint8_t* group_gate_out,
-                             float* kappa_out, float* scores, int32_t* k, int32_t* kept_idx, int32_t* kept_off,
-                             uint32_t* sample_flags, void* ws, size_t ws_bytes, void* stream) {
-  // rule 0: budget count for given gates; 1: paper rule with gate logits;
-  // 2: paper rule, gates decided later (threshold only)
-  if (!m || B <= 0 || n_vis_total < 0 || !vis_off || !text_len || !budget || !scores || !k || !kept_idx || !kept_off)
+// rule 0: budget count for given gates; 1: paper rule with gate logits;
+// 2: paper rule, gates decided later (threshold only).
+struct CtlCall {
+  int32_t B, n_vis_total;
+  const void* vis_feats;
+  const int32_t *vis_off, *text_len;
+  const float* budget;
+  const int32_t* keep_count;
+  const uint8_t *layer_gate, *group_gate;
+  int rule;
+  const float* gate_logits;
+  uint8_t *layer_gate_out, *group_gate_out;
+  float *kappa_out, *scores;
+  int32_t *k, *kept_idx, *kept_off;
+  uint32_t* sample_flags;
+};
+
+// The arguments of every entry point of the token controller.
+svl_status check_select(const svl_model* m, const CtlCall& c) {
+  if (!m || c.B <= 0 || c.n_vis_total < 0 || !c.vis_off || !c.text_len || !c.budget || !c.scores || !c.k ||
+      !c.kept_idx || !c.kept_off)
     return SVL_ERR_INVALID_ARG;
-  if (rule == 0 && (!layer_gate || !group_gate)) return SVL_ERR_INVALID_ARG;
-  if (rule == 1 && (!gate_logits || !layer_gate_out || !group_gate_out)) return SVL_ERR_INVALID_ARG;
-  if (n_vis_total > 0 && (!vis_feats || !aligned16(vis_feats))) return SVL_ERR_INVALID_ARG;
-  const SelLayout L = sel_layout(m->d, B, n_vis_total);
-  svl_status st = check_ws(ws, ws_bytes, L.total);
-  if (st != SVL_OK) return st;
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (c.rule == 0 && (!c.layer_gate || !c.group_gate)) return SVL_ERR_INVALID_ARG;
+  if (c.rule == 1 && (!c.gate_logits || !c.layer_gate_out || !c.group_gate_out)) return SVL_ERR_INVALID_ARG;
+  if (c.n_vis_total > 0 && (!c.vis_feats || !aligned16(c.vis_feats))) return SVL_ERR_INVALID_ARG;
+  return SVL_OK;
+}
+
+// The launches, with scratch for the budget embeddings and (rules 1 and 2) the
+// per-sample kept lists.
+svl_status run_select(svl_model* m, const CtlCall& c, float* e_b, int* kept_local, cudaStream_t s) {
   const svl_model_desc& d = m->d;
-  float* e_b = at<float>(ws, L.e_b);
-
-  {
-    Launch L(m, SVL_TAG_BUDGET_EMBED, s);
-    launch_budget_embed(budget, static_cast<const __nv_bfloat16*>(m->w.bud_w1),
-                        static_cast<const __nv_bfloat16*>(m->w.bud_w2), d.h_ctrl, B, e_b, s);
-  }
-
-  if (n_vis_total > 0) {
-    GemmParams p = base_params(m);
-    if (!make_map(&p.mapA, vis_feats, n_vis_total, d.c_vis)) return SVL_ERR_INVALID_ARG;
+  GemmParams p = base_params(m);
+  if (c.n_vis_total > 0) {
+    if (!make_map(&p.mapA, c.vis_feats, c.n_vis_total, d.c_vis)) return SVL_ERR_INVALID_ARG;
     p.mapB[0] = m->tm_ctrl_w1;
-    p.grid_m = (n_vis_total + kBM - 1) / kBM;
+    p.grid_m = (c.n_vis_total + kBM - 1) / kBM;
     p.grid_n = 1;
     p.bn = d.h_ctrl;
-    p.m_limit = n_vis_total;
+    p.m_limit = c.n_vis_total;
     p.n_limit = d.h_ctrl;
     p.K = d.c_vis;
     p.kgroup = d.c_vis;
-    p.out[0] = scores;
+    p.out[0] = c.scores;
     p.e_b = e_b;
-    p.seg_off = vis_off;
-    p.n_seg = B;
+    p.seg_off = c.vis_off;
+    p.n_seg = c.B;
     p.w2 = static_cast<const __nv_bfloat16*>(m->w.ctrl_w2);
     p.c2 = m->w.ctrl_c2;
     p.b_box_rows = d.h_ctrl;
     p.early = 3;  // only the epilogue reads what the launch before wrote (e_b)
-    st = launch(d.h_ctrl <= 64 ? EPI_SCORE : EPI_SCORE_WIDE, m, SVL_TAG_SCORE, p, p.grid_m, s);
-    if (st != SVL_OK) return st;
   }
-
   SelectArgs a;
   std::memset(&a, 0, sizeof(a));
-  a.scores = scores;
-  a.vis_off = vis_off;
-  a.text_len = text_len;
-  a.budget = budget;
-  a.keep_count = keep_count;
-  a.layer_gate = layer_gate;
-  a.group_gate = group_gate;
+  a.scores = c.scores;
+  a.vis_off = c.vis_off;
+  a.text_len = c.text_len;
+  a.budget = c.budget;
+  a.keep_count = c.keep_count;
+  a.layer_gate = c.layer_gate;
+  a.group_gate = c.group_gate;
   a.L = d.n_layers;
   a.G = d.n_groups;
   a.P = d.n_prefix;
@@ -646,23 +651,52 @@ svl_status score_select_impl(svl_model* m, int32_t B, int32_t n_vis_total, const
   a.Dkv = static_cast<long long>(d.n_kv_heads) * (d.d_model / d.n_heads);
   a.Di = d.d_ffn;
   a.V = d.vocab;
-  a.k_out = k;
-  a.flags = sample_flags;
-  a.kept_local = at<int>(ws, L.kept_local);
-  a.gate_logits = rule == 1 ? gate_logits : nullptr;
-  a.layer_gate_out = layer_gate_out;
-  a.group_gate_out = group_gate_out;
-  a.threshold_only = rule == 2 ? 1 : 0;
-  a.kappa = kappa_out;
+  a.k_out = c.k;
+  a.flags = c.sample_flags;
+  a.kept_local = kept_local;
+  a.gate_logits = c.rule == 1 ? c.gate_logits : nullptr;
+  a.layer_gate_out = c.layer_gate_out;
+  a.group_gate_out = c.group_gate_out;
+  a.threshold_only = c.rule == 2 ? 1 : 0;
+  a.kappa = c.kappa_out;
   {
-    Launch L1(m, SVL_TAG_SELECT, s);
-    launch_select(a, B, s);
+    FrontArgs f;
+    f.B = c.B;
+    f.H = d.h_ctrl;
+    f.budget = c.budget;
+    f.w1 = static_cast<const __nv_bfloat16*>(m->w.bud_w1);
+    f.w2 = static_cast<const __nv_bfloat16*>(m->w.bud_w2);
+    f.w_vec = aligned16(f.w1) && aligned16(f.w2);
+    f.omega = m->omega;
+    f.e_b = e_b;
+    f.sel = a;
+    f.counts = c.rule == 0 ? 1 : 0;
+    Launch L(m, SVL_TAG_BUDGET_EMBED, s);
+    launch_front(f, s);
   }
+  if (c.n_vis_total > 0) {
+    const svl_status st = launch(d.h_ctrl <= 64 ? EPI_SCORE : EPI_SCORE_WIDE, m, SVL_TAG_SCORE, p, p.grid_m, s);
+    if (st != SVL_OK) return st;
+  }
+  Launch L1(m, SVL_TAG_SELECT, s);
+  if (c.rule == 0) {
+    launch_topk(c.B, c.scores, c.vis_off, c.k, c.kept_off, c.kept_idx, s);
+    return last_error();
+  }
+  launch_select(a, c.B, s);
   {
     Launch L2(m, SVL_TAG_SELECT, s);
-    launch_compact(B, vis_off, k, a.kept_local, kept_idx, kept_off, at<int>(ws, L.scalars), s);
+    launch_compact(c.B, c.vis_off, c.k, kept_local, c.kept_idx, c.kept_off, s);
   }
   return last_error();
+}
+
+svl_status score_select_impl(svl_model* m, const CtlCall& c, void* ws, size_t ws_bytes, void* stream) {
+  svl_status st = check_select(m, c);
+  if (st != SVL_OK) return st;
+  const SelLayout L = sel_layout(m->d, c.B, c.n_vis_total);
+  if ((st = check_ws(ws, ws_bytes, L.total)) != SVL_OK) return st;
+  return run_select(m, c, at<float>(ws, L.e_b), at<int>(ws, L.kept_local), static_cast<cudaStream_t>(stream));
 }
 }  // namespace
 
@@ -671,9 +705,9 @@ svl_status svl_score_select(svl_model* m, int32_t B, int32_t n_vis_total, const 
                             const int32_t* keep_count, const uint8_t* layer_gate, const uint8_t* group_gate,
                             float* scores, int32_t* k, int32_t* kept_idx, int32_t* kept_off, uint32_t* sample_flags,
                             void* ws, size_t ws_bytes, void* stream) {
-  return score_select_impl(m, B, n_vis_total, vis_feats, vis_off, text_len, budget, keep_count, layer_gate,
-                           group_gate, 0, nullptr, nullptr, nullptr, nullptr, scores, k, kept_idx, kept_off,
-                           sample_flags, ws, ws_bytes, stream);
+  const CtlCall c{B,       n_vis_total, vis_feats, vis_off, text_len, budget,   keep_count, layer_gate, group_gate, 0,
+                  nullptr, nullptr,     nullptr,   nullptr, scores,   k,        kept_idx,   kept_off,   sample_flags};
+  return score_select_impl(m, c, ws, ws_bytes, stream);
 }
 
 svl_status svl_score_select_paper(svl_model* m, int32_t B, int32_t n_vis_total, const void* vis_feats,
@@ -682,9 +716,10 @@ svl_status svl_score_select_paper(svl_model* m, int32_t B, int32_t n_vis_total, 
                                   int32_t* kept_idx, int32_t* kept_off, uint32_t* sample_flags,
                                   uint8_t* layer_gate_out, uint8_t* group_gate_out, float* kappa_out, void* ws,
                                   size_t ws_bytes, void* stream) {
-  return score_select_impl(m, B, n_vis_total, vis_feats, vis_off, text_len, budget, keep_count, nullptr, nullptr,
-                           gate_logits ? 1 : 2, gate_logits, layer_gate_out, group_gate_out, kappa_out, scores, k,
-                           kept_idx, kept_off, sample_flags, ws, ws_bytes, stream);
+  const CtlCall c{B,           n_vis_total,    vis_feats,      vis_off,   text_len, budget, keep_count, nullptr,
+                  nullptr,     gate_logits ? 1 : 2, gate_logits, layer_gate_out, group_gate_out, kappa_out, scores, k,
+                  kept_idx,    kept_off,       sample_flags};
+  return score_select_impl(m, c, ws, ws_bytes, stream);
 }
 
 namespace {
@@ -731,29 +766,33 @@ svl_status pack_impl(svl_model* m, int32_t B, int32_t n_vis_total, int32_t n_tex
   a.X = static_cast<__nv_bfloat16*>(X);
   a.cu_seqlens = cu_seqlens;
   a.pos = pos;
-  a.t_total = at<int>(ws, L.scalars) + 1;
   a.use_projector = d.proj_hidden ? 1 : 0;
   a.stage = d.proj_hidden ? at<__nv_bfloat16>(ws, L.stage) : nullptr;
   a.row_map = d.proj_hidden ? at<int>(ws, L.row_map) : nullptr;
   a.status = m->d_status;
-  {
-    Launch L1(m, SVL_TAG_PACK, s);
+  if (pack_needs_offsets(B)) {
+    Launch L0(m, SVL_TAG_PACK, s);
     launch_pack_offsets(a, s);
   }
   {
-    Launch L2(m, SVL_TAG_PACK, s);
-    launch_pack_gather(a, s);
+    Launch L1(m, SVL_TAG_PACK, s);
+    if (launch_pack_gather(a, s) != cudaSuccess) return SVL_ERR_CUDA;
   }
 
   if (d.proj_hidden && n_vis_total > 0) {
+    // 128-column tiles (six stages of 32 KB) while at most two thirds of the
+    // SMs would have a 256-column one: a tile then takes half the time, and
+    // even every token kept makes no more than two waves of them
+    const int64_t wide = static_cast<int64_t>((n_vis_total + kBM - 1) / kBM) * ((d.d_model + 255) / 256);
+    const bool narrow = 3 * wide <= 2 * m->num_sms;
     GemmParams p = base_params(m);
     if (!make_map(&p.mapA, a.stage, n_vis_total, d.c_vis)) return SVL_ERR_CUDA;
     p.mapB[0] = m->tm_proj_w1;
     p.early = 2;
     p.late = true;
     p.grid_m = (n_vis_total + kBM - 1) / kBM;
-    p.grid_n = (d.proj_hidden + 255) / 256;
-    p.bn = 256;
+    p.bn = narrow ? kBHalf : 256;
+    p.grid_n = (d.proj_hidden + p.bn - 1) / p.bn;
     p.m_limit_dev = kept_off + B;
     p.m_limit = n_vis_total;
     p.n_limit = d.proj_hidden;
@@ -761,7 +800,7 @@ svl_status pack_impl(svl_model* m, int32_t B, int32_t n_vis_total, int32_t n_tex
     p.kgroup = d.c_vis;
     p.out[0] = at<__nv_bfloat16>(ws, L.hp);
     p.ld[0] = d.proj_hidden;
-    st = launch(EPI_GELU, m, SVL_TAG_PROJECTOR, p, static_cast<int64_t>(p.grid_m) * p.grid_n, s);
+    st = launch(EPI_GELU, m, SVL_TAG_PROJECTOR, p, static_cast<int64_t>(p.grid_m) * p.grid_n, s, false, narrow);
     if (st != SVL_OK) return st;
 
     GemmParams q = base_params(m);
@@ -769,8 +808,8 @@ svl_status pack_impl(svl_model* m, int32_t B, int32_t n_vis_total, int32_t n_tex
     q.mapB[0] = m->tm_proj_w2;
     q.early = 2;
     q.grid_m = p.grid_m;
-    q.grid_n = (d.d_model + 255) / 256;
-    q.bn = 256;
+    q.bn = p.bn;
+    q.grid_n = (d.d_model + q.bn - 1) / q.bn;
     q.m_limit_dev = kept_off + B;
     q.m_limit = n_vis_total;
     q.n_limit = d.d_model;
@@ -779,7 +818,7 @@ svl_status pack_impl(svl_model* m, int32_t B, int32_t n_vis_total, int32_t n_tex
     q.out[0] = X;
     q.ld[0] = d.d_model;
     q.row_map = a.row_map;
-    st = launch(EPI_ROWMAP, m, SVL_TAG_PROJECTOR, q, static_cast<int64_t>(q.grid_m) * q.grid_n, s);
+    st = launch(EPI_ROWMAP, m, SVL_TAG_PROJECTOR, q, static_cast<int64_t>(q.grid_m) * q.grid_n, s, false, narrow);
     if (st != SVL_OK) return st;
   }
   return last_error();
@@ -1713,78 +1752,19 @@ extern "C" svl_status svl_score_select_noalloc(svl_model* m, int32_t B, int32_t 
                                                const uint8_t* group_gate, float* scores, int32_t* k,
                                                int32_t* kept_idx, int32_t* kept_off, uint32_t* sample_flags,
                                                void* stream) {
-  if (!m || B <= 0 || n_vis_total < 0 || !vis_off || !text_len || !budget || !layer_gate || !group_gate ||
-      !scores || !k || !kept_idx || !kept_off)
-    return SVL_ERR_INVALID_ARG;
-  if (n_vis_total > 0 && (!vis_feats || !aligned16(vis_feats))) return SVL_ERR_INVALID_ARG;
+  const CtlCall c{B,       n_vis_total, vis_feats, vis_off, text_len, budget,   keep_count, layer_gate, group_gate, 0,
+                  nullptr, nullptr,     nullptr,   nullptr, scores,   k,        kept_idx,   kept_off,   sample_flags};
+  svl_status st = check_select(m, c);
+  if (st != SVL_OK) return st;
   if (B > kNoAllocMaxBatch || n_vis_total > kNoAllocMaxVis || m->d.h_ctrl > kNoAllocMaxHctrl)
     return SVL_ERR_SHAPE;  // beyond the fixed scratch array
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev != m->device) return SVL_ERR_INVALID_ARG;
   void* scratch = nullptr;
-  svl_status st = noalloc_scratch(&scratch);
-  if (st != SVL_OK) return st;
-  float* e_b = static_cast<float*>(scratch);
-  int* kept_local = reinterpret_cast<int*>(static_cast<unsigned char*>(scratch) + kNoAllocEbBytes);
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const svl_model_desc& d = m->d;
-
-  // Every scratch element read below is written earlier in the same call
-  // (e_b by the budget MLP, kept_local[vis_off[b] ..] by the select kernel
-  // before compaction reads it), so nothing has to be cleared first.
-  {
-    Launch L(m, SVL_TAG_BUDGET_EMBED, s);
-    launch_budget_embed(budget, static_cast<const __nv_bfloat16*>(m->w.bud_w1),
-                        static_cast<const __nv_bfloat16*>(m->w.bud_w2), d.h_ctrl, B, e_b, s);
-  }
-  if (n_vis_total > 0) {
-    GemmParams p = base_params(m);
-    if (!make_map(&p.mapA, vis_feats, n_vis_total, d.c_vis)) return SVL_ERR_INVALID_ARG;
-    p.mapB[0] = m->tm_ctrl_w1;
-    p.grid_m = (n_vis_total + kBM - 1) / kBM;
-    p.grid_n = 1;
-    p.bn = d.h_ctrl;
-    p.m_limit = n_vis_total;
-    p.n_limit = d.h_ctrl;
-    p.K = d.c_vis;
-    p.kgroup = d.c_vis;
-    p.out[0] = scores;
-    p.e_b = e_b;
-    p.seg_off = vis_off;
-    p.n_seg = B;
-    p.w2 = static_cast<const __nv_bfloat16*>(m->w.ctrl_w2);
-    p.c2 = m->w.ctrl_c2;
-    p.b_box_rows = d.h_ctrl;
-    p.early = 3;  // only the epilogue reads what the launch before wrote (e_b)
-    st = launch(d.h_ctrl <= 64 ? EPI_SCORE : EPI_SCORE_WIDE, m, SVL_TAG_SCORE, p, p.grid_m, s);
-    if (st != SVL_OK) return st;
-  }
-  SelectArgs a;
-  std::memset(&a, 0, sizeof(a));
-  a.scores = scores;
-  a.vis_off = vis_off;
-  a.text_len = text_len;
-  a.budget = budget;
-  a.keep_count = keep_count;
-  a.layer_gate = layer_gate;
-  a.group_gate = group_gate;
-  a.L = d.n_layers;
-  a.G = d.n_groups;
-  a.P = d.n_prefix;
-  a.D = d.d_model;
-  a.Dkv = static_cast<long long>(d.n_kv_heads) * (d.d_model / d.n_heads);
-  a.Di = d.d_ffn;
-  a.V = d.vocab;
-  a.k_out = k;
-  a.flags = sample_flags;
-  a.kept_local = kept_local;
-  {
-    Launch L1(m, SVL_TAG_SELECT, s);
-    launch_select(a, B, s);
-  }
-  {
-    Launch L2(m, SVL_TAG_SELECT, s);
-    launch_compact(B, vis_off, k, kept_local, kept_idx, kept_off, nullptr, s);
-  }
-  return last_error();
+  if ((st = noalloc_scratch(&scratch)) != SVL_OK) return st;
+  // Every scratch element read is written earlier in the same call, so nothing
+  // has to be cleared first.
+  return run_select(m, c, static_cast<float*>(scratch),
+                    reinterpret_cast<int*>(static_cast<unsigned char*>(scratch) + kNoAllocEbBytes),
+                    static_cast<cudaStream_t>(stream));
 }

@@ -30,7 +30,7 @@ struct TileInfo {
 struct Work {
   int n;             // tiles
   int ks0, kr, ks;   // K-split tail: first copy, tail tiles, shares (see GemmParams)
-  int mlim;          // dense grid: rows
+  int mlim, gm;      // dense grid: rows and row tiles (those that exist, so that the CTAs share them evenly)
   int4 next;         // the list entry of the CTA's next tile, fetched one ahead
 };
 
@@ -43,6 +43,7 @@ SVL_DEVINL Work load_work(const GemmParams& p, int first) {
   w.ks0 = 0x7fffffff;
   w.kr = w.ks = 0;
   w.mlim = p.m_limit;
+  w.gm = 1;
   w.next = make_int4(0, 0, 0, 0);
   if (p.tiles) {
     const int n = __ldcg(p.tile_count);
@@ -56,7 +57,8 @@ SVL_DEVINL Work load_work(const GemmParams& p, int first) {
     fetch_tile(p, w, first);
   } else {
     if (p.m_limit_dev) w.mlim = min(w.mlim, __ldcg(p.m_limit_dev));
-    w.n = p.grid_m * p.grid_n;
+    w.gm = max((w.mlim + kBM - 1) / kBM, 1);
+    w.n = w.gm * p.grid_n;
   }
   return w;
 }
@@ -75,7 +77,7 @@ SVL_DEVINL TileInfo get_tile(const GemmParams& p, Work& w, int t, int step) {
     ti.kmask = tile_kmask(v.w);
     ti.valid = ti.ncols > 0 && ti.m_end > ti.m0 && ti.mat < 3;
   } else {
-    const int mi = t % p.grid_m, ni = t / p.grid_m;
+    const int ni = t / w.gm, mi = t - ni * w.gm;
     ti.m0 = mi * kBM;
     ti.m_end = min(ti.m0 + kBM, w.mlim);
     ti.n0 = ni * p.bn;
@@ -176,6 +178,15 @@ struct StageCfg<EPI_LOGITS_T, true> {
   static constexpr int abytes = kABytes;
   static constexpr int bytes = kABytes + kThinRows * 128;
 };
+// Projector with few rows: 128-column tiles, six stages.
+template <>
+struct StageCfg<EPI_GELU, true> {
+  static constexpr int stages = 6;
+  static constexpr int abytes = kABytes;
+  static constexpr int bytes = kABytes + kBHalfBytes;
+};
+template <>
+struct StageCfg<EPI_ROWMAP, true> : StageCfg<EPI_GELU, true> {};
 template <>
 struct StageCfg<EPI_SCORE, false> {
   static constexpr int stages = 9;
@@ -533,16 +544,14 @@ SVL_DEVINL void epilogue_tile(const GemmParams& p, const TileInfo& ti, int row, 
       }
       b0 = lo;
     }
-    int b = __shfl_sync(0xffffffffu, b0, 0);
+    b0 = __shfl_sync(0xffffffffu, b0, 0);
+    int b = b0;
     if (rv)
       while (b + 1 < p.n_seg && p.seg_off[b + 1] <= row) ++b;
     const int H = ti.ncols;
-    const float4* eb = reinterpret_cast<const float4*>(p.e_b + static_cast<size_t>(b) * H);
-    const uint4* w2v = reinterpret_cast<const uint4*>(p.w2);
+    // 32 hidden units: e_b as 8 float4, w2 as 4 x 8 bf16 (H is a multiple of 16)
     float z = 0.f;
-    for (int c = 0; c < H; c += 32) {
-      tmem_ld32(taddr + c, v);
-      // 32 hidden units: e_b as 8 float4, w2 as 4 x 8 bf16 (H is a multiple of 16)
+    auto units = [&](int c, const float4* eb, const uint4* w2v) {
       const int n = min(32, H - c);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -557,6 +566,29 @@ SVL_DEVINL void epilogue_tile(const GemmParams& p, const TileInfo& ti, int row, 
         z += w2_.x * silu_f(v[j + 4] + e1.x) + w2_.y * silu_f(v[j + 5] + e1.y);
         z += w3.x * silu_f(v[j + 6] + e1.z) + w3.y * silu_f(v[j + 7] + e1.w);
       }
+    };
+    // The rows of a warp mostly belong to one sample: its e_b row and w2 then
+    // come into shared memory with one read each before the accumulator is
+    // read (reading them unit by unit exposed 2 us of latency per tile).
+    __shared__ __align__(16) float s_eb[4][128];
+    __shared__ __align__(16) __nv_bfloat16 s_w2[4][128];
+    const int wq4 = (threadIdx.x >> 5) & 3;
+    const bool one = __all_sync(0xffffffffu, b == b0);
+    __syncwarp();  // the previous tile's reads are done
+    if (one) {
+      if (lane * 4 < H)
+        *reinterpret_cast<float4*>(&s_eb[wq4][lane * 4]) =
+            *reinterpret_cast<const float4*>(p.e_b + static_cast<size_t>(b0) * H + lane * 4);
+      if (lane * 8 < H)
+        *reinterpret_cast<uint4*>(&s_w2[wq4][lane * 8]) = reinterpret_cast<const uint4*>(p.w2)[lane];
+    }
+    __syncwarp();
+    for (int c = 0; c < H; c += 32) {
+      tmem_ld32(taddr + c, v);
+      if (one)
+        units(c, reinterpret_cast<const float4*>(s_eb[wq4]), reinterpret_cast<const uint4*>(s_w2[wq4]));
+      else
+        units(c, reinterpret_cast<const float4*>(p.e_b + static_cast<size_t>(b) * H), reinterpret_cast<const uint4*>(p.w2));
     }
     if (rv) {
       z += p.c2;
@@ -1522,6 +1554,8 @@ cudaError_t launch_gemm(EpiKind kind, const GemmParams& p, int grid, cudaStream_
         return e4m3 ? launch_kind<EPI_SWIGLU, true, true>(p, grid, stream)
                     : launch_kind<EPI_SWIGLU, false, true>(p, grid, stream);
       case EPI_LOGITS_T: return launch_kind<EPI_LOGITS_T, false, true>(p, grid, stream);
+      case EPI_GELU: return launch_kind<EPI_GELU, false, true>(p, grid, stream);
+      case EPI_ROWMAP: return launch_kind<EPI_ROWMAP, false, true>(p, grid, stream);
       default: return cudaErrorInvalidValue;
     }
   }

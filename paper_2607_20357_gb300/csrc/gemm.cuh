@@ -54,7 +54,8 @@ struct GemmParams {
   const int4* tiles;
   const int* tile_count;
   int max_tiles;
-  // ... or dense grid: grid_m x grid_n tiles of kBM x bn
+  // ... or dense grid: grid_n column tiles of bn times the row tiles below the
+  // rows bound (grid_m: at most)
   int grid_m, grid_n, bn;
   const int* m_limit_dev;  // rows bound read on the device (nullptr: use m_limit)
   int m_limit, n_limit;
@@ -127,7 +128,8 @@ struct GemmParams {
 // `thin`: every tile has at most kThinRows rows and mapA has boxes of
 // kThinRows rows (QKV, residual and SwiGLU epilogues), or at most kThinRows
 // columns and mapB such boxes (EPI_LOGITS_T, whose weights are A): deeper
-// weight pipeline for decode-sized batches.
+// weight pipeline for decode-sized batches. For EPI_GELU and EPI_ROWMAP: tiles
+// of at most 128 columns, six stages.
 cudaError_t launch_gemm(EpiKind kind, const GemmParams& p, int grid, cudaStream_t stream, bool e4m3 = false,
                         bool thin = false);
 

@@ -38,8 +38,7 @@ struct SelectArgs {
   uint32_t* flags;
   int* kept_local;
   // the paper's own rule (Sec. 3.1, 3.3): gates from compute-controller
-  // logits (> 0), k = min(#{z > 0}, budget count), group fallback; nullptr:
-  // gates given, k = budget count
+  // logits (> 0), k = min(#{z > 0}, budget count), group fallback
   const float* gate_logits;  // [B, L, G]
   uint8_t* layer_gate_out;   // [B, L] projected gates (paper rule)
   uint8_t* group_gate_out;   // [B, L, G]
@@ -47,11 +46,25 @@ struct SelectArgs {
   float* kappa;              // [B] sum sigma(z) / N, or nullptr
 };
 
-void launch_budget_embed(const float* budget, const __nv_bfloat16* w1, const __nv_bfloat16* w2, int H, int B,
-                         float* e_b, cudaStream_t s);
+// Before the score GEMM: budget embeddings, and with `counts` k and the flags.
+struct FrontArgs {
+  int B, H;
+  const float* budget;
+  const __nv_bfloat16* w1;
+  const __nv_bfloat16* w2;
+  int w_vec;              // w1 and w2 are 16-byte aligned
+  const double* omega;    // [H / 2] frequencies of Eq. 5
+  float* e_b;             // [B, H]
+  int counts;             // gates given: k does not depend on the scores
+  SelectArgs sel;         // sizes, gates, k_out and flags for `counts`
+};
+void launch_front(const FrontArgs& f, cudaStream_t s);
+void launch_budget_omega(double* omega, int H, cudaStream_t s);
+void launch_topk(int B, const float* scores, const int* vis_off, const int* k, int* kept_off, int* kept_idx,
+                 cudaStream_t s);
 void launch_select(const SelectArgs& a, int B, cudaStream_t s);
 void launch_compact(int B, const int* vis_off, const int* k, const int* kept_local, int* kept_idx, int* kept_off,
-                    int* kept_total, cudaStream_t s);
+                    cudaStream_t s);
 
 // ---------------------------------------------------------------- pack
 struct PackArgs {
@@ -67,7 +80,6 @@ struct PackArgs {
   __nv_bfloat16* X;
   int* cu_seqlens;
   int* pos;
-  int* t_total;            // device scalar: T
   int use_projector;       // 1: visual rows go to the staging buffer
   __nv_bfloat16* stage;    // [kept_total, c_vis]
   int* row_map;            // [kept_total] -> row of X
@@ -77,9 +89,10 @@ struct PackArgs {
 // e^LLM_b = W2 SiLU(W1 PE(b)) (Sec. 3.2: the Eq. 5 encoding, its own MLP to D), bf16 rows.
 void launch_llm_budget_embed(const float* budget, const __nv_bfloat16* w1, const __nv_bfloat16* w2, int H, int D,
                              int B, __nv_bfloat16* out, cudaStream_t s);
-void launch_pack_offsets(const PackArgs& a, cudaStream_t s);
 void launch_offsets_diff(const int* off, int* len, int B, cudaStream_t s);
-void launch_pack_gather(const PackArgs& a, cudaStream_t s);
+cudaError_t launch_pack_gather(const PackArgs& a, cudaStream_t s);
+bool pack_needs_offsets(int B);  // the gather reads cu_seqlens from this launch instead
+void launch_pack_offsets(const PackArgs& a, cudaStream_t s);
 
 // Sample b of the packed row r: cu[b] <= r < cu[b+1].
 SVL_DEVINL int find_sample(const int* cu, int B, int r) {

@@ -7,38 +7,61 @@
 
 namespace svl {
 
-__global__ void pack_offsets_kernel(PackArgs a) {
-  pdl_begin(false);
-  if (threadIdx.x != 0) return;
-  int t = 0;
-  a.cu_seqlens[0] = 0;
-  for (int b = 0; b < a.B; ++b) {
-    const int kb = a.kept_off[b + 1] - a.kept_off[b];
-    const int st = a.text_off[b + 1] - a.text_off[b];
-    t += max(kb, 0) + max(st, 0) + (a.tok_rows ? 1 : 0);
-    if (t > a.t_cap) {
-      report(a.status, SVL_DEV_BAD_INDEX);
-      t = a.t_cap;
+constexpr int kPackThreads = 512;
+constexpr int kPackRows = kPackThreads / 32;  // a warp per output row
+
+constexpr int kPackScan = 4096;  // samples up to which every gather block forms the offsets itself
+
+// Row offsets of all samples into cu[0..B], by a whole block; `out` (or
+// nullptr) gets a copy. Samples past t_cap rows are cut off and reported.
+__device__ void row_offsets(const PackArgs& a, int* cu, int* out) {
+  __shared__ int warp_sums[32];
+  int before = 0;
+  bool over = false;
+  for (int b0 = 0; b0 < a.B; b0 += kPackThreads) {
+    const int b = b0 + threadIdx.x;
+    int rows = 0;
+    if (b < a.B)
+      rows = max(a.kept_off[b + 1] - a.kept_off[b], 0) + max(a.text_off[b + 1] - a.text_off[b], 0) +
+             (a.tok_rows ? 1 : 0);
+    int total;
+    const int end = before + block_exclusive_scan(rows, &total, warp_sums) + rows;
+    if (b < a.B) {
+      over = over || end > a.t_cap;
+      cu[b + 1] = min(end, a.t_cap);
+      if (out) out[b + 1] = min(end, a.t_cap);
     }
-    a.cu_seqlens[b + 1] = t;
+    before += total;
   }
-  *a.t_total = t;
+  if (threadIdx.x == 0) {
+    cu[0] = 0;
+    if (out) out[0] = 0;
+  }
+  if (out && over) report(a.status, SVL_DEV_BAD_INDEX);
 }
 
-// One warp per output row.
-__global__ void pack_gather_kernel(PackArgs a) {
+__global__ void __launch_bounds__(kPackThreads) pack_offsets_kernel(PackArgs a) {
+  pdl_begin(false);
+  row_offsets(a, a.cu_seqlens, a.cu_seqlens);
+}
+
+// Every block forms the row offsets of all samples in shared memory (a launch
+// of one thread that walked them cost 4 us before this one); the first block
+// writes them out. Beyond kPackScan samples they come from their own launch.
+__global__ void __launch_bounds__(kPackThreads) pack_gather_kernel(PackArgs a) {
+  extern __shared__ int pack_cu[];  // [B + 1], up to kPackScan samples
   pdl_begin(a.use_projector);  // the projector GEMM loads weights before it waits
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r = blockIdx.x * (blockDim.x >> 5) + warp;
-  const int T = *a.t_total;
-  if (r >= T) return;
-  int lo = 0, hi = a.B;  // sample b with cu[b] <= r < cu[b+1]
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (a.cu_seqlens[mid] <= r) lo = mid; else hi = mid;
+  const int* cu = a.cu_seqlens;
+  if (a.B <= kPackScan) {
+    row_offsets(a, pack_cu, blockIdx.x == 0 ? a.cu_seqlens : nullptr);
+    cu = pack_cu;
   }
-  const int b = lo;
-  const int i = r - a.cu_seqlens[b];
+  __syncthreads();
+  const int r = blockIdx.x * kPackRows + warp;
+  if (r >= cu[a.B]) return;
+  const int b = find_sample(cu, a.B, r);
+  const int i = r - cu[b];
   const int kb = a.kept_off[b + 1] - a.kept_off[b];
   if (lane == 0) a.pos[r] = i;
   const uint4* src;
@@ -70,7 +93,17 @@ __global__ void pack_gather_kernel(PackArgs a) {
     width = a.D;
   }
   if (bad && lane == 0) report(a.status, SVL_DEV_BAD_INDEX);
-  for (int c = lane; c < width / 8; c += 32) dst[c] = bad ? make_uint4(0, 0, 0, 0) : src[c];
+  // four 16-byte pieces per lane in flight
+  const int n = width / 8;
+  for (int c0 = lane; c0 < n; c0 += 128) {
+    uint4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (c0 + 32 * u < n) v[u] = bad ? make_uint4(0, 0, 0, 0) : __ldg(src + c0 + 32 * u);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (c0 + 32 * u < n) dst[c0 + 32 * u] = v[u];
+  }
 }
 
 __global__ void offsets_diff_kernel(const int* off, int* len, int B) {
@@ -82,8 +115,6 @@ __global__ void offsets_diff_kernel(const int* off, int* len, int B) {
 void launch_offsets_diff(const int* off, int* len, int B, cudaStream_t s) {
   launch_pdl(offsets_diff_kernel, (B + 255) / 256, 256, 0, s, off, len, B);
 }
-
-void launch_pack_offsets(const PackArgs& a, cudaStream_t s) { launch_pdl(pack_offsets_kernel, 1, 32, 0, s, a); }
 
 // One block per sample: PE(b) and the hidden layer in double, then D outputs.
 __global__ void llm_budget_embed_kernel(const float* __restrict__ budget, const __nv_bfloat16* __restrict__ w1,
@@ -119,10 +150,16 @@ void launch_llm_budget_embed(const float* budget, const __nv_bfloat16* w1, const
   launch_pdl(llm_budget_embed_kernel, B, 256, 0, s, budget, w1, w2, H, D, out);
 }
 
-void launch_pack_gather(const PackArgs& a, cudaStream_t s) {
-  const int rows_per_block = 8;
-  const int grid = (a.t_cap + rows_per_block - 1) / rows_per_block;
-  if (grid > 0) launch_pdl(pack_gather_kernel, grid, rows_per_block * 32, 0, s, a);
+cudaError_t launch_pack_gather(const PackArgs& a, cudaStream_t s) {
+  const int grid = (a.t_cap + kPackRows - 1) / kPackRows;
+  // (one block at least: it writes cu_seqlens)
+  return launch_pdl(pack_gather_kernel, grid > 0 ? grid : 1, kPackThreads,
+                    a.B <= kPackScan ? sizeof(int) * (static_cast<size_t>(a.B) + 1) : 0, s, a);
+}
+
+bool pack_needs_offsets(int B) { return B > kPackScan; }
+void launch_pack_offsets(const PackArgs& a, cudaStream_t s) {
+  launch_pdl(pack_offsets_kernel, 1, kPackThreads, 0, s, a);
 }
 
 }  // namespace svl

@@ -6,43 +6,127 @@
 namespace svl {
 
 // e_b = W_b2 SiLU(W_b1 PE(b)), PE(b) = [sin(1000 b w_i) | cos(1000 b w_i)],
-// w_i = 10000^(-2i/H) (Eq. 5). One block per sample. The argument reaches
-// 1000 rad, so it is formed and reduced to [-pi, pi] in double precision
-// before the single-precision sine and cosine (error about 1e-7 either way);
-// the two H x H products run in fp32, four threads per output.
+// w_i = 10000^(-2i/H) (Eq. 5; `omega`, kept by the model: a double-precision
+// pow per call took 2 us). One block per sample. The argument reaches 1000 rad,
+// so it is formed and reduced to [-pi, pi] in double precision before the
+// single-precision sine and cosine (error about 1e-7 either way); the two H x H
+// products run in fp32 from shared memory, four threads per output. The weights
+// are copied there before the wait for the predecessor.
 constexpr double kTwoPi = 6.283185307179586;
+constexpr int kFrontThreads = 256;
 
-SVL_DEVINL void budget_matvec(const __nv_bfloat16* __restrict__ w, const float* x, int H, float* y, bool silu) {
+SVL_DEVINL void budget_matvec(const __nv_bfloat16* w, const float* x, int H, float* y, bool silu) {
   const int i = threadIdx.x, part = i & 3;
-  for (int o0 = 0; o0 < H; o0 += blockDim.x / 4) {
+  for (int o0 = 0; o0 < H; o0 += kFrontThreads / 4) {
     const int o = o0 + i / 4;
     float s = 0.f;
-    if (o < H)
-      for (int j = part; j < H; j += 4) s = fmaf(__bfloat162float(w[static_cast<size_t>(o) * H + j]), x[j], s);
+    if (o < H) {
+#pragma unroll 8
+      for (int j = part; j < H; j += 4) s = fmaf(__bfloat162float(w[o * H + j]), x[j], s);
+    }
     s += __shfl_xor_sync(0xffffffffu, s, 1);
     s += __shfl_xor_sync(0xffffffffu, s, 2);
     if (o < H && part == 0) y[o] = silu ? s / (1.f + expf(-s)) : s;
   }
 }
 
-__global__ void budget_embed_kernel(const float* __restrict__ budget, const __nv_bfloat16* __restrict__ w1,
-                                    const __nv_bfloat16* __restrict__ w2, int H, float* __restrict__ e_b) {
+__global__ void budget_omega_kernel(double* omega, int H) {
+  const int f = threadIdx.x;
+  if (f < H / 2) omega[f] = pow(10000.0, -2.0 * f / H);
+}
+
+void launch_budget_omega(double* omega, int H, cudaStream_t s) { budget_omega_kernel<<<1, 128, 0, s>>>(omega, H); }
+
+// Eq. 8 for one sample, times G so that it is an exact integer.
+struct CostModel {
+  long long lin, D4, lm, GL;
+  SVL_DEVINL CostModel(const SelectArgs& a)
+      : lin(4 * a.D * a.D + 4 * a.D * a.Dkv + 6 * a.D * a.Di), D4(4 * a.D), lm(a.G * 2 * a.D * a.V),
+        GL(static_cast<long long>(a.G) * a.L) {}
+  SVL_DEVINL long long cost(long long n_on, long long S) const { return n_on * (lin * S + D4 * S * S) + lm * S; }
+};
+
+// Blocks 0 .. B-1: the budget embedding of a sample. Blocks B .. 2B-1, when the
+// counts do not depend on the scores (`counts`: gates given): k and the flags of
+// a sample, beside the score GEMM instead of after it. (One block for all
+// samples with a thread each took 10 us for 64 samples.)
+__global__ void __launch_bounds__(kFrontThreads) front_kernel(FrontArgs f) {
+  extern __shared__ __align__(16) uint8_t front_smem[];
   __shared__ float pe[256];
   __shared__ float hid[256];
+  const int b = blockIdx.x, i = threadIdx.x, H = f.H;
+  __nv_bfloat16* sw1 = reinterpret_cast<__nv_bfloat16*>(front_smem);
+  __nv_bfloat16* sw2 = sw1 + H * H;
+  if (b < f.B) {
+    if (f.w_vec) {
+      for (int c = i; c < H * H / 8; c += kFrontThreads) {
+        reinterpret_cast<uint4*>(sw1)[c] = reinterpret_cast<const uint4*>(f.w1)[c];
+        reinterpret_cast<uint4*>(sw2)[c] = reinterpret_cast<const uint4*>(f.w2)[c];
+      }
+    } else {
+      for (int c = i; c < H * H; c += kFrontThreads) {
+        sw1[c] = f.w1[c];
+        sw2[c] = f.w2[c];
+      }
+    }
+  }
   pdl_begin(true);  // the score GEMM loads its operands before it waits
-  const int b = blockIdx.x, i = threadIdx.x;
-  if (i < H) {
-    const int half = H / 2;
-    const int f = i < half ? i : i - half;
-    const double omega = pow(10000.0, -2.0 * f / H);
-    const double arg = 1000.0 * static_cast<double>(budget[b]) * omega;
-    const float r = static_cast<float>(arg - rint(arg / kTwoPi) * kTwoPi);
-    pe[i] = i < half ? sinf(r) : cosf(r);
+  if (b < f.B) {
+    if (i < H) {
+      const int half = H / 2;
+      const double arg = 1000.0 * static_cast<double>(f.budget[b]) * f.omega[i < half ? i : i - half];
+      const float r = static_cast<float>(arg - rint(arg / kTwoPi) * kTwoPi);
+      pe[i] = i < half ? sinf(r) : cosf(r);
+    }
+    __syncthreads();
+    budget_matvec(sw1, pe, H, hid, true);
+    __syncthreads();
+    budget_matvec(sw2, hid, H, f.e_b + static_cast<size_t>(b) * H, false);
+    return;
+  }
+  const SelectArgs& a = f.sel;
+  const int s = b - f.B;
+  __shared__ int on_groups, best_k;
+  if (i == 0) {
+    on_groups = 0;
+    best_k = -1;
   }
   __syncthreads();
-  budget_matvec(w1, pe, H, hid, true);
+  const int n = max(0, a.vis_off[s + 1] - a.vis_off[s]);
+  const int kc = a.keep_count ? a.keep_count[s] : -1;
+  const long long st = a.text_len[s];
+  const double budget = static_cast<double>(a.budget[s]);
+  const uint8_t* lg = a.layer_gate + static_cast<size_t>(s) * a.L;
+  const uint8_t* gg = a.group_gate + static_cast<size_t>(s) * a.L * a.G;
+  int on = 0;  // active (layer, group) pairs
+  for (int idx = i; idx < a.L * a.G; idx += kFrontThreads) {
+    const int l = idx / a.G;
+    on += (l < a.P || (gg[idx] && lg[l])) ? 1 : 0;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) on += __shfl_xor_sync(0xffffffffu, on, o);
+  if ((i & 31) == 0 && on) atomicAdd(&on_groups, on);
   __syncthreads();
-  budget_matvec(w2, hid, H, e_b + static_cast<size_t>(b) * H, false);
+  const CostModel cm(a);
+  const double limit = budget * static_cast<double>(cm.cost(cm.GL, n + st));
+  // the cost grows with k, so the feasible counts are a prefix: take the largest
+  int mine = -1;
+  for (int kk = i; kk <= n; kk += kFrontThreads)
+    if (static_cast<double>(cm.cost(on_groups, st + kk)) <= limit) mine = kk;
+  mine = __reduce_max_sync(0xffffffffu, mine);
+  if ((i & 31) == 0 && mine >= 0) atomicMax(&best_k, mine);
+  __syncthreads();
+  if (i == 0) {
+    a.k_out[s] = kc >= 0 ? min(kc, n) : max(best_k, 0);
+    if (a.flags) a.flags[s] = (kc < 0 && best_k < 0) ? SVL_FLAG_OVER_BUDGET : 0;
+  }
+}
+
+void launch_front(const FrontArgs& f, cudaStream_t s) {
+  const size_t smem = 2 * sizeof(__nv_bfloat16) * static_cast<size_t>(f.H) * f.H;
+  if (smem > 40 * 1024)
+    cudaFuncSetAttribute(front_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  launch_pdl(front_kernel, f.B * (f.counts ? 2 : 1), kFrontThreads, smem, s, f);
 }
 
 // Orderable key: unsigned comparison of keys matches float comparison.
@@ -52,9 +136,129 @@ SVL_DEVINL uint32_t order_key(float z) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// One block per sample: k from the budget (largest k with Eq. 8 cost within
-// b * C_full), then the k largest logits (ties: lower index), written in
-// ascending index order to kept_local[vis_off[b] ...].
+// Selection of one sample by a whole block: the k largest logits of z[0..n)
+// (equal logits: lower index first), as ascending indices to out. The keys are
+// read once, into shared memory while they fit (kKeysShared).
+constexpr int kKeysShared = 4096;
+
+__device__ void top_k(const float* z, int n, int k, int* out, uint32_t* skeys) {
+  __shared__ int hist[256];
+  __shared__ int warp_sums[32];
+  __shared__ int s_prefix_cnt[2];
+  const int tid = threadIdx.x;
+  if (k == 0) return;
+  if (k >= n) {
+    for (int i = tid; i < n; i += blockDim.x) out[i] = i;
+    return;
+  }
+  const bool shared = n <= kKeysShared;
+  if (shared)
+    for (int i = tid; i < n; i += blockDim.x) skeys[i] = order_key(z[i]);
+  auto key_at = [&](int i) -> uint32_t { return shared ? skeys[i] : order_key(z[i]); };
+
+  // ---- radix select of the k-th largest key, 8 bits per pass, MSB first
+  uint32_t prefix = 0, mask = 0;
+  int remaining = k;  // keys still to take among those matching `prefix`
+  for (int shift = 24; shift >= 0; shift -= 8) {
+    for (int i = tid; i < 256; i += blockDim.x) hist[i] = 0;
+    __syncthreads();
+    for (int i = tid; i < n; i += blockDim.x) {
+      const uint32_t key = key_at(i);
+      if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 0xFF], 1);
+    }
+    __syncthreads();
+    if (tid < 32) {
+      // warp 0: counts above each digit (suffix sums from 255 down), then the
+      // largest digit d whose keys with digit >= d reach `remaining`
+      int cnt[8], sum = 0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        cnt[u] = hist[255 - (tid * 8 + u)];  // lane t holds digits 255-8t .. 248-8t
+        sum += cnt[u];
+      }
+      int incl = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (tid >= o) incl += y;
+      }
+      int above = incl - sum;  // keys with a digit above this lane's first digit
+      int found = -1, found_above = 0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if (found < 0 && above + cnt[u] >= remaining) {
+          found = 255 - (tid * 8 + u);
+          found_above = above;
+        }
+        above += cnt[u];
+      }
+      const unsigned ballot = __ballot_sync(0xffffffffu, found >= 0);
+      const int first = ballot ? __ffs(ballot) - 1 : 31;
+      const int d = __shfl_sync(0xffffffffu, found, first);
+      const int ab = __shfl_sync(0xffffffffu, found_above, first);
+      if (tid == 0) {
+        s_prefix_cnt[0] = d < 0 ? 0 : d;
+        s_prefix_cnt[1] = remaining - (d < 0 ? 0 : ab);
+      }
+    }
+    __syncthreads();
+    prefix |= static_cast<uint32_t>(s_prefix_cnt[0]) << shift;
+    mask |= 0xFFu << shift;
+    remaining = s_prefix_cnt[1];
+  }
+  const uint32_t tau = prefix;  // key of the k-th largest logit
+  // keys > tau are kept; of the keys == tau, the `remaining` lowest indices
+
+  // ---- ordered pass: per chunk the ranks of equal keys and the output
+  // positions by index from one scan of both counts (16 bits each: a chunk has
+  // at most 1,024 keys)
+  int eq_before = 0, kept_before = 0;
+  for (int base = 0; base < n; base += blockDim.x) {
+    const int i = base + tid;
+    const uint32_t key = i < n ? key_at(i) : 0;
+    const int gt = (i < n && key > tau) ? 1 : 0, eq = (i < n && key == tau) ? 1 : 0;
+    int total;
+    const int ex = block_exclusive_scan(gt | (eq << 16), &total, warp_sums);
+    const int eq_rank = eq_before + (ex >> 16);
+    // kept before this key: the greater ones and the equal ones taken so far
+    const int pos = kept_before + (ex & 0xFFFF) + min(eq_rank, remaining) - min(eq_before, remaining);
+    if (gt || (eq && eq_rank < remaining)) out[pos] = i;
+    const int eq_after = eq_before + (total >> 16);
+    kept_before += (total & 0xFFFF) + min(eq_after, remaining) - min(eq_before, remaining);
+    eq_before = eq_after;
+  }
+}
+
+// One block per sample whose k is known (front_kernel): its kept offset is the
+// sum of the k before it, and its indices go to their final place.
+__global__ void __launch_bounds__(kSelectThreads) topk_kernel(int B, const float* scores, const int* vis_off,
+                                                              const int* k, int* kept_off, int* kept_idx) {
+  __shared__ uint32_t topk_keys[kKeysShared];
+  __shared__ int off;
+  pdl_begin(false);
+  const int b = blockIdx.x, tid = threadIdx.x, v0 = vis_off[b], n = max(0, vis_off[b + 1] - v0), kb = k[b];
+  if (tid == 0) off = 0;
+  __syncthreads();
+  int part = 0;
+  for (int i = tid; i < b; i += kSelectThreads) part += k[i];
+  part = __reduce_add_sync(0xffffffffu, part);
+  if ((tid & 31) == 0 && part) atomicAdd(&off, part);
+  __syncthreads();
+  if (tid == 0) {
+    kept_off[b] = off;
+    if (b == B - 1) kept_off[B] = off + kb;
+  }
+  top_k(scores + v0, n, kb, kept_idx + off, topk_keys);
+}
+
+void launch_topk(int B, const float* scores, const int* vis_off, const int* k, int* kept_off, int* kept_idx,
+                 cudaStream_t s) {
+  launch_pdl(topk_kernel, B, kSelectThreads, 0, s, B, scores, vis_off, k, kept_off, kept_idx);
+}
+
+// One block per sample, for the rules whose k depends on the scores: k, then
+// the k largest logits (ties: lower index), written in ascending index order to
+// kept_local[vis_off[b] ...].
 //
 // Under the paper's own rule (a.gate_logits set; Sec. 3.1 and Sec. 3.3
 // "Inference") the gates are the compute controller's logits > 0 (prefix
@@ -63,10 +267,8 @@ SVL_DEVINL uint32_t order_key(float z) {
 // l >= P that make it fit are switched off, lowest logit first (equal logits:
 // lower (l, j) first); the projected gates are written out.
 __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectArgs a) {
-  __shared__ int hist[256];
-  __shared__ int warp_sums[32];
+  __shared__ uint32_t topk_keys[kKeysShared];
   __shared__ int best_k;
-  __shared__ int s_prefix_cnt[2];
   __shared__ long long n_on_sum;  // updated with 64-bit atomics
   __shared__ int n_pos, keep_groups;
   __shared__ double kappa_sum;
@@ -87,11 +289,7 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectArgs a) {
   }
   __syncthreads();
   const float* gl = a.gate_logits ? a.gate_logits + static_cast<size_t>(b) * a.L * a.G : nullptr;
-  auto active = [&](int idx) -> bool {
-    const int l = idx / a.G;
-    if (l < a.P) return true;
-    return gl ? gl[idx] > 0.f : (a.layer_gate[b * a.L + l] && a.group_gate[b * a.L * a.G + idx]);
-  };
+  auto active = [&](int idx) -> bool { return idx / a.G < a.P || gl[idx] > 0.f; };
   {
     // active (layer, group) pairs of this sample; not needed (and no gates
     // given) when the gates are decided later
@@ -101,13 +299,11 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectArgs a) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) on += __shfl_xor_sync(0xffffffffu, on, o);
     if ((tid & 31) == 0 && on) atomicAdd(reinterpret_cast<unsigned long long*>(&n_on_sum), static_cast<unsigned long long>(on));
-    if (gl || a.threshold_only) {
-      int pos = 0;  // logits z > 0, i.e. sigma(z) > 0.5
-      for (int i = tid; i < n; i += blockDim.x) pos += a.scores[v0 + i] > 0.f ? 1 : 0;
+    int pos = 0;  // logits z > 0, i.e. sigma(z) > 0.5
+    for (int i = tid; i < n; i += blockDim.x) pos += a.scores[v0 + i] > 0.f ? 1 : 0;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) pos += __shfl_xor_sync(0xffffffffu, pos, o);
-      if ((tid & 31) == 0 && pos) atomicAdd(&n_pos, pos);
-    }
+    for (int o = 16; o > 0; o >>= 1) pos += __shfl_xor_sync(0xffffffffu, pos, o);
+    if ((tid & 31) == 0 && pos) atomicAdd(&n_pos, pos);
     if (a.kappa) {
       // survival rate kappa = sum sigma(z_i) / N that conditions the compute controller (Sec. 3.2)
       double sg = 0.0;
@@ -142,10 +338,7 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectArgs a) {
     if (mine >= 0) atomicMax(&best_k, static_cast<int>(mine));
     __syncthreads();
     if (best_k >= 0) {
-      k = gl ? min(best_k, n_pos) : best_k;
-    } else if (!gl) {
-      k = 0;
-      flags |= SVL_FLAG_OVER_BUDGET;
+      k = min(best_k, n_pos);
     } else {
       // paper rule: no visual token fits, so head groups go. The most groups
       // that still fit with the text alone (prefix groups cannot go):
@@ -191,90 +384,13 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectArgs a) {
     if (a.flags) a.flags[b] = flags;
   }
 
-  const float* z = a.scores + v0;
-  int* out = a.kept_local + v0;
-  if (k == 0) return;
-  if (k >= n) {
-    for (int i = tid; i < n; i += blockDim.x) out[i] = i;
-    return;
-  }
-
-  // ---- radix select of the k-th largest key, 8 bits per pass, MSB first
-  uint32_t prefix = 0, mask = 0;
-  int remaining = k;  // keys still to take among those matching `prefix`
-  for (int shift = 24; shift >= 0; shift -= 8) {
-    for (int i = tid; i < 256; i += blockDim.x) hist[i] = 0;
-    __syncthreads();
-    for (int i = tid; i < n; i += blockDim.x) {
-      const uint32_t key = order_key(z[i]);
-      if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 0xFF], 1);
-    }
-    __syncthreads();
-    if (tid < 32) {
-      // warp 0: counts above each digit (suffix sums from 255 down), then the
-      // largest digit d whose keys with digit >= d reach `remaining`
-      int cnt[8], sum = 0;
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        cnt[u] = hist[255 - (tid * 8 + u)];  // lane t holds digits 255-8t .. 248-8t
-        sum += cnt[u];
-      }
-      int incl = sum;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (tid >= o) incl += y;
-      }
-      int above = incl - sum;  // keys with a digit above this lane's first digit
-      int found = -1, found_above = 0;
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        if (found < 0 && above + cnt[u] >= remaining) {
-          found = 255 - (tid * 8 + u);
-          found_above = above;
-        }
-        above += cnt[u];
-      }
-      const unsigned ballot = __ballot_sync(0xffffffffu, found >= 0);
-      const int first = ballot ? __ffs(ballot) - 1 : 31;
-      const int d = __shfl_sync(0xffffffffu, found, first);
-      const int ab = __shfl_sync(0xffffffffu, found_above, first);
-      if (tid == 0) {
-        s_prefix_cnt[0] = d < 0 ? 0 : d;
-        s_prefix_cnt[1] = remaining - (d < 0 ? 0 : ab);
-      }
-    }
-    __syncthreads();
-    prefix |= static_cast<uint32_t>(s_prefix_cnt[0]) << shift;
-    mask |= 0xFFu << shift;
-    remaining = s_prefix_cnt[1];
-    __syncthreads();
-  }
-  const uint32_t tau = prefix;  // key of the k-th largest logit
-  // keys > tau are kept; of the keys == tau, the `remaining` lowest indices
-
-  // ---- ordered pass: ranks of equal keys and output positions by index
-  int eq_before = 0, kept_before = 0;
-  for (int base = 0; base < n; base += blockDim.x) {
-    const int i = base + tid;
-    uint32_t key = 0;
-    if (i < n) key = order_key(z[i]);
-    const int is_eq = (i < n && key == tau) ? 1 : 0;
-    int eq_total;
-    const int eq_rank = eq_before + block_exclusive_scan(is_eq, &eq_total, warp_sums);
-    const int keep = (i < n && (key > tau || (is_eq && eq_rank < remaining))) ? 1 : 0;
-    int keep_total;
-    const int pos = kept_before + block_exclusive_scan(keep, &keep_total, warp_sums);
-    if (keep) out[pos] = i;
-    eq_before += eq_total;
-    kept_before += keep_total;
-  }
+  top_k(a.scores + v0, n, k, a.kept_local + v0, topk_keys);
 }
 
 // Compacts the per-sample kept lists: kept_off[b] = k_0 + ... + k_{b-1}.
 __global__ void compact_kernel(int B, const int* __restrict__ vis_off, const int* __restrict__ k,
                                const int* __restrict__ kept_local, int* __restrict__ kept_idx,
-                               int* __restrict__ kept_off, int* __restrict__ kept_total) {
+                               int* __restrict__ kept_off) {
   __shared__ int off;
   pdl_begin(false);
   const int b = blockIdx.x;
@@ -288,19 +404,11 @@ __global__ void compact_kernel(int B, const int* __restrict__ vis_off, const int
   __syncthreads();
   if (threadIdx.x == 0) {
     kept_off[b] = off;
-    if (b == B - 1) {
-      kept_off[B] = off + k[b];
-      if (kept_total) *kept_total = off + k[b];
-    }
+    if (b == B - 1) kept_off[B] = off + k[b];
   }
   const int kb = k[b];
   const int* src = kept_local + vis_off[b];
   for (int i = threadIdx.x; i < kb; i += blockDim.x) kept_idx[off + i] = src[i];
-}
-
-void launch_budget_embed(const float* budget, const __nv_bfloat16* w1, const __nv_bfloat16* w2, int H, int B,
-                         float* e_b, cudaStream_t s) {
-  launch_pdl(budget_embed_kernel, B, 256, 0, s, budget, w1, w2, H, e_b);
 }
 
 void launch_select(const SelectArgs& a, int B, cudaStream_t s) {
@@ -308,8 +416,8 @@ void launch_select(const SelectArgs& a, int B, cudaStream_t s) {
 }
 
 void launch_compact(int B, const int* vis_off, const int* k, const int* kept_local, int* kept_idx, int* kept_off,
-                    int* kept_total, cudaStream_t s) {
-  launch_pdl(compact_kernel, B, 256, 0, s, B, vis_off, k, kept_local, kept_idx, kept_off, kept_total);
+                    cudaStream_t s) {
+  launch_pdl(compact_kernel, B, 256, 0, s, B, vis_off, k, kept_local, kept_idx, kept_off);
 }
 
 }  // namespace svl
