@@ -166,7 +166,9 @@ PreLayout pre_layout(const svl_model_desc& d, int B, int64_t t_cap) {
   L.t_pad = (t_cap + 7) & ~int64_t(7);
   L.n_pad = ((B + 15) / 16) * 16;
   L.mt_max = static_cast<int>(t_cap / 128 + B + 1);
-  const int qkv_nt = static_cast<int>((hq / 256 + G + 1) + 2 * (dkv / 256 + G + 1));
+  // (THIN launches cut Q, K and V into 128-column tiles)
+  const int step = t_cap <= kThinRows ? kBHalf : 2 * kBHalf;
+  const int qkv_nt = static_cast<int>((hq / step + G + 1) + 2 * (dkv / step + G + 1));
   // + 256: room for the split tail (at most half a wave of extra tiles)
   L.qkv_cap = L.mt_max * qkv_nt + 256;
   L.o_cap = L.mt_max * ((d.d_model + 255) / 256) + 256;
@@ -900,6 +902,7 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
   const bool thin_launch = t_cap <= kThinRows;
   const bool pair = m->pair_clusters > 0 && !m->e4m3 && !thin_launch;
   sa.nsparse_rows = pair ? 2 * kBM : kBM;
+  sa.qkv_step = thin_launch ? kBHalf : 2 * kBHalf;
   sa.nsparse_wave = pair ? m->pair_clusters : m->num_sms;
   sa.A = d.n_heads;
   sa.Akv = d.n_kv_heads;

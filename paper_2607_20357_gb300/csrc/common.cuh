@@ -107,6 +107,20 @@ SVL_DEVINL float ex2(float x) {
 // Upper bound of a device-side wait, in SM clock cycles (about 2 s at 2 GHz).
 constexpr long long kWaitCycles = 4000000000LL;
 
+// True in exactly one thread of a converged warp. (For the single-thread roles:
+// under this predicate the compiler knows that one thread runs and keeps the
+// operands of TMA and tcgen05 instructions in uniform registers; under
+// `lane == 0` it does not.)
+SVL_DEVINL bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.b32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+
 // ---------------------------------------------------------------- mbarrier
 SVL_DEVINL void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));

@@ -66,9 +66,9 @@ void launch_kv_store(const KvArgs& a, int t_cap, cudaStream_t s) {
 //  - one query head per KV head: a block per head, a warp per run, and the V
 //    rows are requested into registers before the scores are formed;
 //  - several (GQA): a cluster of kRuns blocks per KV head, a block per run, a
-//    warp per query head, so the cache is read once for all of them; the tiles
-//    of the next 32 positions load while these are worked on, and the runs meet
-//    through distributed shared memory.
+//    warp per query head, so the cache is read once for all of them; 128
+//    positions at a time (the score chains of four tiles side by side) while
+//    the next 128 load, and the runs meet through distributed shared memory.
 constexpr int kRuns = 8;
 constexpr int kDecThreads = kRuns * 32;
 
@@ -93,50 +93,65 @@ struct RunState {
   float m = -INFINITY, l = 0.f, o[PER];
 };
 
-// Score of key `lane` of a K tile against sq (q * scale): one chain over the
-// dimensions, its operands read eight 16-byte chunks at a time so that only
-// the first read's latency is exposed.
-template <int DH>
-SVL_DEVINL float tile_score(const uint8_t* ktile, const float* sq, int lane) {
+// Scores of key `lane` of KT consecutive K tiles (`pitch` bytes apart) against
+// sq (q * scale): one chain over the dimensions per tile, the tiles' chains side
+// by side, operands read four 16-byte chunks at a time so that only the first
+// read's latency is exposed.
+template <int DH, int KT>
+SVL_DEVINL void tile_scores(const uint8_t* ktile, int pitch, const float* sq, int lane, float* acc) {
   const uint8_t* row = ktile + lane * DH * 2;
   const int sw = (lane & 7) << 4;
-  float acc = 0.f;
+  constexpr int CB = KT > 1 ? 4 : 8;  // chunks per batch
 #pragma unroll
-  for (int c0 = 0; c0 < DH / 8; c0 += 8) {
-    uint4 u[8];
+  for (int t = 0; t < KT; ++t) acc[t] = 0.f;
 #pragma unroll
-    for (int c = 0; c < 8; ++c) u[c] = *reinterpret_cast<const uint4*>(row + (((c0 + c) << 4) ^ sw));
+  for (int c0 = 0; c0 < DH / 8; c0 += CB) {
+    uint4 u[KT][CB];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
+    for (int t = 0; t < KT; ++t)
+#pragma unroll
+      for (int c = 0; c < CB; ++c)
+        u[t][c] = *reinterpret_cast<const uint4*>(row + t * pitch + (((c0 + c) << 4) ^ sw));
+#pragma unroll
+    for (int c = 0; c < CB; ++c) {
       const float4 q0 = *reinterpret_cast<const float4*>(sq + 8 * (c0 + c));
       const float4 q1 = *reinterpret_cast<const float4*>(sq + 8 * (c0 + c) + 4);
-      const float2 k0 = unpack_bf16x2(u[c].x), k1 = unpack_bf16x2(u[c].y), k2 = unpack_bf16x2(u[c].z),
-                   k3 = unpack_bf16x2(u[c].w);
-      acc = fmaf(q0.x, k0.x, acc);
-      acc = fmaf(q0.y, k0.y, acc);
-      acc = fmaf(q0.z, k1.x, acc);
-      acc = fmaf(q0.w, k1.y, acc);
-      acc = fmaf(q1.x, k2.x, acc);
-      acc = fmaf(q1.y, k2.y, acc);
-      acc = fmaf(q1.z, k3.x, acc);
-      acc = fmaf(q1.w, k3.y, acc);
+#pragma unroll
+      for (int t = 0; t < KT; ++t) {
+        const float2 k0 = unpack_bf16x2(u[t][c].x), k1 = unpack_bf16x2(u[t][c].y), k2 = unpack_bf16x2(u[t][c].z),
+                     k3 = unpack_bf16x2(u[t][c].w);
+        float s = acc[t];
+        s = fmaf(q0.x, k0.x, s);
+        s = fmaf(q0.y, k0.y, s);
+        s = fmaf(q0.z, k1.x, s);
+        s = fmaf(q0.w, k1.y, s);
+        s = fmaf(q1.x, k2.x, s);
+        s = fmaf(q1.y, k2.y, s);
+        s = fmaf(q1.z, k3.x, s);
+        acc[t] = fmaf(q1.w, k3.y, s);
+      }
     }
   }
-  return acc;
 }
 
-// Folds 32 scores (valid where `in`) into the run's max and row sum; returns
-// this lane's probability.
-template <int PER>
-SVL_DEVINL float fold_scores(RunState<PER>& r, float sc, bool in) {
-  float mx = sc;
+SVL_DEVINL float warp_max(float x) {
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+  for (int off = 16; off > 0; off >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, off));
+  return x;
+}
+SVL_DEVINL float warp_sum(float x) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+  return x;
+}
+
+// Folds a tile's 32 scores into the run's max and row sum, given their max
+// over the warp; returns this lane's probability (0 where not `in`).
+template <int PER>
+SVL_DEVINL float fold_scores(RunState<PER>& r, float sc, float mx, bool in) {
   const float mn = fmaxf(r.m, mx);
   const float e = in ? __expf(sc - mn) : 0.f;
-  float es = e;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) es += __shfl_xor_sync(0xffffffffu, es, off);
+  const float es = warp_sum(e);
   const float corr = __expf(r.m - mn);  // 0 while m is -inf
   r.l = r.l * corr + es;
 #pragma unroll
@@ -217,7 +232,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(DecAttnArgs
   // rows at a time as far as the run goes
   const __nv_bfloat16* kc = a.k_cache + cbase + (lane % CH) * 8;
   const __nv_bfloat16* vc = a.v_cache + cbase + lane * PER;
-  auto request = [&](int p0) {
+  auto request_k = [&](int p0) {
     constexpr int RI = 32 / CH;  // rows per instruction
 #pragma unroll
     for (int it = 0; it < CH; ++it) {
@@ -227,6 +242,8 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(DecAttnArgs
                    p < len ? kc + static_cast<size_t>(p) * a.dkv : knew + (lane % CH) * 8);
     }
     cp_async_commit();
+  };
+  auto request_v = [&](int p0) {
     const int cached = min(p_end, len) - p0;
 #pragma unroll
     for (int j0 = 0; j0 < 32; j0 += 8) {
@@ -236,7 +253,8 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(DecAttnArgs
         vv[j] = row_part<PER>(vc + static_cast<size_t>(p0 + min(j, cached - 1)) * a.dkv);
     }
   };
-  request(p_begin);
+  request_k(p_begin);
+  request_v(p_begin);
   if (tid < DH) {
     sq[tid] = __bfloat162float(a.q[static_cast<size_t>(b) * a.ldq + h * DH + tid]) * a.scale;
     const __nv_bfloat16 vnew = a.vt[static_cast<size_t>(h * DH + tid) * a.t_pad + b];
@@ -251,12 +269,15 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(DecAttnArgs
 #pragma unroll
   for (int i = 0; i < PER; ++i) r.o[i] = 0.f;
   for (int p0 = p_begin; p0 < p_end; p0 += 32) {
-    if (p0 > p_begin) request(p0);
     cp_async_wait<0>();
     __syncwarp();
     const bool in = p0 + lane < p_end;
-    const float sc = tile_score<DH>(ktile, sq, lane);
-    const float e = fold_scores<PER>(r, in ? sc : -INFINITY, in);
+    float sc;
+    tile_scores<DH, 1>(ktile, 0, sq, lane, &sc);
+    __syncwarp();  // the tile is read before it is filled again
+    if (p0 + 32 < p_end) request_k(p0 + 32);  // lands while this tile is folded
+    if (!in) sc = -INFINITY;
+    const float e = fold_scores<PER>(r, sc, warp_max(sc), in);
     fold_rows<PER>(r, e, min(p_end, len) - p0, [&](int j) { return vv[j]; });
     if (len >= p0 && len < p0 + 32 && len < p_end) {  // the new token, last of the last run
       const float en = __shfl_sync(0xffffffffu, e, len - p0);
@@ -269,7 +290,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(DecAttnArgs
         r.o[3] = fmaf(en, v1.y, r.o[3]);
       }
     }
-    __syncwarp();  // the tile is read before it is filled again
+    if (p0 + 32 < p_end) request_v(p0 + 32);
   }
   if (lane == 0) {
     sm_m[warp] = r.m;
@@ -292,14 +313,14 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(DecAttnArgs
   }
 }
 
-constexpr int kGqaRing = 5;  // tiles in flight per run (16 KB each at d_head 128)
+constexpr int kGqaTiles = 4;  // tiles per step (16 KB each at d_head 128); two steps in shared memory
 
 // Several query heads per KV head: cluster of kRuns blocks, block = run, warp
 // = query head; blockIdx.y = KV head times passes of kRuns query heads.
 template <int DH>
-__global__ void __launch_bounds__(kDecThreads) decode_attn_gqa_kernel(DecAttnArgs a) {
+__global__ void __launch_bounds__(kDecThreads, 1) decode_attn_gqa_kernel(DecAttnArgs a) {
   constexpr int PER = DH / 32, CH = DH / 8, TB = 32 * DH * 2;
-  extern __shared__ __align__(128) uint8_t dec_smem[];  // kGqaRing tiles of 32 K rows and 32 V rows
+  extern __shared__ __align__(128) uint8_t dec_smem[];  // [2][kGqaTiles] of 32 K rows and 32 V rows
   __shared__ __align__(16) float sq[kRuns][DH];
   __shared__ float sm_m[kRuns], sm_l[kRuns];  // per query head, read by the cluster
   __shared__ float sm_o[kRuns][DH];
@@ -322,22 +343,23 @@ __global__ void __launch_bounds__(kDecThreads) decode_attn_gqa_kernel(DecAttnArg
   const size_t cbase = static_cast<size_t>(b) * a.max_len * a.dkv + static_cast<size_t>(kvh) * DH;
   const int n = len + 1, per_run = (n + kRuns - 1) / kRuns;
   const int p_begin = run * per_run, p_end = min(n, p_begin + per_run);
-  auto request = [&](int p0, int buf) {
-    uint8_t *kt = dec_smem + buf * 2 * TB, *vt = kt + TB;
-    for (int idx = tid; idx < 32 * CH; idx += kDecThreads) {
+  auto request = [&](int p0, int buf) {  // the tiles of one step into half `buf` of the ring
+    uint8_t* tiles = dec_smem + buf * kGqaTiles * 2 * TB;
+    for (int idx = tid; idx < 32 * kGqaTiles * CH; idx += kDecThreads) {
       const int row = idx / CH, c = idx % CH, p = p0 + row;
-      if (p < p_end) {
-        const size_t at = cbase + static_cast<size_t>(p) * a.dkv + c * 8;
-        cp_async16(kt + row * DH * 2 + ((c ^ (row & 7)) << 4), p < len ? a.k_cache + at : knew + c * 8);
-        if (p < len) cp_async16(vt + row * DH * 2 + c * 16, a.v_cache + at);
-      }
+      if (p >= p_end) break;  // rows only grow
+      uint8_t* kt = tiles + (row >> 5) * 2 * TB + (row & 31) * DH * 2;
+      const size_t at = cbase + static_cast<size_t>(p) * a.dkv + c * 8;
+      cp_async16(kt + ((c ^ (row & 7)) << 4), p < len ? a.k_cache + at : knew + c * 8);
+      if (p < len) cp_async16(kt + TB + c * 16, a.v_cache + at);
     }
     cp_async_commit();
     const int jn = len - p0;  // the new token's V row (transposed in this step's V^T)
-    if (jn >= 0 && jn < 32 && len < p_end && tid < DH)
-      reinterpret_cast<__nv_bfloat16*>(vt)[jn * DH + tid] = vnew[static_cast<size_t>(tid) * a.t_pad];
+    if (jn >= 0 && jn < 32 * kGqaTiles && len < p_end && tid < DH)
+      reinterpret_cast<__nv_bfloat16*>(tiles + (jn >> 5) * 2 * TB + TB)[(jn & 31) * DH + tid] =
+          vnew[static_cast<size_t>(tid) * a.t_pad];
   };
-  for (int i = 0; i < kGqaRing - 1; ++i) request(p_begin + 32 * i, i);
+  request(p_begin, 0);
   for (int i = tid; i < nh * DH; i += kDecThreads)
     sq[i / DH][i % DH] = __bfloat162float(a.q[static_cast<size_t>(b) * a.ldq + h0 * DH + i]) * a.scale;
   if (run == 0 && h0 == kvh * grp && tid < DH) {  // append the new key and value to the cache
@@ -349,18 +371,29 @@ __global__ void __launch_bounds__(kDecThreads) decode_attn_gqa_kernel(DecAttnArg
 #pragma unroll
   for (int i = 0; i < PER; ++i) r.o[i] = 0.f;
   int buf = 0;
-  for (int p0 = p_begin; p0 < p_end; p0 += 32) {
-    cp_async_wait<kGqaRing - 2>();
-    __syncthreads();  // this tile has landed, and the previous one is read
-    request(p0 + 32 * (kGqaRing - 1), buf == 0 ? kGqaRing - 1 : buf - 1);
+  for (int p0 = p_begin; p0 < p_end; p0 += 32 * kGqaTiles) {
+    cp_async_wait<0>();
+    __syncthreads();  // this step's tiles have landed, and the previous step's are read
+    request(p0 + 32 * kGqaTiles, buf ^ 1);
     if (warp < nh) {
-      const bool in = p0 + lane < p_end;
-      const uint8_t* kt = dec_smem + buf * 2 * TB;
-      const float e = fold_scores<PER>(r, in ? tile_score<DH>(kt, sq[warp], lane) : -INFINITY, in);
-      const uint8_t* vrows = kt + TB + lane * PER * 2;
-      fold_rows<PER>(r, e, min(32, p_end - p0), [&](int j) { return row_part<PER>(vrows + j * DH * 2); });
+      const uint8_t* kt = dec_smem + buf * kGqaTiles * 2 * TB;
+      float sc[kGqaTiles], mx[kGqaTiles];
+      tile_scores<DH, kGqaTiles>(kt, 2 * TB, sq[warp], lane, sc);
+#pragma unroll
+      for (int t = 0; t < kGqaTiles; ++t) {
+        if (p0 + 32 * t + lane >= p_end) sc[t] = -INFINITY;
+        mx[t] = warp_max(sc[t]);
+      }
+#pragma unroll
+      for (int t = 0; t < kGqaTiles; ++t) {
+        const int n = p_end - (p0 + 32 * t);
+        if (n <= 0) break;
+        const float e = fold_scores<PER>(r, sc[t], mx[t], lane < n);
+        const uint8_t* vrows = kt + t * 2 * TB + TB + lane * PER * 2;
+        fold_rows<PER>(r, e, min(32, n), [&](int j) { return row_part<PER>(vrows + j * DH * 2); });
+      }
     }
-    if (++buf == kGqaRing) buf = 0;
+    buf ^= 1;
   }
   cp_async_wait<0>();
   if (warp < nh) {
@@ -399,7 +432,7 @@ template <int DH>
 static cudaError_t launch_dec(const DecAttnArgs& a, cudaStream_t s) {
   const int grp = a.A / a.Akv;
   if (grp > 1) {
-    constexpr int ring = kGqaRing * 2 * 32 * DH * 2;
+    constexpr int ring = 2 * kGqaTiles * 2 * 32 * DH * 2;
     const cudaError_t e =
         cudaFuncSetAttribute(decode_attn_gqa_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, ring);
     if (e != cudaSuccess) return e;

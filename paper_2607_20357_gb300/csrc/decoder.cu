@@ -259,7 +259,7 @@ __device__ void build_list(const ScheduleArgs& a, int l, int kind, int* dyn) {
       int j1 = j0;
       while (j1 + 1 < G && !((neq >> j1) & 1)) ++j1;
       ColSet cs{};
-      cs.step = qkv ? 256 : 128;
+      cs.step = qkv ? a.qkv_step : 128;
       if (qkv) {
         cs.set(0, j0 * hq, (j1 + 1) * hq);
         cs.set(1, j0 * hk, (j1 + 1) * hk);

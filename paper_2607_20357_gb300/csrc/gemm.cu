@@ -105,40 +105,35 @@ SVL_DEVINL void k_share(const TileInfo& ti, int nkb, int kgb, int& i0, int& i1) 
   i1 = (n * (ti.part + 1)) / ti.nsplit;
 }
 
-// Walks the K blocks of a tile, skipping the blocks of gated-off groups
-// (kmask bit j clear: K blocks [j*kgb, (j+1)*kgb) are not visited). The group
-// index is kept incrementally: no division in the issue loops.
+// Walks the active K blocks of a tile from its n-th on (gated-off groups
+// skipped: kmask bit j clear means K blocks [j*kgb, (j+1)*kgb) are not visited).
+// The start is computed, not stepped to: stepping took 0.1 us a block, 8 us for
+// the last of eight shares of an 11,008-deep product. A step is an increment
+// and a count-down to the end of the group.
 struct KWalk {
-  int kb, grp, kin;
-  const int nkb, kgb, kmask;
-  SVL_DEVINL KWalk(int nkb_, int kgb_, int kmask_) : kb(-1), grp(0), kin(-1), nkb(nkb_), kgb(kgb_), kmask(kmask_) {}
-  // Moves to the n-th active block (n >= 1), as n calls of next() would. The
-  // shares of a K-split tile start here: stepping took 0.1 us a block, 8 us
-  // for the last of eight shares of an 11,008-deep product.
-  SVL_DEVINL void skip(int n) {
-    if (n <= 0) return;
-    const int g = (n - 1) / kgb, r = (n - 1) - g * kgb;
+  int kb, left;  // this block; blocks to the end of its group, this one included
+  int rest;      // mask of the active groups after this one
+  int kgb;
+  SVL_DEVINL KWalk(int kgb_, int kmask, int n) : kgb(kgb_) {
     if (kmask == 0) {
-      kb = n - 1;
-      grp = g;
-    } else {
-      int m = kmask;
-      for (int i = 0; i < g; ++i) m &= m - 1;  // drop the g lowest active groups
-      grp = __ffs(m) - 1;
-      kb = grp * kgb + r;
+      kb = n;
+      left = 0x7fffffff;
+      rest = 0;
+      return;
     }
-    kin = r;
+    const int g = n / kgb, r = n - g * kgb;
+    for (int i = 0; i < g; ++i) kmask &= kmask - 1;  // drop the g lowest active groups
+    kb = (__ffs(kmask) - 1) * kgb + r;
+    left = kgb - r;
+    rest = kmask & (kmask - 1);
   }
-  // advances to the next active K block; false when the tile is done
-  SVL_DEVINL bool next() {
-    while (true) {
-      ++kb;
-      if (kb >= nkb) return false;
-      if (++kin == kgb) {
-        kin = 0;
-        ++grp;
-      }
-      if (kmask == 0 || ((kmask >> grp) & 1)) return true;
+  // the next active block (there must be one)
+  SVL_DEVINL void next() {
+    ++kb;
+    if (--left == 0) {
+      kb = (__ffs(rest) - 1) * kgb;
+      left = kgb;
+      rest &= rest - 1;
     }
   }
 };
@@ -167,6 +162,16 @@ struct StageCfg<KIND, true> {
   static constexpr int stages = 6;
   static constexpr int abytes = kThinRows * 128;
   static constexpr int bytes = abytes + 2 * kBHalfBytes;
+};
+// QKV of a THIN launch: 128-column tiles (see ScheduleArgs::qkv_step), so a
+// stage is 20 KB and ten of them fit. With 256 columns in the list and 36 KB
+// stages the tail's halves left 120 KB in flight per SM: 100 MB of weights in
+// 24 us (96 SMs), 33 MB in 24 us (36 SMs).
+template <>
+struct StageCfg<EPI_QKV_ROPE, true> {
+  static constexpr int stages = 10;
+  static constexpr int abytes = kThinRows * 128;
+  static constexpr int bytes = abytes + kBHalfBytes;
 };
 // LM head of at most kThinRows samples: a stage is 16 KB of weights (A) and
 // the samples' rows in a box of kThinRows, so ten stages keep 160 KB of
@@ -219,18 +224,17 @@ SVL_DEVINL void producer_loop(const GemmParams& p, uint8_t* stages, uint64_t* fu
   for (int t = blockIdx.x; t < wk.n; t += gridDim.x) {
     const TileInfo ti = get_tile(p, wk, t, gridDim.x);
     if (!ti.valid) continue;
-    const int halves = p.b_split ? 2 : (ti.ncols > kBHalf ? 2 : 1);
+    const bool two = p.b_split || ti.ncols > kBHalf;
     const CUtensorMap* mb0 = p.b_split ? &p.mapB[0] : &p.mapB[ti.mat];
     const CUtensorMap* mb1 = p.b_split ? &p.mapB[1] : &p.mapB[ti.mat];
     const int y1 = p.b_split ? ti.n0 : ti.n0 + kBHalf;
-    const uint32_t bytes = OP == 0 ? ABYTES : halves * (p.b_box_rows ? p.b_box_rows * 128 : kBHalfBytes);
-    KWalk w(nkb, kgb, ti.kmask);
+    const uint32_t bytes = OP == 0 ? ABYTES : (two ? 2 : 1) * (p.b_box_rows ? p.b_box_rows * 128 : kBHalfBytes);
     int i0, i1;
     k_share(ti, nkb, kgb, i0, i1);
-    w.skip(i0);
-    w.next();
-    for (int i = i0; i < i1; ++i) {
+    KWalk w(kgb, ti.kmask, i0);
+    for (int n = i1 - i0; n > 0; --n) {
       uint8_t* dst = stages + s * SBYTES + (OP == 0 ? 0 : ABYTES);
+      const int x = w.kb * BK;
       if (!mbar_wait(&empty[s], ph, abort)) {
         set_abort(abort, p.status);
         return;
@@ -238,12 +242,12 @@ SVL_DEVINL void producer_loop(const GemmParams& p, uint8_t* stages, uint64_t* fu
       mbar_arrive_expect_tx(&full[s], bytes);
       if constexpr (OP == 0) {
         if (p.a_evict_first)
-          tma_load_2d_hint(dst, &p.mapA, &full[s], w.kb * BK, ti.m0, pol);
+          tma_load_2d_hint(dst, &p.mapA, &full[s], x, ti.m0, pol);
         else
-          tma_load_2d(dst, &p.mapA, &full[s], w.kb * BK, ti.m0);
+          tma_load_2d(dst, &p.mapA, &full[s], x, ti.m0);
       } else {
-        tma_load_2d(dst, mb0, &full[s], w.kb * BK, ti.n0);
-        if (halves == 2) tma_load_2d(dst + kBHalfBytes, mb1, &full[s], w.kb * BK, y1);
+        tma_load_2d(dst, mb0, &full[s], x, ti.n0);
+        if (two) tma_load_2d(dst + kBHalfBytes, mb1, &full[s], x, y1);
       }
       w.next();
       if (++s == NST) {
@@ -261,6 +265,8 @@ SVL_DEVINL void mma_loop(const GemmParams& p, uint8_t* stages, uint64_t* full, u
   constexpr int BK = F8 ? kBK8 : kBK;
   Work wk = load_work(p, blockIdx.x);
   const int nkb = p.K / BK, kgb = p.kgroup / BK;
+  // descriptors of stage 0; stage s and K step k are (s * SBYTES + 32 k) / 16 further
+  const uint64_t da0 = smem_desc_sw128(smem_u32(stages)), db0 = smem_desc_sw128(smem_u32(stages) + ABYTES);
   int s = 0, it = 0;
   uint32_t ph = 0;
   for (int t = blockIdx.x; t < wk.n; t += gridDim.x) {
@@ -273,27 +279,26 @@ SVL_DEVINL void mma_loop(const GemmParams& p, uint8_t* stages, uint64_t* full, u
       return;
     }
     tc_fence_after();
-    const int n = p.b_split ? 2 * kBHalf : ((ti.ncols + 15) & ~15);
-    const uint32_t idesc = F8 ? idesc_e4m3_f32(kBM, n) : idesc_bf16_f32(kBM, n);
+    const int ncols = p.b_split ? 2 * kBHalf : ((ti.ncols + 15) & ~15);
+    const uint32_t idesc = F8 ? idesc_e4m3_f32(kBM, ncols) : idesc_bf16_f32(kBM, ncols);
     const uint32_t d = tmem + acc * kAccCols;
     uint32_t accumulate = 0;
     int i0, i1;
     k_share(ti, nkb, kgb, i0, i1);
-    for (int i = i0; i < i1; ++i) {
+    for (int n = i1 - i0; n > 0; --n) {
+      const uint64_t da = da0 + static_cast<uint32_t>(s * (SBYTES / 16)), db = db0 + static_cast<uint32_t>(s * (SBYTES / 16));
       if (!mbar_wait(&full[s], ph, abort)) {
         set_abort(abort, p.status);
         return;
       }
       tc_fence_after();
-      const uint32_t a0 = smem_u32(stages + s * SBYTES);
-      const uint32_t b0 = a0 + ABYTES;
       // four instructions per stage, each over the next 32 bytes of K
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         if constexpr (F8)
-          tc_mma_e4m3(d, smem_desc_sw128(a0 + k * 32), smem_desc_sw128(b0 + k * 32), idesc, accumulate);
+          tc_mma_e4m3(d, da + 2 * k, db + 2 * k, idesc, accumulate);
         else
-          tc_mma_bf16(d, smem_desc_sw128(a0 + k * 32), smem_desc_sw128(b0 + k * 32), idesc, accumulate);
+          tc_mma_bf16(d, da + 2 * k, db + 2 * k, idesc, accumulate);
         accumulate = 1;
       }
       tc_commit(&empty[s]);
@@ -1154,7 +1159,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
   uint8_t* rstage = stages + NST * SBYTES + 1024;
   static_assert(2 * NST + (kStaged ? 16 : 8) <= 31, "barriers");
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);  // uniform over the warp
   if (threadIdx.x == 0) {
     for (int i = 0; i < NST; ++i) {
       mbar_init(&full[i], 2);  // the A and the B producer
@@ -1194,11 +1199,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
   }
 
   if (warp == 0) {
-    if (lane == 0) producer_loop<1, NST, SBYTES, ABYTES, F8>(p, stages, full, empty, abort);
+    if (elect_one()) producer_loop<1, NST, SBYTES, ABYTES, F8>(p, stages, full, empty, abort);
   } else if (warp == 6) {
-    if (lane == 0) producer_loop<0, NST, SBYTES, ABYTES, F8>(p, stages, full, empty, abort);
+    if (elect_one()) producer_loop<0, NST, SBYTES, ABYTES, F8>(p, stages, full, empty, abort);
   } else if (warp == 1) {
-    if (lane == 0) mma_loop<NST, SBYTES, ABYTES, F8>(p, stages, full, empty, tfull, tempty, tmem, abort);
+    if (elect_one()) mma_loop<NST, SBYTES, ABYTES, F8>(p, stages, full, empty, tfull, tempty, tmem, abort);
   } else {
     epilogue_loop<KIND, F8, THIN>(p, tfull, tempty, tmem, abort, ks, rstage, rbar, stages);
   }
@@ -1275,8 +1280,10 @@ SVL_DEVINL void pair_producer(const GemmParams& p, uint8_t* stages, uint64_t* fu
     const CUtensorMap* mb = p.b_split ? &p.mapB[rank] : &p.mapB[ti.mat];
     const int by = p.b_split ? ti.n0 : ti.n0 + static_cast<int>(rank) * brows;
     const uint32_t bytes = 2u * static_cast<uint32_t>(kABytes + brows * 128);
-    KWalk w(nkb, kgb, ti.kmask);
-    while (w.next()) {
+    int i0, i1;
+    k_share(ti, nkb, kgb, i0, i1);
+    KWalk w(kgb, ti.kmask, i0);
+    for (int n = i1 - i0; n > 0; --n, w.next()) {
       if (!mbar_wait(&empty[s], ph ^ 1, abort)) {
         set_abort(abort, p.status);
         return;
@@ -1320,8 +1327,9 @@ SVL_DEVINL void pair_mma(const GemmParams& p, uint8_t* stages, uint64_t* full, u
     const uint32_t idesc = idesc_bf16_f32(2 * kBM, pair_n(p, ti));
     const uint32_t d = tmem + acc * kAccCols;
     uint32_t accumulate = 0;
-    KWalk w(nkb, kgb, ti.kmask);
-    while (w.next()) {
+    int i0, i1;
+    k_share(ti, nkb, kgb, i0, i1);
+    for (int n = i1 - i0; n > 0; --n) {
       if (!mbar_wait(&full[s], ph, abort)) {
         set_abort(abort, p.status);
         return;

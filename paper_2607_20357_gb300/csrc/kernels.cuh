@@ -195,6 +195,7 @@ struct ScheduleArgs {
   int B, L, G, P;
   int num_sms;              // CTAs of the persistent GEMM (one wave of tiles)
   int nsparse_rows;         // rows per tile of the QKV and gate/up lists (128, or 256 for CTA pairs)
+  int qkv_step;             // columns per QKV tile (256; 128 for THIN launches)
   int nsparse_wave;         // tiles of those lists that run at once (CTAs, or CTA pairs)
   int mband;                // m-tiles per raster band of those lists (see kMBandBytes)
   int A, Akv, dh, D, Di;
