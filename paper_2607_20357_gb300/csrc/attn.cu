@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) attn_tc_kernel(const __grid_c
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2);
   volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // warp: uniform
   if (threadIdx.x == 0) {
     for (int sl = 0; sl < 2; ++sl) {
       PipeBars* b = bars + sl;
@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) attn_tc_kernel(const __grid_c
 
   if (role == 0) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       int g = 0, nq = 0;
       bool ok = true;
       // passes unit u (-1: none left) and its item to the MMA and softmax
@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) attn_tc_kernel(const __grid_c
     }
   } else if (role == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t id_s = idesc_bf16_f32(128, kPipeKeys), id_o = idesc_bf16_f32(128, DH);
       int g = 0, nq = 0, t = 0;  // ring position, units, tiles so far
       bool ok = true;
