@@ -22,6 +22,9 @@ constexpr int kNBandO = 16;       // O list (16 n-tiles of 256 x 4,096 weights: 
 // reads everything once. 100 MB of rows in one band no longer stay in L2
 // (4.2 GB).
 constexpr long long kMBandBytes = 40ll << 20;
+constexpr int kAttnSorted = 64;                    // samples up to which attention items may be ordered by size ...
+constexpr int kAttnLong = 768;                     // ... which they are when one has more rows than this
+constexpr long long kAttnChunkBytes = 40ll << 20;  // keys and values of the samples ordered together
 constexpr int kBM_SCHED = 128;    // tile rows (the GEMM's M)
 
 struct SelectArgs {
