@@ -31,6 +31,7 @@ struct Work {
   int n;             // tiles
   int ks0, kr, ks;   // K-split tail: first copy, tail tiles, shares (see GemmParams)
   int mlim, gm;      // dense grid: rows and row tiles (those that exist, so that the CTAs share them evenly)
+  int whole;         // dense grid: tiles before the last wave's halves (see load_work)
   int4 next;         // the list entry of the CTA's next tile, fetched one ahead
 };
 
@@ -58,7 +59,14 @@ SVL_DEVINL Work load_work(const GemmParams& p, int first) {
   } else {
     if (p.m_limit_dev) w.mlim = min(w.mlim, __ldcg(p.m_limit_dev));
     w.gm = max((w.mlim + kBM - 1) / kBM, 1);
-    w.n = w.gm * p.grid_n;
+    w.whole = w.n = w.gm * p.grid_n;
+    // a last wave of 256-column tiles that is at most half full is cut into
+    // 128-column halves, which fit in one wave and take half the time
+    const int r = w.n % gridDim.x;
+    if (p.bn == 2 * kBHalf && 2 * r <= static_cast<int>(gridDim.x)) {
+      w.whole -= r;
+      w.n += r;
+    }
   }
   return w;
 }
@@ -77,11 +85,13 @@ SVL_DEVINL TileInfo get_tile(const GemmParams& p, Work& w, int t, int step) {
     ti.kmask = tile_kmask(v.w);
     ti.valid = ti.ncols > 0 && ti.m_end > ti.m0 && ti.mat < 3;
   } else {
-    const int ni = t / w.gm, mi = t - ni * w.gm;
+    const int half = t - w.whole;  // >= 0: half tile
+    const int u = half < 0 ? t : w.whole + (half >> 1);
+    const int ni = u / w.gm, mi = u - ni * w.gm;
     ti.m0 = mi * kBM;
     ti.m_end = min(ti.m0 + kBM, w.mlim);
-    ti.n0 = ni * p.bn;
-    ti.ncols = min(p.bn, p.n_limit - ti.n0);
+    ti.n0 = ni * p.bn + (half >= 0 && (half & 1) ? kBHalf : 0);
+    ti.ncols = min(half < 0 ? p.bn : kBHalf, p.n_limit - ti.n0);
     ti.mat = 0;
     ti.kmask = 0;
     ti.valid = ti.m0 < w.mlim && ti.ncols > 0;
