@@ -141,19 +141,23 @@ SVL_DEVINL uint32_t order_key(float z) {
 // read once, into shared memory while they fit (kKeysShared).
 constexpr int kKeysShared = 4096;
 
-__device__ void top_k(const float* z, int n, int k, int* out, uint32_t* skeys) {
+SVL_DEVINL void load_keys(const float* z, int n, uint32_t* skeys) {
+  if (n <= kKeysShared)
+    for (int i = threadIdx.x; i < n; i += blockDim.x) skeys[i] = order_key(z[i]);
+}
+
+// (skeys: load_keys of the same logits)
+__device__ void top_k(const float* z, int n, int k, int* out, const uint32_t* skeys) {
   __shared__ int hist[256];
   __shared__ int warp_sums[32];
-  __shared__ int s_prefix_cnt[2];
-  const int tid = threadIdx.x;
+  __shared__ int s_prefix_cnt[3];
+  const int tid = threadIdx.x, lane = tid & 31;
   if (k == 0) return;
   if (k >= n) {
     for (int i = tid; i < n; i += blockDim.x) out[i] = i;
     return;
   }
   const bool shared = n <= kKeysShared;
-  if (shared)
-    for (int i = tid; i < n; i += blockDim.x) skeys[i] = order_key(z[i]);
   auto key_at = [&](int i) -> uint32_t { return shared ? skeys[i] : order_key(z[i]); };
 
   // ---- radix select of the k-th largest key, 8 bits per pass, MSB first
@@ -162,9 +166,15 @@ __device__ void top_k(const float* z, int n, int k, int* out, uint32_t* skeys) {
   for (int shift = 24; shift >= 0; shift -= 8) {
     for (int i = tid; i < 256; i += blockDim.x) hist[i] = 0;
     __syncthreads();
-    for (int i = tid; i < n; i += blockDim.x) {
-      const uint32_t key = key_at(i);
-      if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 0xFF], 1);
+    // logits share their leading digits: the lanes of a warp with the same one
+    // count together (32 atomics on one address made a pass 2 us)
+    for (int base = 0; base < n; base += blockDim.x) {
+      const int i = base + tid;
+      const uint32_t key = i < n ? key_at(i) : 0;
+      const bool in = i < n && (key & mask) == prefix;
+      const int digit = in ? static_cast<int>((key >> shift) & 0xFF) : -1;
+      const unsigned same = __match_any_sync(0xffffffffu, digit);
+      if (in && lane == __ffs(same) - 1) atomicAdd(&hist[digit], __popc(same));
     }
     __syncthreads();
     if (tid < 32) {
@@ -199,15 +209,17 @@ __device__ void top_k(const float* z, int n, int k, int* out, uint32_t* skeys) {
       if (tid == 0) {
         s_prefix_cnt[0] = d < 0 ? 0 : d;
         s_prefix_cnt[1] = remaining - (d < 0 ? 0 : ab);
+        s_prefix_cnt[2] = hist[d < 0 ? 0 : d];
       }
     }
     __syncthreads();
     prefix |= static_cast<uint32_t>(s_prefix_cnt[0]) << shift;
     mask |= 0xFFu << shift;
     remaining = s_prefix_cnt[1];
+    if (s_prefix_cnt[2] == remaining) break;  // every key with this prefix is kept: lower digits do not matter
   }
-  const uint32_t tau = prefix;  // key of the k-th largest logit
-  // keys > tau are kept; of the keys == tau, the `remaining` lowest indices
+  const uint32_t tau = prefix;  // the digits read so far of the k-th largest key
+  // keys > tau (in these digits) are kept; of the keys == tau, the `remaining` lowest indices
 
   // ---- ordered pass: per chunk the ranks of equal keys and the output
   // positions by index from one scan of both counts (16 bits each: a chunk has
@@ -215,7 +227,7 @@ __device__ void top_k(const float* z, int n, int k, int* out, uint32_t* skeys) {
   int eq_before = 0, kept_before = 0;
   for (int base = 0; base < n; base += blockDim.x) {
     const int i = base + tid;
-    const uint32_t key = i < n ? key_at(i) : 0;
+    const uint32_t key = i < n ? key_at(i) & mask : 0;
     const int gt = (i < n && key > tau) ? 1 : 0, eq = (i < n && key == tau) ? 1 : 0;
     int total;
     const int ex = block_exclusive_scan(gt | (eq << 16), &total, warp_sums);
@@ -238,9 +250,10 @@ __global__ void __launch_bounds__(kSelectThreads) topk_kernel(int B, const float
   pdl_begin(false);
   const int b = blockIdx.x, tid = threadIdx.x, v0 = vis_off[b], n = max(0, vis_off[b + 1] - v0), kb = k[b];
   if (tid == 0) off = 0;
-  __syncthreads();
   int part = 0;
   for (int i = tid; i < b; i += kSelectThreads) part += k[i];
+  load_keys(scores + v0, n, topk_keys);
+  __syncthreads();
   part = __reduce_add_sync(0xffffffffu, part);
   if ((tid & 31) == 0 && part) atomicAdd(&off, part);
   __syncthreads();
@@ -384,6 +397,7 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectArgs a) {
     if (a.flags) a.flags[b] = flags;
   }
 
+  load_keys(a.scores + v0, n, topk_keys);
   top_k(a.scores + v0, n, k, a.kept_local + v0, topk_keys);
 }
 
