@@ -703,41 +703,62 @@ SVL_DEVINL void ksplit_rows(const GemmParams& p, const TileInfo& ti, uint8_t* ri
 #pragma unroll
       for (int i = 0; i < 8; ++i) cs[i] = __ldg(p.b_scale[0] + ti.n0 + c + i);
     }
-#pragma unroll 2
-    for (int r = a0; r < a1; ++r) {
-      uint4* xr = reinterpret_cast<uint4*>(ring + kKsResid + r * 512 + c * 2);
-      const int sw = (r0 + r) & 7, u0 = (c >> 2) & 7;
-      const uint8_t* src = ring + static_cast<size_t>(r) * (kAccCols * 4) + (c >> 5) * 128;
-      float v[8];
+    // four rows at a time: a row alone exposed its reads' latency (600 cycles)
+    const int u0 = (c >> 2) & 7;
+    const size_t pitch = static_cast<size_t>(n) * (kAccCols * 4);  // from share to share
+    for (int rb = a0; rb < a1; rb += 4) {
+      float v[4][8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = 0.f;
-      for (int q = 0; q < ti.nsplit; ++q, src += static_cast<size_t>(n) * (kAccCols * 4)) {
-        const float4 f = *reinterpret_cast<const float4*>(src + ((u0 ^ sw) << 4));
-        const float4 g = *reinterpret_cast<const float4*>(src + (((u0 + 1) ^ sw) << 4));
-        v[0] += f.x;
-        v[1] += f.y;
-        v[2] += f.z;
-        v[3] += f.w;
-        v[4] += g.x;
-        v[5] += g.y;
-        v[6] += g.z;
-        v[7] += g.w;
-      }
-      if constexpr (F8) {
-        const float rs = p.a_scale[ti.m0 + r0 + r];
+      for (int k = 0; k < 4; ++k)
 #pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] *= rs * cs[i];
-      }
-      const uint4 x = *xr;
-      const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
-      uint32_t o[4];
+        for (int i = 0; i < 8; ++i) v[k][i] = 0.f;
+      const uint8_t* src = ring + static_cast<size_t>(rb) * (kAccCols * 4) + (c >> 5) * 128;
+      for (int q = 0; q < ti.nsplit; ++q, src += pitch) {
+        float4 f[4], g[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float2 f = unpack_bf16x2(xw[i]);
-        o[i] = pack_bf16x2(v[2 * i] + f.x, v[2 * i + 1] + f.y);
+        for (int k = 0; k < 4; ++k) {
+          if (rb + k < a1) {
+            const int sw = (r0 + rb + k) & 7;
+            f[k] = *reinterpret_cast<const float4*>(src + k * (kAccCols * 4) + ((u0 ^ sw) << 4));
+            g[k] = *reinterpret_cast<const float4*>(src + k * (kAccCols * 4) + (((u0 + 1) ^ sw) << 4));
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          v[k][0] += f[k].x;
+          v[k][1] += f[k].y;
+          v[k][2] += f[k].z;
+          v[k][3] += f[k].w;
+          v[k][4] += g[k].x;
+          v[k][5] += g[k].y;
+          v[k][6] += g[k].z;
+          v[k][7] += g[k].w;
+        }
       }
-      *xr = make_uint4(o[0], o[1], o[2], o[3]);
-      *reinterpret_cast<uint4*>(X + static_cast<size_t>(r) * p.ld[0] + c) = make_uint4(o[0], o[1], o[2], o[3]);
+      uint4 x[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (rb + k < a1) x[k] = *reinterpret_cast<const uint4*>(ring + kKsResid + (rb + k) * 512 + c * 2);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int r = rb + k;
+        if (r >= a1) break;
+        if constexpr (F8) {
+          const float rs = p.a_scale[ti.m0 + r0 + r];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) v[k][i] *= rs * cs[i];
+        }
+        const uint32_t xw[4] = {x[k].x, x[k].y, x[k].z, x[k].w};
+        uint32_t o[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float2 e = unpack_bf16x2(xw[i]);
+          o[i] = pack_bf16x2(v[k][2 * i] + e.x, v[k][2 * i + 1] + e.y);
+        }
+        const uint4 ov = make_uint4(o[0], o[1], o[2], o[3]);
+        *reinterpret_cast<uint4*>(ring + kKsResid + r * 512 + c * 2) = ov;
+        *reinterpret_cast<uint4*>(X + static_cast<size_t>(r) * p.ld[0] + c) = ov;
+      }
     }
   }
   if (!p.ss_out) return;
