@@ -25,8 +25,9 @@ struct svl_model {
   bool ks_resident = false;
   // QKV and gate/up on CTA pairs (256-row tiles, tcgen05 cta_group::2):
   // clusters of two resident at once (0: single-CTA kernel); per layer the
-  // q, k, v, g, u weights as tensor maps with 64-row boxes
+  // q, k, v weights as tensor maps with 64-row boxes
   int pair_clusters = 0;
+  int pair_rows = 0;  // rows from which batches use them
   std::vector<CUtensorMap> tm_pair;
   uint32_t* d_status = nullptr;
   float2* rope_cs = nullptr;
@@ -107,6 +108,13 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 int round128(int x) { return (x + 127) & ~127; }
 
 constexpr int kMaxPrefillBatch = 4096;  // samples per prefill call
+
+// Row capacity from which the QKV and gate/up GEMMs run on CTA pairs. Their 256-row
+// tiles move a third less per MMA; with fewer rows, and with runs of gated samples
+// that end inside a tile, more of a tile is padding. Measured over one layer's MLP
+// and QKV + O at LLaVA-7B and Qwen2-VL-7B widths, all groups on and mixed masks: 4 to
+// 10 % faster at 3,072 rows and more, -2 to +6 % at 1,024 to 2,048, -4 % (MLP) at 320.
+constexpr int kPairRows = 3072;
 
 // Each call keeps its scratch at the start of the workspace: no data flows
 // between calls through the workspace, so the three layouts overlap and the
@@ -507,26 +515,24 @@ svl_status svl_model_create(const svl_model_desc* desc, const svl_weights* w, sv
     svl_model_destroy(m);
     return SVL_ERR_INVALID_ARG;
   }
-  // CTA-pair QKV and gate/up GEMMs for bf16 models, chosen with
-  // SVL_PAIR_GEMM=1 in the environment at model creation. They move a third
-  // less data through shared memory and L2 per FLOP but run at the same speed
-  // as the single-CTA kernel on GB300, whose GEMMs are held by the power cap,
-  // so the single-CTA kernel stays the default.
+  // CTA-pair QKV and gate/up GEMMs for bf16 models: from kPairRows rows on, or
+  // as SVL_PAIR_GEMM in the environment at model creation says (1: for every
+  // batch but decode-sized ones, 0: never).
   if (ok && !m->e4m3) {
     const char* env = std::getenv("SVL_PAIR_GEMM");
-    if (env && env[0] == '1') {
+    m->pair_rows = env && env[0] == '1' ? 0 : kPairRows;
+    if (!env || env[0] != '0') {
       const int c = std::min(gemm_pair_max_clusters(EPI_QKV_ROPE), gemm_pair_max_clusters(EPI_SWIGLU));
       m->pair_clusters = std::min(c, m->num_sms / 2);
     }
     cudaGetLastError();  // a failed occupancy query only disables the pair kernel
     if (m->pair_clusters > 0) {
-      m->tm_pair.resize(static_cast<size_t>(d.n_layers) * 5);
+      m->tm_pair.resize(static_cast<size_t>(d.n_layers) * 3);
       for (int l = 0; l < d.n_layers && ok; ++l) {
         const svl_layer_weights& lw = m->layers[l];
-        CUtensorMap* t = &m->tm_pair[static_cast<size_t>(l) * 5];
+        CUtensorMap* t = &m->tm_pair[static_cast<size_t>(l) * 3];
         ok = make_map(t + 0, lw.wq, hq, d.d_model, 64) && make_map(t + 1, lw.wk, dkv, d.d_model, 64) &&
-             make_map(t + 2, lw.wv, dkv, d.d_model, 64) && make_map(t + 3, lw.wg, d.d_ffn, d.d_model, 64) &&
-             make_map(t + 4, lw.wu, d.d_ffn, d.d_model, 64);
+             make_map(t + 2, lw.wv, dkv, d.d_model, 64);
       }
       if (!ok) {
         svl_model_destroy(m);
@@ -900,7 +906,7 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
   sa.P = d.n_prefix;
   sa.num_sms = m->num_sms;
   const bool thin_launch = t_cap <= kThinRows;
-  const bool pair = m->pair_clusters > 0 && !m->e4m3 && !thin_launch;
+  const bool pair = m->pair_clusters > 0 && !m->e4m3 && !thin_launch && t_cap >= m->pair_rows;
   sa.nsparse_rows = pair ? 2 * kBM : kBM;
   sa.qkv_step = thin_launch ? kBHalf : 2 * kBHalf;
   sa.nsparse_wave = pair ? m->pair_clusters : m->num_sms;
@@ -1147,10 +1153,12 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
     p.mapB[2] = tm[2];
     if (f8) set_f8(p, map_aq_x, tm8, sc8, {0, 1, 2});
     if (pair) {
-      const CUtensorMap* tp = &m->tm_pair[static_cast<size_t>(l) * 5];
+      // (tiles of at most 128 columns have 64 rows of B per CTA)
+      const CUtensorMap* tp = &m->tm_pair[static_cast<size_t>(l) * 3];
       p.mapB[0] = tp[0];
       p.mapB[1] = tp[1];
       p.mapB[2] = tp[2];
+      p.b_box_rows = 64;
     }
     p.tiles = sa.qkv_tiles + static_cast<size_t>(l) * L.qkv_cap;
     p.tile_count = counts + l;
@@ -1277,10 +1285,6 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
     p.mapB[0] = tm[4];
     p.mapB[1] = tm[5];
     if (f8) set_f8(p, map_aq_x, tm8, sc8, {4, 5});
-    if (pair) {
-      p.mapB[0] = m->tm_pair[static_cast<size_t>(l) * 5 + 3];
-      p.mapB[1] = m->tm_pair[static_cast<size_t>(l) * 5 + 4];
-    }
     p.b_split = 1;
     p.tiles = sa.gu_tiles + static_cast<size_t>(l) * L.gu_cap;
     p.tile_count = counts + 2 * nl + l;

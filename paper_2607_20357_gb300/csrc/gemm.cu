@@ -1278,10 +1278,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
 #define SVL_PAIR_STAGES 6
 #endif
 constexpr int kPairStages = SVL_PAIR_STAGES;
-constexpr int kPairBox = 64;                         // B rows per TMA box (64-row tensor maps)
 constexpr int kPairBBytes = kBHalf * kBK * 2;        // up to 128 B rows per CTA
 constexpr int kPairStageBytes = kABytes + kPairBBytes;
-constexpr int kPairSmem = kPairStages * kPairStageBytes + 1024 + 256;
+constexpr int kPairSmem = kPairStages * kPairStageBytes + 1024 + 1024 + kResidStageBytes;
 static_assert(kPairSmem <= 232448, "shared memory per CTA");
 
 // MMA N of a pair tile: gate/up tiles are 128 gate + 128 up rows; others
@@ -1291,6 +1290,9 @@ SVL_DEVINL int pair_n(const GemmParams& p, const TileInfo& ti) {
   return ti.ncols > kBHalf ? 2 * kBHalf : kBHalf;
 }
 
+// One thread per CTA loads its rows of A (OP 0), one its half of B (OP 1); the
+// leader's post the byte counts of both CTAs.
+template <int OP>
 SVL_DEVINL void pair_producer(const GemmParams& p, uint8_t* stages, uint64_t* full, uint64_t* empty, uint32_t rank,
                               volatile int* abort) {
   const int npairs = gridDim.x >> 1, pair = blockIdx.x >> 1;
@@ -1307,10 +1309,10 @@ SVL_DEVINL void pair_producer(const GemmParams& p, uint8_t* stages, uint64_t* fu
   for (int t = pair; t < wk.n; t += npairs) {
     const TileInfo ti = get_tile(p, wk, t, npairs);
     if (!ti.valid) continue;
-    const int brows = pair_n(p, ti) / 2;
+    const int brows = pair_n(p, ti) / 2, box = p.b_box_rows ? p.b_box_rows : kBHalf;
     const CUtensorMap* mb = p.b_split ? &p.mapB[rank] : &p.mapB[ti.mat];
     const int by = p.b_split ? ti.n0 : ti.n0 + static_cast<int>(rank) * brows;
-    const uint32_t bytes = 2u * static_cast<uint32_t>(kABytes + brows * 128);
+    const uint32_t bytes = 2u * static_cast<uint32_t>(OP == 0 ? kABytes : brows * 128);
     int i0, i1;
     k_share(ti, nkb, kgb, i0, i1);
     KWalk w(kgb, ti.kmask, i0);
@@ -1320,11 +1322,14 @@ SVL_DEVINL void pair_producer(const GemmParams& p, uint8_t* stages, uint64_t* fu
         return;
       }
       uint8_t* sa = stages + s * kPairStageBytes;
-      uint8_t* sb = sa + kABytes;
       if (rank == 0) mbar_arrive_expect_tx(&full[s], bytes);
       const uint32_t fb = mapa_shared(&full[s], 0);
-      tma_load_2d_pair(sa, &p.mapA, fb, w.kb * kBK, ti.m0 + static_cast<int>(rank) * kBM);
-      for (int r = 0; r < brows; r += kPairBox) tma_load_2d_pair(sb + r * 128, mb, fb, w.kb * kBK, by + r);
+      if constexpr (OP == 0) {
+        tma_load_2d_pair(sa, &p.mapA, fb, w.kb * kBK, ti.m0 + static_cast<int>(rank) * kBM);
+      } else {
+        for (int r = 0; r < brows; r += box)
+          tma_load_2d_pair(sa + kABytes + r * 128, mb, fb, w.kb * kBK, by + r);
+      }
       next();
     }
   }
@@ -1343,6 +1348,7 @@ SVL_DEVINL void pair_mma(const GemmParams& p, uint8_t* stages, uint64_t* full, u
   const int npairs = gridDim.x >> 1, pair = blockIdx.x >> 1;
   Work wk = load_work(p, pair);
   const int nkb = p.K / kBK, kgb = p.kgroup / kBK;
+  const uint64_t da0 = smem_desc_sw128(smem_u32(stages)), db0 = smem_desc_sw128(smem_u32(stages) + kABytes);
   int s = 0, it = 0;
   uint32_t ph = 0;
   for (int t = pair; t < wk.n; t += npairs) {
@@ -1366,11 +1372,11 @@ SVL_DEVINL void pair_mma(const GemmParams& p, uint8_t* stages, uint64_t* full, u
         return;
       }
       tc_fence_after();
-      const uint32_t a0 = smem_u32(stages + s * kPairStageBytes);
-      const uint32_t b0 = a0 + kABytes;
+      const uint64_t da = da0 + static_cast<uint32_t>(s * (kPairStageBytes / 16));
+      const uint64_t db = db0 + static_cast<uint32_t>(s * (kPairStageBytes / 16));
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        tc_mma_bf16_pair(d, smem_desc_sw128(a0 + k * 32), smem_desc_sw128(b0 + k * 32), idesc, accumulate);
+        tc_mma_bf16_pair(d, da + 2 * k, db + 2 * k, idesc, accumulate);
         accumulate = 1;
       }
       tc_commit_pair(&empty[s]);
@@ -1386,17 +1392,21 @@ SVL_DEVINL void pair_mma(const GemmParams& p, uint8_t* stages, uint64_t* full, u
 
 template <int KIND>
 SVL_DEVINL void pair_epilogue(const GemmParams& p, uint64_t* tfull, uint64_t* tempty, uint32_t tmem, uint32_t rank,
-                              volatile int* abort) {
+                              volatile int* abort, uint8_t* rstage) {
   const int npairs = gridDim.x >> 1, pair = blockIdx.x >> 1;
   Work wk = load_work(p, pair);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = warp & 3;  // TMEM lane quarter this warp may access
+  uint8_t* wst = rstage + q * 2 * kResidChunk;
+  uint32_t sbuf = 0;
   int it = 0;
   for (int t = pair; t < wk.n; t += npairs) {
-    const TileInfo ti = get_tile(p, wk, t, npairs);
+    TileInfo ti = get_tile(p, wk, t, npairs);
     if (!ti.valid) continue;
+    ti.m0 += static_cast<int>(rank) * kBM;  // this CTA's rows
     const int acc = it & 1;
     const uint32_t aph = (it >> 1) & 1;
+    const bool staged = p.stage_tma && (ti.ncols & 63) == 0 && (ti.n0 & 7) == 0 && ti.m0 + q * 32 + 32 <= ti.m_end;
     const bool ok = mbar_wait(&tfull[acc], aph, abort);
     __syncwarp();
     if (!__all_sync(0xffffffffu, ok)) {
@@ -1404,9 +1414,14 @@ SVL_DEVINL void pair_epilogue(const GemmParams& p, uint64_t* tfull, uint64_t* te
       return;
     }
     tc_fence_after();
-    const int row = ti.m0 + static_cast<int>(rank) * kBM + q * 32 + lane;
+    const int row = ti.m0 + q * 32 + lane;
     const uint32_t taddr = tmem + acc * kAccCols + (static_cast<uint32_t>(q * 32) << 16);
-    epilogue_tile<KIND, false>(p, ti, row, row < ti.m_end, taddr);
+    if (KIND == EPI_SWIGLU && staged)
+      swiglu_tile_tma<false>(p, ti, q, taddr, wst, sbuf);
+    else if (KIND == EPI_QKV_ROPE && staged && ti.mat < 2 && (p.d_head & 63) == 0)
+      qkv_tile_tma<false>(p, ti, q, taddr, wst);
+    else
+      epilogue_tile<KIND, false>(p, ti, row, row < ti.m_end, taddr);
     tc_fence_before();
     if (rank == 0)
       mbar_arrive(&tempty[acc]);
@@ -1414,6 +1429,7 @@ SVL_DEVINL void pair_epilogue(const GemmParams& p, uint64_t* tfull, uint64_t* te
       mbar_arrive_cluster(mapa_shared(&tempty[acc], 0));
     ++it;
   }
+  if (lane == 0) bulk_wait0();  // this warp's staged stores are complete
 }
 
 template <int KIND>
@@ -1428,10 +1444,10 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kPairStages + 4);
   volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const uint32_t rank = cluster_rank();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);  // uniform over the warp
   if (threadIdx.x == 0) {
     for (int i = 0; i < kPairStages; ++i) {
-      mbar_init(&full[i], 1);
+      mbar_init(&full[i], 2);  // the leader's two producers
       mbar_init(&empty[i], 1);
     }
     for (int i = 0; i < 2; ++i) {
@@ -1456,11 +1472,13 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
   pdl_begin(p.late);
 
   if (warp == 0) {
-    if (lane == 0) pair_producer(p, stages, full, empty, rank, abort);
+    if (elect_one()) pair_producer<1>(p, stages, full, empty, rank, abort);
+  } else if (warp == 6) {
+    if (elect_one()) pair_producer<0>(p, stages, full, empty, rank, abort);
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) pair_mma(p, stages, full, empty, tfull, tempty, tmem, abort);
+    if (rank == 0 && elect_one()) pair_mma(p, stages, full, empty, tfull, tempty, tmem, abort);
   } else {
-    pair_epilogue<KIND>(p, tfull, tempty, tmem, rank, abort);
+    pair_epilogue<KIND>(p, tfull, tempty, tmem, rank, abort, stages + kPairStages * kPairStageBytes + 1024);
   }
 
   __syncwarp();

@@ -21,7 +21,7 @@ constexpr int kABytes = kBM * kBK * 2;
 constexpr int kBHalfBytes = kBHalf * kBK * 2;
 constexpr int kStageBytes = kABytes + 2 * kBHalfBytes;
 constexpr int kGemmThreads = 224;  // warp 0 TMA of B, warp 1 MMA + TMEM, warps 2-5 epilogue, warp 6 TMA of A
-constexpr int kPairThreads = 192;  // CTA pairs: one TMA warp
+constexpr int kPairThreads = 224;  // CTA pairs: the same roles
 constexpr int kAccCols = 256;      // fp32 columns per accumulator
 constexpr int kTmemCols = 512;     // two accumulators (epilogue overlaps the next tile)
 constexpr int kGemmSmem = kStages * kStageBytes + 1024 /*align*/ + 256 /*barriers*/;
@@ -135,7 +135,8 @@ cudaError_t launch_gemm(EpiKind kind, const GemmParams& p, int grid, cudaStream_
 
 // The gated QKV / gate-up GEMM on 256-row tiles by clusters of two CTAs
 // (tcgen05 cta_group::2): `pairs` clusters walk the tile list (tiles of up to
-// 256 rows), mapA has 128-row boxes, mapB 64-row boxes. bf16 only.
+// 256 rows), mapA has 128-row boxes, mapB b_box_rows (0: 128; 64 where tiles may
+// have 128 columns or fewer). bf16 only.
 cudaError_t launch_gemm_pair(EpiKind kind, const GemmParams& p, int pairs, cudaStream_t stream);
 // Clusters of two of the pair kernel that can be resident at once (0 if the
 // query fails).
