@@ -114,6 +114,7 @@ constexpr int kMaxPrefillBatch = 4096;  // samples per prefill call
 // that end inside a tile, more of a tile is padding. Measured over one layer's MLP
 // and QKV + O at LLaVA-7B and Qwen2-VL-7B widths, all groups on and mixed masks: 4 to
 // 10 % faster at 3,072 rows and more, -2 to +6 % at 1,024 to 2,048, -4 % (MLP) at 320.
+// e4m3 models: the MLP of one layer with its quantisers at 5,400 rows 584 -> 548 us.
 constexpr int kPairRows = 3072;
 
 // Each call keeps its scratch at the start of the workspace: no data flows
@@ -319,7 +320,7 @@ svl_status launch_pair(EpiKind kind, svl_model* m, int tag, const GemmParams& p,
   if (tiles <= 0) return SVL_OK;
   Launch L(m, tag, s);
   const int pairs = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(m->pair_clusters, tiles)));
-  return launch_gemm_pair(kind, p, pairs, s) == cudaSuccess ? SVL_OK : SVL_ERR_CUDA;
+  return launch_gemm_pair(kind, p, pairs, s, m->e4m3) == cudaSuccess ? SVL_OK : SVL_ERR_CUDA;
 }
 
 svl_status last_error() { return cudaGetLastError() == cudaSuccess ? SVL_OK : SVL_ERR_CUDA; }
@@ -467,6 +468,7 @@ svl_status svl_model_create(const svl_model_desc* desc, const svl_weights* w, sv
     m->f8_mem.assign(d.n_layers, nullptr);
     m->f8_scale.assign(static_cast<size_t>(d.n_layers) * 7, nullptr);
     m->tm8.resize(static_cast<size_t>(d.n_layers) * 7);
+    m->tm_pair.resize(static_cast<size_t>(d.n_layers) * 3);
     for (int l = 0; l < d.n_layers && ok; ++l) {
       const svl_layer_weights& lw = m->layers[l];
       const void* src[7] = {lw.wq, lw.wk, lw.wv, lw.wo, lw.wg, lw.wu, lw.wd};
@@ -488,7 +490,8 @@ svl_status svl_model_create(const svl_model_desc* desc, const svl_weights* w, sv
         qa.scale = reinterpret_cast<float*>(base + scale_off[i]);
         m->f8_scale[static_cast<size_t>(l) * 7 + i] = qa.scale;
         ok = launch_quant_rows(qa, 0) == cudaSuccess &&
-             make_map8(&m->tm8[static_cast<size_t>(l) * 7 + i], qa.dst, rows[i], qa.ld_dst);
+             make_map8(&m->tm8[static_cast<size_t>(l) * 7 + i], qa.dst, rows[i], qa.ld_dst) &&
+             (i > 2 || make_map8(&m->tm_pair[static_cast<size_t>(l) * 3 + i], qa.dst, rows[i], qa.ld_dst, 64));
         g_launches++;
       }
     }
@@ -515,18 +518,18 @@ svl_status svl_model_create(const svl_model_desc* desc, const svl_weights* w, sv
     svl_model_destroy(m);
     return SVL_ERR_INVALID_ARG;
   }
-  // CTA-pair QKV and gate/up GEMMs for bf16 models: from kPairRows rows on, or
+  // CTA-pair QKV and gate/up GEMMs: from kPairRows rows on, or
   // as SVL_PAIR_GEMM in the environment at model creation says (1: for every
   // batch but decode-sized ones, 0: never).
-  if (ok && !m->e4m3) {
+  if (ok) {
     const char* env = std::getenv("SVL_PAIR_GEMM");
     m->pair_rows = env && env[0] == '1' ? 0 : kPairRows;
     if (!env || env[0] != '0') {
-      const int c = std::min(gemm_pair_max_clusters(EPI_QKV_ROPE), gemm_pair_max_clusters(EPI_SWIGLU));
+      const int c = std::min(gemm_pair_max_clusters(EPI_QKV_ROPE, m->e4m3), gemm_pair_max_clusters(EPI_SWIGLU, m->e4m3));
       m->pair_clusters = std::min(c, m->num_sms / 2);
     }
     cudaGetLastError();  // a failed occupancy query only disables the pair kernel
-    if (m->pair_clusters > 0) {
+    if (m->pair_clusters > 0 && !m->e4m3) {
       m->tm_pair.resize(static_cast<size_t>(d.n_layers) * 3);
       for (int l = 0; l < d.n_layers && ok; ++l) {
         const svl_layer_weights& lw = m->layers[l];
@@ -790,7 +793,9 @@ svl_status pack_impl(svl_model* m, int32_t B, int32_t n_vis_total, int32_t n_tex
   if (d.proj_hidden && n_vis_total > 0) {
     // 128-column tiles (six stages of 32 KB) while at most two thirds of the
     // SMs would have a 256-column one: a tile then takes half the time, and
-    // even every token kept makes no more than two waves of them
+    // even every token kept makes no more than two waves of them (one request of
+    // 576 tokens, 5 x 16 wide tiles, over four layers: 828 us; 801 with these tiles and the
+    // controller's and the gather's launches merged)
     const int64_t wide = static_cast<int64_t>((n_vis_total + kBM - 1) / kBM) * ((d.d_model + 255) / 256);
     const bool narrow = 3 * wide <= 2 * m->num_sms;
     GemmParams p = base_params(m);
@@ -906,7 +911,7 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
   sa.P = d.n_prefix;
   sa.num_sms = m->num_sms;
   const bool thin_launch = t_cap <= kThinRows;
-  const bool pair = m->pair_clusters > 0 && !m->e4m3 && !thin_launch && t_cap >= m->pair_rows;
+  const bool pair = m->pair_clusters > 0 && !thin_launch && t_cap >= m->pair_rows;
   sa.nsparse_rows = pair ? 2 * kBM : kBM;
   sa.qkv_step = thin_launch ? kBHalf : 2 * kBHalf;
   sa.nsparse_wave = pair ? m->pair_clusters : m->num_sms;

@@ -61,7 +61,8 @@ SVL_DEVINL Work load_work(const GemmParams& p, int first) {
     w.gm = max((w.mlim + kBM - 1) / kBM, 1);
     w.whole = w.n = w.gm * p.grid_n;
     // a last wave of 256-column tiles that is at most half full is cut into
-    // 128-column halves, which fit in one wave and take half the time
+    // 128-column halves, which fit in one wave and take half the time (gather
+    // and projector of 16 samples of 576 tokens at half the budget: 141.8 -> 137.1 us)
     const int r = w.n % gridDim.x;
     if (p.bn == 2 * kBHalf && 2 * r <= static_cast<int>(gridDim.x)) {
       w.whole -= r;
@@ -193,7 +194,7 @@ struct StageCfg<EPI_LOGITS_T, true> {
   static constexpr int abytes = kABytes;
   static constexpr int bytes = kABytes + kThinRows * 128;
 };
-// Projector with few rows: 128-column tiles, six stages.
+// Projector with few rows (see pack_impl): 128-column tiles, six stages of 32 KB.
 template <>
 struct StageCfg<EPI_GELU, true> {
   static constexpr int stages = 6;
@@ -801,7 +802,9 @@ SVL_DEVINL void ksplit_rows(const GemmParams& p, const TileInfo& ti, uint8_t* ri
 // accumulator rows are staged there and stored 32 rows at a time, the residual
 // rows of the slice load while the shares meet, and the slice of every share
 // follows. At 309 rows (O projection, three shares) the epilogue threads'
-// own stores took 5.4 us and their loads 14 us; the bulk copies take 3 and 4.
+// own stores took 5.4 us and their loads 14 us; the bulk copies take 3 and 4,
+// and the sums 1.3 (four rows at a time; one at a time 3.5). THIN tiles were
+// slower through bulk copies (17 against 13 us a launch).
 template <bool F8, bool THIN>
 SVL_DEVINL bool ksplit_tile(const GemmParams& p, const TileInfo& ti, int lrow, uint32_t taddr, bool empty, KsSync& ks,
                             volatile int* abort, uint8_t* ring) {
@@ -1292,12 +1295,13 @@ SVL_DEVINL int pair_n(const GemmParams& p, const TileInfo& ti) {
 
 // One thread per CTA loads its rows of A (OP 0), one its half of B (OP 1); the
 // leader's post the byte counts of both CTAs.
-template <int OP>
+template <int OP, bool F8>
 SVL_DEVINL void pair_producer(const GemmParams& p, uint8_t* stages, uint64_t* full, uint64_t* empty, uint32_t rank,
                               volatile int* abort) {
   const int npairs = gridDim.x >> 1, pair = blockIdx.x >> 1;
   Work wk = load_work(p, pair);
-  const int nkb = p.K / kBK, kgb = p.kgroup / kBK;
+  constexpr int BK = F8 ? kBK8 : kBK;
+  const int nkb = p.K / BK, kgb = p.kgroup / BK;
   int s = 0;
   uint32_t ph = 0;
   auto next = [&]() {
@@ -1325,10 +1329,10 @@ SVL_DEVINL void pair_producer(const GemmParams& p, uint8_t* stages, uint64_t* fu
       if (rank == 0) mbar_arrive_expect_tx(&full[s], bytes);
       const uint32_t fb = mapa_shared(&full[s], 0);
       if constexpr (OP == 0) {
-        tma_load_2d_pair(sa, &p.mapA, fb, w.kb * kBK, ti.m0 + static_cast<int>(rank) * kBM);
+        tma_load_2d_pair(sa, &p.mapA, fb, w.kb * BK, ti.m0 + static_cast<int>(rank) * kBM);
       } else {
         for (int r = 0; r < brows; r += box)
-          tma_load_2d_pair(sa + kABytes + r * 128, mb, fb, w.kb * kBK, by + r);
+          tma_load_2d_pair(sa + kABytes + r * 128, mb, fb, w.kb * BK, by + r);
       }
       next();
     }
@@ -1343,11 +1347,13 @@ SVL_DEVINL void pair_producer(const GemmParams& p, uint8_t* stages, uint64_t* fu
   }
 }
 
+template <bool F8>
 SVL_DEVINL void pair_mma(const GemmParams& p, uint8_t* stages, uint64_t* full, uint64_t* empty, uint64_t* tfull,
                          uint64_t* tempty, uint32_t tmem, volatile int* abort) {
   const int npairs = gridDim.x >> 1, pair = blockIdx.x >> 1;
   Work wk = load_work(p, pair);
-  const int nkb = p.K / kBK, kgb = p.kgroup / kBK;
+  constexpr int BK = F8 ? kBK8 : kBK;
+  const int nkb = p.K / BK, kgb = p.kgroup / BK;
   const uint64_t da0 = smem_desc_sw128(smem_u32(stages)), db0 = smem_desc_sw128(smem_u32(stages) + kABytes);
   int s = 0, it = 0;
   uint32_t ph = 0;
@@ -1361,7 +1367,7 @@ SVL_DEVINL void pair_mma(const GemmParams& p, uint8_t* stages, uint64_t* full, u
       return;
     }
     tc_fence_after();
-    const uint32_t idesc = idesc_bf16_f32(2 * kBM, pair_n(p, ti));
+    const uint32_t idesc = F8 ? idesc_e4m3_f32(2 * kBM, pair_n(p, ti)) : idesc_bf16_f32(2 * kBM, pair_n(p, ti));
     const uint32_t d = tmem + acc * kAccCols;
     uint32_t accumulate = 0;
     int i0, i1;
@@ -1376,7 +1382,10 @@ SVL_DEVINL void pair_mma(const GemmParams& p, uint8_t* stages, uint64_t* full, u
       const uint64_t db = db0 + static_cast<uint32_t>(s * (kPairStageBytes / 16));
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        tc_mma_bf16_pair(d, da + 2 * k, db + 2 * k, idesc, accumulate);
+        if constexpr (F8)
+          tc_mma_e4m3_pair(d, da + 2 * k, db + 2 * k, idesc, accumulate);
+        else
+          tc_mma_bf16_pair(d, da + 2 * k, db + 2 * k, idesc, accumulate);
         accumulate = 1;
       }
       tc_commit_pair(&empty[s]);
@@ -1390,7 +1399,7 @@ SVL_DEVINL void pair_mma(const GemmParams& p, uint8_t* stages, uint64_t* full, u
   }
 }
 
-template <int KIND>
+template <int KIND, bool F8>
 SVL_DEVINL void pair_epilogue(const GemmParams& p, uint64_t* tfull, uint64_t* tempty, uint32_t tmem, uint32_t rank,
                               volatile int* abort, uint8_t* rstage) {
   const int npairs = gridDim.x >> 1, pair = blockIdx.x >> 1;
@@ -1417,11 +1426,11 @@ SVL_DEVINL void pair_epilogue(const GemmParams& p, uint64_t* tfull, uint64_t* te
     const int row = ti.m0 + q * 32 + lane;
     const uint32_t taddr = tmem + acc * kAccCols + (static_cast<uint32_t>(q * 32) << 16);
     if (KIND == EPI_SWIGLU && staged)
-      swiglu_tile_tma<false>(p, ti, q, taddr, wst, sbuf);
+      swiglu_tile_tma<F8>(p, ti, q, taddr, wst, sbuf);
     else if (KIND == EPI_QKV_ROPE && staged && ti.mat < 2 && (p.d_head & 63) == 0)
-      qkv_tile_tma<false>(p, ti, q, taddr, wst);
+      qkv_tile_tma<F8>(p, ti, q, taddr, wst);
     else
-      epilogue_tile<KIND, false>(p, ti, row, row < ti.m_end, taddr);
+      epilogue_tile<KIND, F8>(p, ti, row, row < ti.m_end, taddr);
     tc_fence_before();
     if (rank == 0)
       mbar_arrive(&tempty[acc]);
@@ -1432,7 +1441,7 @@ SVL_DEVINL void pair_epilogue(const GemmParams& p, uint64_t* tfull, uint64_t* te
   if (lane == 0) bulk_wait0();  // this warp's staged stores are complete
 }
 
-template <int KIND>
+template <int KIND, bool F8>
 __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid_constant__ GemmParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -1472,13 +1481,13 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
   pdl_begin(p.late);
 
   if (warp == 0) {
-    if (elect_one()) pair_producer<1>(p, stages, full, empty, rank, abort);
+    if (elect_one()) pair_producer<1, F8>(p, stages, full, empty, rank, abort);
   } else if (warp == 6) {
-    if (elect_one()) pair_producer<0>(p, stages, full, empty, rank, abort);
+    if (elect_one()) pair_producer<0, F8>(p, stages, full, empty, rank, abort);
   } else if (warp == 1) {
-    if (rank == 0 && elect_one()) pair_mma(p, stages, full, empty, tfull, tempty, tmem, abort);
+    if (rank == 0 && elect_one()) pair_mma<F8>(p, stages, full, empty, tfull, tempty, tmem, abort);
   } else {
-    pair_epilogue<KIND>(p, tfull, tempty, tmem, rank, abort, stages + kPairStages * kPairStageBytes + 1024);
+    pair_epilogue<KIND, F8>(p, tfull, tempty, tmem, rank, abort, stages + kPairStages * kPairStageBytes + 1024);
   }
 
   __syncwarp();
@@ -1497,11 +1506,12 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
   }
 }
 
-template <int KIND>
+template <int KIND, bool F8>
 static cudaError_t launch_pair_kind(const GemmParams& p, int pairs, cudaStream_t stream) {
   static bool configured = false;
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_pair_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmem);
+    cudaError_t e =
+        cudaFuncSetAttribute(gemm_pair_kernel<KIND, F8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmem);
     if (e != cudaSuccess) return e;
     configured = true;
   }
@@ -1519,19 +1529,25 @@ static cudaError_t launch_pair_kind(const GemmParams& p, int pairs, cudaStream_t
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, gemm_pair_kernel<KIND>, p);
+  return cudaLaunchKernelEx(&cfg, gemm_pair_kernel<KIND, F8>, p);
 }
 
-cudaError_t launch_gemm_pair(EpiKind kind, const GemmParams& p, int pairs, cudaStream_t stream) {
+cudaError_t launch_gemm_pair(EpiKind kind, const GemmParams& p, int pairs, cudaStream_t stream, bool e4m3) {
   if (pairs <= 0) return cudaSuccess;
+  if (e4m3 && (!p.a_scale || !p.b_scale[0])) return cudaErrorInvalidValue;
   switch (kind) {
-    case EPI_QKV_ROPE: return launch_pair_kind<EPI_QKV_ROPE>(p, pairs, stream);
-    case EPI_SWIGLU: return launch_pair_kind<EPI_SWIGLU>(p, pairs, stream);
+    case EPI_QKV_ROPE:
+      return e4m3 ? launch_pair_kind<EPI_QKV_ROPE, true>(p, pairs, stream)
+                  : launch_pair_kind<EPI_QKV_ROPE, false>(p, pairs, stream);
+    case EPI_SWIGLU:
+      return e4m3 ? launch_pair_kind<EPI_SWIGLU, true>(p, pairs, stream)
+                  : launch_pair_kind<EPI_SWIGLU, false>(p, pairs, stream);
     default: return cudaErrorInvalidValue;
   }
 }
 
-int gemm_pair_max_clusters(EpiKind kind) {
+template <int KIND, bool F8>
+static int pair_max_clusters_kind() {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2);
   cfg.blockDim = dim3(kPairThreads);
@@ -1544,15 +1560,16 @@ int gemm_pair_max_clusters(EpiKind kind) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  cudaError_t e;
-  if (kind == EPI_QKV_ROPE) {
-    e = cudaFuncSetAttribute(gemm_pair_kernel<EPI_QKV_ROPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, gemm_pair_kernel<EPI_QKV_ROPE>, &cfg);
-  } else {
-    e = cudaFuncSetAttribute(gemm_pair_kernel<EPI_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, gemm_pair_kernel<EPI_SWIGLU>, &cfg);
-  }
+  cudaError_t e =
+      cudaFuncSetAttribute(gemm_pair_kernel<KIND, F8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, gemm_pair_kernel<KIND, F8>, &cfg);
   return e == cudaSuccess ? n : 0;
+}
+
+int gemm_pair_max_clusters(EpiKind kind, bool e4m3) {
+  if (kind == EPI_QKV_ROPE)
+    return e4m3 ? pair_max_clusters_kind<EPI_QKV_ROPE, true>() : pair_max_clusters_kind<EPI_QKV_ROPE, false>();
+  return e4m3 ? pair_max_clusters_kind<EPI_SWIGLU, true>() : pair_max_clusters_kind<EPI_SWIGLU, false>();
 }
 
 // Dynamic shared memory of gemm_kernel: the stages, the alignment slack and

@@ -136,11 +136,11 @@ cudaError_t launch_gemm(EpiKind kind, const GemmParams& p, int grid, cudaStream_
 // The gated QKV / gate-up GEMM on 256-row tiles by clusters of two CTAs
 // (tcgen05 cta_group::2): `pairs` clusters walk the tile list (tiles of up to
 // 256 rows), mapA has 128-row boxes, mapB b_box_rows (0: 128; 64 where tiles may
-// have 128 columns or fewer). bf16 only.
-cudaError_t launch_gemm_pair(EpiKind kind, const GemmParams& p, int pairs, cudaStream_t stream);
+// have 128 columns or fewer).
+cudaError_t launch_gemm_pair(EpiKind kind, const GemmParams& p, int pairs, cudaStream_t stream, bool e4m3 = false);
 // Clusters of two of the pair kernel that can be resident at once (0 if the
 // query fails).
-int gemm_pair_max_clusters(EpiKind kind);
+int gemm_pair_max_clusters(EpiKind kind, bool e4m3);
 
 // CTAs of the residual (EPI_RESID) GEMM that fit on one SM at once, the
 // smaller of the wide and THIN instantiations (0 if the query fails).

@@ -48,6 +48,7 @@ __global__ void __launch_bounds__(kPackThreads) pack_offsets_kernel(PackArgs a) 
 // Every block forms the row offsets of all samples in shared memory (a launch
 // of one thread that walked them cost 4 us before this one); the first block
 // writes them out. Beyond kPackScan samples they come from their own launch.
+// Bound by memory: rows in, rows out, once each.
 __global__ void __launch_bounds__(kPackThreads) pack_gather_kernel(PackArgs a) {
   extern __shared__ int pack_cu[];  // [B + 1], up to kPackScan samples
   pdl_begin(a.use_projector);  // the projector GEMM loads weights before it waits

@@ -242,7 +242,10 @@ __device__ void top_k(const float* z, int n, int k, int* out, const uint32_t* sk
 }
 
 // One block per sample whose k is known (front_kernel): its kept offset is the
-// sum of the k before it, and its indices go to their final place.
+// sum of the k before it, and its indices go to their final place. Bound by the
+// latency of its radix passes over shared memory. A fourth launch that moved the
+// indices took 3.9 us; the controller of one 576-token sample went from 20.7 to
+// 18.4 us, of 64 samples from 33.5 to 28.9 us.
 __global__ void __launch_bounds__(kSelectThreads) topk_kernel(int B, const float* scores, const int* vis_off,
                                                               const int* k, int* kept_off, int* kept_idx) {
   __shared__ uint32_t topk_keys[kKeysShared];
