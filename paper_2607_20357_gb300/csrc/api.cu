@@ -175,11 +175,13 @@ PreLayout pre_layout(const svl_model_desc& d, int B, int64_t t_cap) {
   L.t_pad = (t_cap + 7) & ~int64_t(7);
   L.n_pad = ((B + 15) / 16) * 16;
   L.mt_max = static_cast<int>(t_cap / 128 + B + 1);
-  // (THIN launches cut Q, K and V into 128-column tiles)
-  const int step = t_cap <= kThinRows ? kBHalf : 2 * kBHalf;
-  const int qkv_nt = static_cast<int>((hq / step + G + 1) + 2 * (dkv / step + G + 1));
+  // Q, K and V are cut into 256-column tiles, in THIN launches into 128-column ones.
+  // The workspace of t_cap rows also serves every call of fewer, THIN ones among
+  // them, so its list has room for either (sizes grow with each argument).
+  auto qkv_nt = [&](int step) { return static_cast<int>((hq / step + G + 1) + 2 * (dkv / step + G + 1)); };
+  const int thin_tiles = (B + 1) * qkv_nt(kBHalf);  // (at most kThinRows < 128 rows)
   // + 256: room for the split tail (at most half a wave of extra tiles)
-  L.qkv_cap = L.mt_max * qkv_nt + 256;
+  L.qkv_cap = (t_cap <= kThinRows ? thin_tiles : std::max(thin_tiles, L.mt_max * qkv_nt(2 * kBHalf))) + 256;
   L.o_cap = L.mt_max * ((d.d_model + 255) / 256) + 256;
   L.dn_cap = L.o_cap;
   L.gu_cap = L.mt_max * (d.d_ffn / 128 + G + 1);
