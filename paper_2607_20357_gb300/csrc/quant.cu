@@ -161,15 +161,21 @@ __global__ void __launch_bounds__(kQuantThreads, NCH <= 4 ? 7 : NCH <= 12 ? 4 : 
   const int per_g = a.kgp / 8, src_per_g = a.kg / 8, nchunk = a.G * per_g;
   const bool gated = a.group_gate && a.l >= a.P;
   int col[NCH];  // source column of each chunk, its group in the top bits; group 31: padding (never in a mask)
-  uint4 gv[GAIN ? NCH : 1];  // (weights: no kernel of the call writes them)
+  uint4 gv[GAIN ? NCH : 1];
 #pragma unroll
   for (int i = 0; i < NCH; ++i) {
     const int c = tid + i * kQuantThreads, j = c / per_g, cc = c - j * per_g;
     const bool src = c < nchunk && cc < src_per_g;
     col[i] = src ? (j << 26) | (j * a.kg + cc * 8) : static_cast<int>(31u << 26);
-    if (GAIN) gv[i] = src ? *reinterpret_cast<const uint4*>(a.gain + (col[i] & kColMask)) : ones8();
   }
   pdl_begin(a.late);
+  // (the gain too may come from the launch before: svl_quantize_rows_e4m3 takes a caller's vector)
+  if constexpr (GAIN) {
+#pragma unroll
+    for (int i = 0; i < NCH; ++i)
+      gv[i] = static_cast<unsigned>(col[i]) >> 26 != 31u ? *reinterpret_cast<const uint4*>(a.gain + (col[i] & kColMask))
+                                                         : ones8();
+  }
   int64_t rows = a.rows;
   if (a.cu_seqlens) rows = min(rows, static_cast<int64_t>(a.cu_seqlens[a.B]));
   auto load = [&](int64_t r, int mask, uint4* v) {

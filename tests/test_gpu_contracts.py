@@ -54,3 +54,40 @@ def test_decode_of_32_samples_in_a_workspace_of_more(deep, sized_for):
     svl.svl_decode_step(deep.handle, B, tok, kv, max_len, length, lg, gg, logits, nxt, ws, ws.numel())
     assert svl.svl_get_device_status(deep.handle) == 0
     assert length.tolist() == [1] * B and torch.equal(nxt.long(), logits.argmax(1))
+
+
+# Calls are stream-ordered: what the launch before a call writes is an input like any other, although the library's
+# kernels start before their predecessor has ended. A pack whose projector is the identity makes such a predecessor:
+# it lets its successor start at once and then writes rows of X, which the next call reads.
+def _packer(rows, seed):
+    """A model and a batch of one sample whose pack writes `rows` text rows (embedding rows, so any bf16 data) to X."""
+    w = synth.make_weights(TINY.dims, seed, device="cuda")
+    m = svl.GatedPrefill(TINY.dims, w, max_seq=1024)
+    b = synth.make_batch(TINY, seed, n_vis_list=[1], s_text_list=[rows], keep_list=[0], device="cuda")
+    out = m.run(b, stages=("select", "pack"))
+    torch.cuda.synchronize()
+    assert torch.equal(out["X"][:rows], w["embed"][b["text_ids"].long()])
+    return m, b, out
+
+
+def test_quantiser_reads_a_gain_written_by_the_launch_before():
+    m, b, out = _packer(16, 91)
+    cols = 16 * TINY.dims.d_model  # one gain vector from 16 rows of X
+    gain = out["X"][:16].view(-1).clone()
+    src = torch.randn(64, cols, device="cuda", generator=torch.Generator("cuda").manual_seed(92)).to(torch.bfloat16)
+
+    def quant(g):
+        codes, scale = torch.zeros(64, cols, dtype=torch.uint8, device="cuda"), torch.zeros(64, device="cuda")
+        svl.svl_quantize_rows_e4m3(src, 64, cols, cols, codes, cols, scale, gain=g)
+        return codes, scale
+
+    want = quant(gain)
+    torch.cuda.synchronize()
+    for _ in range(20):
+        out["X"].zero_()
+        torch.cuda.synchronize()
+        m.run(b, out=out, stages=("pack",))
+        got = quant(out["X"][:16])
+        torch.cuda.synchronize()
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    m.close()
