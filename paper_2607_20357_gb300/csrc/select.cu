@@ -10,8 +10,7 @@ namespace svl {
 // pow per call took 2 us). One block per sample. The argument reaches 1000 rad,
 // so it is formed and reduced to [-pi, pi] in double precision before the
 // single-precision sine and cosine (error about 1e-7 either way); the two H x H
-// products run in fp32 from shared memory, four threads per output. The weights
-// are copied there before the wait for the predecessor.
+// products run in fp32 from shared memory, four threads per output.
 constexpr double kTwoPi = 6.283185307179586;
 constexpr int kFrontThreads = 256;
 
@@ -57,7 +56,9 @@ __global__ void __launch_bounds__(kFrontThreads) front_kernel(FrontArgs f) {
   const int b = blockIdx.x, i = threadIdx.x, H = f.H;
   __nv_bfloat16* sw1 = reinterpret_cast<__nv_bfloat16*>(front_smem);
   __nv_bfloat16* sw2 = sw1 + H * H;
+  pdl_begin(true);  // the score GEMM loads its operands before it waits
   if (b < f.B) {
+    // (after the wait: the launch before may be the caller's update of these weights)
     if (f.w_vec) {
       for (int c = i; c < H * H / 8; c += kFrontThreads) {
         reinterpret_cast<uint4*>(sw1)[c] = reinterpret_cast<const uint4*>(f.w1)[c];
@@ -69,9 +70,6 @@ __global__ void __launch_bounds__(kFrontThreads) front_kernel(FrontArgs f) {
         sw2[c] = f.w2[c];
       }
     }
-  }
-  pdl_begin(true);  // the score GEMM loads its operands before it waits
-  if (b < f.B) {
     if (i < H) {
       const int half = H / 2;
       const double arg = 1000.0 * static_cast<double>(f.budget[b]) * f.omega[i < half ? i : i - half];

@@ -91,3 +91,30 @@ def test_quantiser_reads_a_gain_written_by_the_launch_before():
         torch.cuda.synchronize()
         assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
     m.close()
+
+
+def test_controller_reads_budget_weights_written_by_the_launch_before():
+    packer, b, out = _packer(32, 93)
+    dims = synth.reduced(LLAVA.dims, n_layers=1, vocab=512)
+    w = synth.make_weights(dims, 94, device="cuda")
+    H, X = dims.h_ctrl, out["X"]
+    rows = H * H // TINY.dims.d_model  # bud_w1 and bud_w2 are rows of X
+    w["bud_w1"], w["bud_w2"] = X[:rows].view(H, H), X[rows:2 * rows].view(H, H)
+    m = svl.GatedPrefill(dims, w, max_seq=1024)
+    batch = synth.make_batch(LLAVA, 95, batch=4, dims=dims, budget_list=[0.2, 0.5, 0.7, 1.0], device="cuda")
+    got = m.run(batch, stages=("select",))
+    torch.cuda.synchronize()
+    want = {k: got[k].clone() for k in ("scores", "k", "kept_idx", "kept_off")}
+    assert float(want["scores"].std()) > 0
+    for _ in range(20):
+        X.zero_()
+        torch.cuda.synchronize()
+        packer.run(b, out=out, stages=("pack",))
+        m.run(batch, out=got, stages=("select",))
+        torch.cuda.synchronize()
+        for key in ("scores", "k", "kept_off"):
+            assert torch.equal(got[key], want[key]), key
+        n = int(want["kept_off"][-1])
+        assert torch.equal(got["kept_idx"][:n], want["kept_idx"][:n])
+    m.close()
+    packer.close()
