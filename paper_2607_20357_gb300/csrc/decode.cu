@@ -457,8 +457,9 @@ cudaError_t launch_decode_attn(const DecAttnArgs& a, cudaStream_t s) {
 // Greedy next token per sample (largest logit; equal logits: lower id) and
 // the cache length advanced by the fed token. A cluster of kFinSplit CTAs
 // scans a sample's logits in contiguous parts (one block took 11 us for
-// 152,064 logits); with V a multiple of 4 each thread reads float4s (4
-// consecutive ids, kept in id order, so the tie rule holds).
+// 152,064 logits); with V a multiple of 4 and 16-byte aligned logits (`vec`)
+// each thread reads float4s (4 consecutive ids, kept in id order, so the tie
+// rule holds).
 constexpr int kFinThreads = 512, kFinSplit = 8;
 
 SVL_DEVINL void arg_better(float x, int v, float& best, int& idx) {
@@ -468,8 +469,8 @@ SVL_DEVINL void arg_better(float x, int v, float& best, int& idx) {
   }
 }
 
-__global__ void __launch_bounds__(kFinThreads) decode_finish_kernel(int B, int V, const float* logits, int* next_token,
-                                                                    int* cache_len, int max_len) {
+__global__ void __launch_bounds__(kFinThreads) decode_finish_kernel(int B, int V, const float* logits, bool vec,
+                                                                    int* next_token, int* cache_len, int max_len) {
   __shared__ float bv[kFinThreads / 32];
   __shared__ int bi[kFinThreads / 32];
   __shared__ float cta_v;
@@ -479,7 +480,7 @@ __global__ void __launch_bounds__(kFinThreads) decode_finish_kernel(int B, int V
   const float* row = logits + static_cast<size_t>(b) * V;
   float best = -INFINITY;
   int idx = 0x7fffffff;
-  if ((V & 3) == 0) {
+  if (vec) {
     const float4* r4 = reinterpret_cast<const float4*>(row);
     const int n4 = V / 4, per = (n4 + kFinSplit - 1) / kFinSplit, c1 = min(n4, (part + 1) * per);
 #pragma unroll 4
@@ -527,7 +528,9 @@ __global__ void __launch_bounds__(kFinThreads) decode_finish_kernel(int B, int V
 
 cudaError_t launch_decode_finish(int B, int V, const float* logits, int* next_token, int* cache_len, int max_len,
                                  cudaStream_t s) {
-  return launch_pdl_cluster(decode_finish_kernel, dim3(kFinSplit, B), kFinThreads, 0, kFinSplit, s, B, V, logits,
+  // (the ABI asks for no alignment of the caller's logits beyond a float's)
+  const bool vec = (V & 3) == 0 && (reinterpret_cast<uintptr_t>(logits) & 15) == 0;
+  return launch_pdl_cluster(decode_finish_kernel, dim3(kFinSplit, B), kFinThreads, 0, kFinSplit, s, B, V, logits, vec,
                             next_token, cache_len, max_len);
 }
 

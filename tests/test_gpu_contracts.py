@@ -118,3 +118,30 @@ def test_controller_reads_budget_weights_written_by_the_launch_before():
         assert torch.equal(got["kept_idx"][:n], want["kept_idx"][:n])
     m.close()
     packer.close()
+
+
+def test_decode_with_logits_aligned_to_a_float_only():
+    """Logits that start 4 bytes past a 16-byte boundary, a vocabulary that is a multiple of four."""
+    dims = synth.reduced(TINY.dims, vocab=1024)
+    m = svl.GatedPrefill(dims, synth.make_weights(dims, 96, device="cuda"), max_seq=64)
+    B, V, max_len = 3, dims.vocab, 8
+    i32 = dict(dtype=torch.int32, device="cuda")
+    lg = torch.ones(B, dims.n_layers, dtype=torch.uint8, device="cuda")
+    gg = torch.ones(B, dims.n_layers, dims.n_groups, dtype=torch.uint8, device="cuda")
+    ws = torch.empty(svl.svl_decode_workspace_size(m.handle, B), dtype=torch.uint8, device="cuda")
+
+    def step(logits):
+        kv = torch.zeros(svl.svl_kv_cache_size(m.handle, B, max_len) // 2, dtype=torch.bfloat16, device="cuda")
+        nxt, length = torch.full((B,), -5, **i32), torch.zeros(B, **i32)
+        svl.svl_decode_step(m.handle, B, torch.arange(B, **i32), kv, max_len, length, lg, gg, logits, nxt, ws,
+                            ws.numel())
+        assert svl.svl_get_device_status(m.handle) == 0
+        return nxt
+
+    aligned, base = torch.empty(B, V, device="cuda"), torch.empty(B * V + 4, device="cuda")
+    want = step(aligned)
+    for shift in (1, 2, 3):
+        view = base[shift:shift + B * V].view(B, V)
+        assert torch.equal(step(view), want) and torch.equal(view, aligned)
+        assert torch.equal(want.long(), view.argmax(1))
+    m.close()
