@@ -312,10 +312,10 @@ svl_status svl_quantize_rows_e4m3(const void* src, const void* gain, int64_t row
 /* The e4m3 GEMM of the gated projections on its own, with an fp32 output:
  * C[m, n] = a_scale[m] * b_scale[n] * sum_k A[m, k] B[n, k], A [M, K] and
  * B [N, K] device uint8 e4m3 codes (row-major, K contiguous, 16-byte
- * aligned), scales float32, C float32 [M, N] row-major; all caller-owned.
- * Requires K a multiple of 128 and N a multiple of 32 (else
- * SVL_ERR_INVALID_ARG). The model supplies the device status word and the
- * SM count only. Asynchronous on `stream`. */
+ * aligned), scales float32 (b_scale 16-byte aligned), C float32 [M, N]
+ * row-major; all caller-owned. Requires K a multiple of 128, N a multiple of
+ * 32 and that alignment (else SVL_ERR_INVALID_ARG). The model supplies the
+ * device status word and the SM count only. Asynchronous on `stream`. */
 svl_status svl_gemm_e4m3(svl_model* model, const void* A, const float* a_scale, const void* B, const float* b_scale,
                          int32_t M, int32_t N, int32_t K, float* C, void* stream);
 

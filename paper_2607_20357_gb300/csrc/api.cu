@@ -1531,7 +1531,8 @@ svl_status svl_quantize_rows_e4m3(const void* src, const void* gain, int64_t row
 
 svl_status svl_gemm_e4m3(svl_model* m, const void* A, const float* a_scale, const void* B, const float* b_scale,
                          int32_t M, int32_t N, int32_t K, float* C, void* stream) {
-  if (!m || !A || !a_scale || !B || !b_scale || !C || M <= 0 || N <= 0 || K <= 0 || (K % kBK8) || (N & 31))
+  if (!m || !A || !a_scale || !B || !b_scale || !C || M <= 0 || N <= 0 || K <= 0 || (K % kBK8) || (N & 31) ||
+      !aligned16(b_scale))  // read as 16-byte vectors
     return SVL_ERR_INVALID_ARG;
   GemmParams p = base_params(m);
   if (!make_map8(&p.mapA, A, M, K) || !make_map8(&p.mapB[0], B, N, K)) return SVL_ERR_INVALID_ARG;

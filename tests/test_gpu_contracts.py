@@ -145,3 +145,20 @@ def test_decode_with_logits_aligned_to_a_float_only():
         assert torch.equal(step(view), want) and torch.equal(view, aligned)
         assert torch.equal(want.long(), view.argmax(1))
     m.close()
+
+
+def test_e4m3_gemm_refuses_column_scales_it_cannot_read():
+    """b_scale is read as 16-byte vectors: other alignments are an argument error and launch nothing."""
+    m = svl.GatedPrefill(TINY.dims, synth.make_weights(TINY.dims, 97, device="cuda"), max_seq=64)
+    M, N, K = 16, 64, 128
+    one = 0x38  # e4m3 code of 1
+    A, B = (torch.full((n, K), one, dtype=torch.uint8, device="cuda") for n in (M, N))
+    a_scale, b_scale = torch.ones(M + 1, device="cuda"), torch.ones(N + 4, device="cuda")
+    C, before = torch.zeros(M, N, device="cuda"), svl.svl_launch_count()
+    for shift in (1, 2, 3):
+        with pytest.raises(svl.SvlError) as e:
+            svl.svl_gemm_e4m3(m.handle, A, a_scale, B, b_scale[shift:], M, N, K, C)
+        assert e.value.code == 1 and svl.svl_launch_count() == before
+    svl.svl_gemm_e4m3(m.handle, A, a_scale[1:], B, b_scale[4:], M, N, K, C)  # rows: any float
+    assert svl.svl_get_device_status(m.handle) == 0 and bool((C == K).all())
+    m.close()
