@@ -26,6 +26,9 @@ namespace svl {
 //    what no kernel of the call writes (weights). Only kernels in front of one
 //    that does so pay for it: in chains of kernels of a few microseconds a
 //    late trigger exposes about 3 us of launch latency per kernel.
+// A kernel may thus be resident while its inputs are written, so nothing an
+// earlier launch (or the caller) writes is read through the non-coherent path
+// (__ldg, or __restrict__ pointers, from which the compiler derives it).
 SVL_DEVINL void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 SVL_DEVINL void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

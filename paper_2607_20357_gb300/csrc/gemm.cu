@@ -380,7 +380,7 @@ SVL_DEVINL void scale_cols(float* v, const float* cs, float f) {
   const float4* c4 = reinterpret_cast<const float4*>(cs);
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    const float4 c = __ldg(c4 + i);
+    const float4 c = c4[i];
     v[4 * i] *= f * c.x;
     v[4 * i + 1] *= f * c.y;
     v[4 * i + 2] *= f * c.z;
@@ -657,7 +657,7 @@ SVL_DEVINL void ksplit_slot(const GemmParams& p, const TileInfo& ti, const float
       }
     }
     if constexpr (F8) {
-      const float4 cs = __ldg(reinterpret_cast<const float4*>(p.b_scale[0] + ti.n0 + col));
+      const float4 cs = *reinterpret_cast<const float4*>(p.b_scale[0] + ti.n0 + col);
       const float rs = p.a_scale[ti.m0 + row];
       v.x *= rs * cs.x;
       v.y *= rs * cs.y;
@@ -702,7 +702,7 @@ SVL_DEVINL void ksplit_rows(const GemmParams& p, const TileInfo& ti, uint8_t* ri
     float cs[8];
     if constexpr (F8) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) cs[i] = __ldg(p.b_scale[0] + ti.n0 + c + i);
+      for (int i = 0; i < 8; ++i) cs[i] = p.b_scale[0][ti.n0 + c + i];
     }
     // four rows at a time: a row alone exposed its reads' latency (600 cycles)
     const int u0 = (c >> 2) & 7;

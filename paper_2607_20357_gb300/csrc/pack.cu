@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kPackThreads) pack_gather_kernel(PackArgs a) {
     uint4 v[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u)
-      if (c0 + 32 * u < n) v[u] = bad ? make_uint4(0, 0, 0, 0) : __ldg(src + c0 + 32 * u);
+      if (c0 + 32 * u < n) v[u] = bad ? make_uint4(0, 0, 0, 0) : src[c0 + 32 * u];
 #pragma unroll
     for (int u = 0; u < 4; ++u)
       if (c0 + 32 * u < n) dst[c0 + 32 * u] = v[u];
@@ -118,9 +118,8 @@ void launch_offsets_diff(const int* off, int* len, int B, cudaStream_t s) {
 }
 
 // One block per sample: PE(b) and the hidden layer in double, then D outputs.
-__global__ void llm_budget_embed_kernel(const float* __restrict__ budget, const __nv_bfloat16* __restrict__ w1,
-                                        const __nv_bfloat16* __restrict__ w2, int H, int D,
-                                        __nv_bfloat16* __restrict__ out) {
+__global__ void llm_budget_embed_kernel(const float* budget, const __nv_bfloat16* w1, const __nv_bfloat16* w2, int H,
+                                        int D, __nv_bfloat16* out) {
   __shared__ double pe[256];
   __shared__ double hid[256];
   pdl_begin(false);

@@ -403,9 +403,8 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(SelectArgs a) {
 }
 
 // Compacts the per-sample kept lists: kept_off[b] = k_0 + ... + k_{b-1}.
-__global__ void compact_kernel(int B, const int* __restrict__ vis_off, const int* __restrict__ k,
-                               const int* __restrict__ kept_local, int* __restrict__ kept_idx,
-                               int* __restrict__ kept_off) {
+__global__ void compact_kernel(int B, const int* vis_off, const int* k, const int* kept_local, int* kept_idx,
+                               int* kept_off) {
   __shared__ int off;
   pdl_begin(false);
   const int b = blockIdx.x;

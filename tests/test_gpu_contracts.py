@@ -162,3 +162,23 @@ def test_e4m3_gemm_refuses_column_scales_it_cannot_read():
     svl.svl_gemm_e4m3(m.handle, A, a_scale[1:], B, b_scale[4:], M, N, K, C)  # rows: any float
     assert svl.svl_get_device_status(m.handle) == 0 and bool((C == K).all())
     m.close()
+
+
+def test_packs_chained_through_their_rows():
+    """A pack whose visual features are the rows another pack writes just before it."""
+    first, b, out = _packer(96, 98)
+    want = out["X"][:96].clone()
+    m = svl.GatedPrefill(TINY.dims, first.w, max_seq=1024)
+    b2 = synth.make_batch(TINY, 99, n_vis_list=[96], s_text_list=[5], keep_list=[96], device="cuda")
+    b2["vis"] = out["X"][:96]
+    got = m.run(b2, stages=("select", "pack"))
+    for _ in range(20):
+        out["X"].zero_()
+        got["X"].zero_()
+        torch.cuda.synchronize()
+        first.run(b, out=out, stages=("pack",))
+        m.run(b2, out=got, stages=("pack",))
+        torch.cuda.synchronize()
+        assert torch.equal(got["X"][:96], want)
+    m.close()
+    first.close()
