@@ -160,10 +160,10 @@ typedef struct svl_model svl_model;
  * weight pointers, allocates the device status word and the RoPE cos/sin
  * table (max_seq x d_head/2 float2, computed in double precision).
  * Returns SVL_ERR_UNSUPPORTED for dims outside the list above.
- * QKV and gate/up GEMMs run on clusters of two CTAs (256-row tiles, tcgen05
- * cta_group::2) for calls with room for 3,072 rows (t_cap) or more; the results
- * are the same. SVL_PAIR_GEMM in the environment overrides the rule: 0 never, 1
- * for every call with more than 32 rows.
+ * QKV and gate/up GEMMs run on clusters of two CTAs (two 128-row tiles of the
+ * same columns, tcgen05 cta_group::2) for calls with room for 3,072 rows (t_cap)
+ * or more; the results are the same. SVL_PAIR_GEMM in the environment overrides
+ * the rule: 0 never, 1 for every call with more than 32 rows.
  */
 svl_status svl_model_create(const svl_model_desc* desc, const svl_weights* weights, svl_model** out);
 void svl_model_destroy(svl_model* model);

@@ -23,7 +23,7 @@ struct svl_model {
   // every CTA of the persistent residual GEMM fits on the GPU at once, so
   // the shares of a K-split tail can wait for each other (else no split)
   bool ks_resident = false;
-  // QKV and gate/up on CTA pairs (256-row tiles, tcgen05 cta_group::2):
+  // QKV and gate/up on CTA pairs (two 128-row tiles of the same columns, tcgen05 cta_group::2):
   // clusters of two resident at once (0: single-CTA kernel); per layer the
   // q, k, v weights as tensor maps with 64-row boxes
   int pair_clusters = 0;
@@ -109,12 +109,16 @@ int round128(int x) { return (x + 127) & ~127; }
 
 constexpr int kMaxPrefillBatch = 4096;  // samples per prefill call
 
-// Row capacity from which the QKV and gate/up GEMMs run on CTA pairs. Their 256-row
-// tiles move a third less per MMA; with fewer rows, and with runs of gated samples
-// that end inside a tile, more of a tile is padding. Measured over one layer's MLP
-// and QKV + O at LLaVA-7B and Qwen2-VL-7B widths, all groups on and mixed masks: 4 to
-// 10 % faster at 3,072 rows and more, -2 to +6 % at 1,024 to 2,048, -4 % (MLP) at 320.
-// e4m3 models: the MLP of one layer with its quantisers at 5,400 rows 584 -> 548 us.
+// Row capacity from which the QKV and gate/up GEMMs run on CTA pairs, which move
+// a third less per MMA. The host knows the capacity only; the rows are what the
+// budgets leave of it. Forwards of four layers with room for 3,200 to 10,240 rows
+// at LLaVA-7B and Qwen2-VL-7B widths, single CTAs' time over pairs', every share of
+// the rows from 0.1 to 1: all groups on 1.01 to 1.10 but 0.98 at 5 and 7 row tiles
+// (an odd tile has no partner) and 0.91 at 3 (a tenth of 3,200 rows); gates scaled
+// with the budget 1.00 to 1.07, but 0.97 at a tenth; 64 samples with budgets and
+// gates of their own 1.08 to 1.11. e4m3 models 0.91, 0.95 to 1.08 and 1.08. With
+// room for 1,024 to 2,048 rows, one layer's MLP and QKV + O gained -2 to +6 %; at
+// 320 the MLP lost 4 %.
 constexpr int kPairRows = 3072;
 
 // Each call keeps its scratch at the start of the workspace: no data flows
@@ -317,11 +321,11 @@ svl_status launch(EpiKind kind, svl_model* m, int tag, const GemmParams& p, int6
 }
 
 // The same for the CTA-pair kernel (QKV, gate/up): up to pair_clusters
-// clusters of two, no more than the list's tiles.
+// clusters of two, no more than the list's pairs of tiles.
 svl_status launch_pair(EpiKind kind, svl_model* m, int tag, const GemmParams& p, int64_t tiles, cudaStream_t s) {
   if (tiles <= 0) return SVL_OK;
   Launch L(m, tag, s);
-  const int pairs = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(m->pair_clusters, tiles)));
+  const int pairs = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(m->pair_clusters, tiles / 2)));
   return launch_gemm_pair(kind, p, pairs, s, m->e4m3) == cudaSuccess ? SVL_OK : SVL_ERR_CUDA;
 }
 
@@ -914,17 +918,18 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
   sa.num_sms = m->num_sms;
   const bool thin_launch = t_cap <= kThinRows;
   const bool pair = m->pair_clusters > 0 && !thin_launch && t_cap >= m->pair_rows;
-  sa.nsparse_rows = pair ? 2 * kBM : kBM;
+  sa.pairs = pair ? 1 : 0;
   sa.qkv_step = thin_launch ? kBHalf : 2 * kBHalf;
-  sa.nsparse_wave = pair ? m->pair_clusters : m->num_sms;
+  sa.nsparse_wave = pair ? 2 * m->pair_clusters : m->num_sms;
   sa.A = d.n_heads;
   sa.Akv = d.n_kv_heads;
   sa.dh = dh;
   sa.D = d.d_model;
   sa.Di = d.d_ffn;
   {
-    const long long row_bytes = static_cast<long long>(sa.nsparse_rows) * d.d_model * (m->e4m3 ? 1 : 2);
-    sa.mband = static_cast<int>(std::max<long long>(1, kMBandBytes / row_bytes));
+    const long long tile_bytes = static_cast<long long>(kBM) * d.d_model * (m->e4m3 ? 1 : 2);
+    sa.mband = static_cast<int>(std::max<long long>(1, kMBandBytes / tile_bytes));
+    if (pair) sa.mband = std::max(2, sa.mband & ~1);  // whole pairs
   }
   sa.cu_seqlens = cu_seqlens;
   sa.layer_gate = layer_gate;

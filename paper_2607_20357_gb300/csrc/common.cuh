@@ -363,7 +363,7 @@ SVL_DEVINL void tmem_st32(uint32_t taddr, const uint32_t* r) {
 SVL_DEVINL void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // ---------------------------------------------------------------- CTA pairs (tcgen05 cta_group::2)
-// A cluster of two CTAs on two SMs computes one 256-row tile: the CTA of
+// A cluster of two CTAs on two SMs computes one product of 256 rows: the CTA of
 // even rank (the leader) issues the MMAs, which read A's rows 0-127 and half
 // of B from the leader's shared memory and A's rows 128-255 and the other half
 // of B from the peer's, at the same offsets, and write D rows 0-127 into the

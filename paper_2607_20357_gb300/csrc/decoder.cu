@@ -166,10 +166,10 @@ struct ColSet {
 // runs are written by one flat loop over the block's threads (a binary search
 // finds a tile's run). Returns the number of tiles.
 __device__ int emit_runs(ListShared& sh, int nrun, int4* tiles, int base, int cap, const ColSet& cs, bool kmask,
-                         uint32_t* status, int* s_scan, int bm, int nband, int mband) {
+                         uint32_t* status, int* s_scan, int nband, int mband) {
   const int n_nt = cs.total();
-  const int total =
-      prefix_offsets(sh, nrun, s_scan, [&](int i) { return ((sh.r1[i] - sh.r0[i] + bm - 1) / bm) * n_nt; });
+  const int total = prefix_offsets(
+      sh, nrun, s_scan, [&](int i) { return ((sh.r1[i] - sh.r0[i] + kBM_SCHED - 1) / kBM_SCHED) * n_nt; });
   for (int t = threadIdx.x; t < total; t += blockDim.x) {
     int lo = 0, hi = nrun;
     while (hi - lo > 1) {
@@ -177,7 +177,7 @@ __device__ int emit_runs(ListShared& sh, int nrun, int4* tiles, int base, int ca
       if (sh.off[mid] <= t) lo = mid; else hi = mid;
     }
     const int u = t - sh.off[lo], r0 = sh.r0[lo], r1 = sh.r1[lo];
-    const int mt = (r1 - r0 + bm - 1) / bm;
+    const int mt = (r1 - r0 + kBM_SCHED - 1) / kBM_SCHED;
     int mi, ni;
     if (mband > 0) {
       const int band = u / (mband * n_nt);
@@ -192,14 +192,52 @@ __device__ int emit_runs(ListShared& sh, int nrun, int4* tiles, int base, int ca
       mi = rem / bw;
       ni = band * nband + rem % bw;
     }
-    const int m0 = r0 + mi * bm;
+    const int m0 = r0 + mi * kBM_SCHED;
     const int idx = base + t;
     if (idx >= cap) {
       report(status, SVL_DEV_BAD_INDEX);
       continue;
     }
     const int2 n = cs.tile(ni);
-    tiles[idx] = make_int4(m0, min(m0 + bm, r1), n.x, n.y | (kmask ? static_cast<int>(sh.key[lo]) << 24 : 0));
+    tiles[idx] = make_int4(m0, min(m0 + kBM_SCHED, r1), n.x, n.y | (kmask ? static_cast<int>(sh.key[lo]) << 24 : 0));
+  }
+  __syncthreads();  // off, r0, r1 and key are reused by the caller
+  return total;
+}
+
+// The list of CTA pairs: entries 2i and 2i + 1 are the 128-row tiles of one
+// pair, which share their columns (the B operand) but need not adjoin. The
+// m-tiles of all runs are numbered through, so only the last of an odd number
+// has no partner (an entry without rows), and go in bands of `mband` (even)
+// m-tiles, each sweeping all n-tiles. (With 256 adjoining rows to a pair, every
+// run that ended in a pair's first half cost a whole pair: 16 samples with masks
+// of their own, 970 rows in all, a forward of four layers 1,125 us against 920
+// on single CTAs.) Returns the number of entries.
+__device__ int emit_pairs(ListShared& sh, int nrun, int4* tiles, int base, int cap, const ColSet& cs, uint32_t* status,
+                          int* s_scan, int mband) {
+  const int n_nt = cs.total();
+  const int mt =
+      prefix_offsets(sh, nrun, s_scan, [&](int i) { return (sh.r1[i] - sh.r0[i] + kBM_SCHED - 1) / kBM_SCHED; });
+  const int mt2 = mt + (mt & 1), total = mt2 * n_nt;
+  for (int t = threadIdx.x; t < total; t += blockDim.x) {
+    const int band = t / (mband * n_nt);
+    const int rem = t - band * mband * n_nt;
+    const int bh = min(mband, mt2 - band * mband);
+    const int ni = rem / bh, mi = band * mband + rem % bh;
+    const int m = min(mi, mt - 1);  // (the missing partner loads its neighbour's rows and stores none)
+    int lo = 0, hi = nrun;
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (sh.off[mid] <= m) lo = mid; else hi = mid;
+    }
+    const int m0 = sh.r0[lo] + (m - sh.off[lo]) * kBM_SCHED;
+    const int idx = base + t;
+    if (idx >= cap) {
+      report(status, SVL_DEV_BAD_INDEX);
+      continue;
+    }
+    const int2 n = cs.tile(ni);
+    tiles[idx] = make_int4(m0, mi < mt ? min(m0 + kBM_SCHED, sh.r1[lo]) : m0, n.x, n.y);
   }
   __syncthreads();  // off, r0, r1 and key are reused by the caller
   return total;
@@ -261,7 +299,8 @@ __device__ void build_list(const ScheduleArgs& a, int l, int kind, int* dyn) {
     // maximal row runs of samples where the block runs times its columns
     const bool qkv = kind == kListQkv;
     int4* tiles = qkv ? a.qkv_tiles + static_cast<size_t>(l) * a.qkv_cap : a.gu_tiles + static_cast<size_t>(l) * a.gu_cap;
-    const int cap = qkv ? a.qkv_cap : a.gu_cap;
+    // (CTA pairs: an even number of entries, whole pairs)
+    const int cap = (qkv ? a.qkv_cap : a.gu_cap) & (a.pairs ? ~1 : ~0);
     const int hq = (a.A / G) * a.dh, hk = (a.Akv / G) * a.dh;
     int off = 0;
     for (int j0 = 0; j0 < G;) {
@@ -277,7 +316,8 @@ __device__ void build_list(const ScheduleArgs& a, int l, int kind, int* dyn) {
         cs.set(0, j0 * (a.Di / G), (j1 + 1) * (a.Di / G));
       }
       const int nrun = find_runs(sh, j0, s_scan);
-      off += emit_runs(sh, nrun, tiles, off, cap, cs, false, a.status, s_scan, a.nsparse_rows, 0, a.mband);
+      off += a.pairs ? emit_pairs(sh, nrun, tiles, off, cap, cs, a.status, s_scan, a.mband)
+                     : emit_runs(sh, nrun, tiles, off, cap, cs, false, a.status, s_scan, 0, a.mband);
       j0 = j1 + 1;
     }
     off = min(off, cap);
@@ -293,7 +333,7 @@ __device__ void build_list(const ScheduleArgs& a, int l, int kind, int* dyn) {
     cs.step = 256;
     cs.set(0, 0, a.D);
     const int nrun = find_runs(sh, -1, s_scan);
-    int off = emit_runs(sh, nrun, tiles, 0, cap, cs, true, a.status, s_scan, kBM_SCHED, o ? kNBandO : kNBand, 0);
+    int off = emit_runs(sh, nrun, tiles, 0, cap, cs, true, a.status, s_scan, o ? kNBandO : kNBand, 0);
     off = split_k_tail(tiles, min(off, cap), cap, a.num_sms, a.ks_units,
                        a.ks_info + static_cast<size_t>(l) * 8 + (o ? 0 : 4));
     if (tid == 0) (o ? a.o_count : a.dn_count)[l] = off;

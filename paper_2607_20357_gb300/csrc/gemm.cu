@@ -1259,14 +1259,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
 }
 
 // ------------------------------------------------------------------ CTA-pair kernel
-// The same GEMM on 256-row tiles computed by a cluster of two CTAs on two SMs
-// (tcgen05 cta_group::2). Each CTA loads its 128 rows of A and half of B (the
-// first or the second N/2 rows of the tile's B, or the gate or the up rows of
-// a gate/up tile) into its own shared memory; the leader (cluster rank 0)
-// issues the MMAs, which read both CTAs' halves and write D rows 0-127 into
-// the leader's tensor memory and rows 128-255 into the peer's. Per SM and K
-// block this moves 32 KB through shared memory for a 128 x N product where the
-// single-CTA kernel moves 48 KB, which is what caps that kernel's tensor pipe.
+// The same GEMM on two 128-row tiles of the same columns at a time, computed by
+// a cluster of two CTAs on two SMs (tcgen05 cta_group::2): list entries 2i and
+// 2i + 1, one per CTA (an odd last tile's partner has no rows). Each CTA loads
+// its 128 rows of A and half of B (the first or the second N/2 rows of the
+// tiles' B, or the gate or the up rows of a gate/up tile) into its own shared
+// memory; the leader (cluster rank 0) issues the MMAs, which read both CTAs'
+// halves and write D rows 0-127 into the leader's tensor memory and rows
+// 128-255 into the peer's. Per SM and K block this moves 32 KB through shared
+// memory for a 128 x N product where the single-CTA kernel moves 48 KB, which is
+// what caps that kernel's tensor pipe.
 //
 //   full[s]    leader only: both CTAs' TMA loads of stage s (the leader posts
 //              the byte count of both, the peer's loads complete on it);
@@ -1286,7 +1288,15 @@ constexpr int kPairStageBytes = kABytes + kPairBBytes;
 constexpr int kPairSmem = kPairStages * kPairStageBytes + 1024 + 1024 + kResidStageBytes;
 static_assert(kPairSmem <= 232448, "shared memory per CTA");
 
-// MMA N of a pair tile: gate/up tiles are 128 gate + 128 up rows; others
+// The list entries of CTA pairs: this CTA's (its pair's first or second), and
+// the same for all roles of both CTAs, whole pairs only.
+SVL_DEVINL Work load_pair_work(const GemmParams& p, int first) {
+  Work w = load_work(p, first);
+  w.n &= ~1;
+  return w;
+}
+
+// MMA N of a pair's tiles: gate/up tiles are 128 gate + 128 up rows; others
 // round their columns up to 128 or 256 (each CTA holds N / 2 rows of B).
 SVL_DEVINL int pair_n(const GemmParams& p, const TileInfo& ti) {
   if (p.b_split) return 2 * kBHalf;
@@ -1298,8 +1308,7 @@ SVL_DEVINL int pair_n(const GemmParams& p, const TileInfo& ti) {
 template <int OP, bool F8>
 SVL_DEVINL void pair_producer(const GemmParams& p, uint8_t* stages, uint64_t* full, uint64_t* empty, uint32_t rank,
                               volatile int* abort) {
-  const int npairs = gridDim.x >> 1, pair = blockIdx.x >> 1;
-  Work wk = load_work(p, pair);
+  Work wk = load_pair_work(p, blockIdx.x);
   constexpr int BK = F8 ? kBK8 : kBK;
   const int nkb = p.K / BK, kgb = p.kgroup / BK;
   int s = 0;
@@ -1310,9 +1319,8 @@ SVL_DEVINL void pair_producer(const GemmParams& p, uint8_t* stages, uint64_t* fu
       ph ^= 1;
     }
   };
-  for (int t = pair; t < wk.n; t += npairs) {
-    const TileInfo ti = get_tile(p, wk, t, npairs);
-    if (!ti.valid) continue;
+  for (int t = blockIdx.x; t < wk.n; t += gridDim.x) {
+    const TileInfo ti = get_tile(p, wk, t, gridDim.x);
     const int brows = pair_n(p, ti) / 2, box = p.b_box_rows ? p.b_box_rows : kBHalf;
     const CUtensorMap* mb = p.b_split ? &p.mapB[rank] : &p.mapB[ti.mat];
     const int by = p.b_split ? ti.n0 : ti.n0 + static_cast<int>(rank) * brows;
@@ -1329,7 +1337,7 @@ SVL_DEVINL void pair_producer(const GemmParams& p, uint8_t* stages, uint64_t* fu
       if (rank == 0) mbar_arrive_expect_tx(&full[s], bytes);
       const uint32_t fb = mapa_shared(&full[s], 0);
       if constexpr (OP == 0) {
-        tma_load_2d_pair(sa, &p.mapA, fb, w.kb * BK, ti.m0 + static_cast<int>(rank) * kBM);
+        tma_load_2d_pair(sa, &p.mapA, fb, w.kb * BK, ti.m0);
       } else {
         for (int r = 0; r < brows; r += box)
           tma_load_2d_pair(sa + kABytes + r * 128, mb, fb, w.kb * BK, by + r);
@@ -1350,16 +1358,14 @@ SVL_DEVINL void pair_producer(const GemmParams& p, uint8_t* stages, uint64_t* fu
 template <bool F8>
 SVL_DEVINL void pair_mma(const GemmParams& p, uint8_t* stages, uint64_t* full, uint64_t* empty, uint64_t* tfull,
                          uint64_t* tempty, uint32_t tmem, volatile int* abort) {
-  const int npairs = gridDim.x >> 1, pair = blockIdx.x >> 1;
-  Work wk = load_work(p, pair);
+  Work wk = load_pair_work(p, blockIdx.x);
   constexpr int BK = F8 ? kBK8 : kBK;
   const int nkb = p.K / BK, kgb = p.kgroup / BK;
   const uint64_t da0 = smem_desc_sw128(smem_u32(stages)), db0 = smem_desc_sw128(smem_u32(stages) + kABytes);
   int s = 0, it = 0;
   uint32_t ph = 0;
-  for (int t = pair; t < wk.n; t += npairs) {
-    const TileInfo ti = get_tile(p, wk, t, npairs);
-    if (!ti.valid) continue;
+  for (int t = blockIdx.x; t < wk.n; t += gridDim.x) {
+    const TileInfo ti = get_tile(p, wk, t, gridDim.x);
     const int acc = it & 1;
     const uint32_t aph = (it >> 1) & 1;
     if (!mbar_wait(&tempty[acc], aph ^ 1, abort)) {
@@ -1402,17 +1408,14 @@ SVL_DEVINL void pair_mma(const GemmParams& p, uint8_t* stages, uint64_t* full, u
 template <int KIND, bool F8>
 SVL_DEVINL void pair_epilogue(const GemmParams& p, uint64_t* tfull, uint64_t* tempty, uint32_t tmem, uint32_t rank,
                               volatile int* abort, uint8_t* rstage) {
-  const int npairs = gridDim.x >> 1, pair = blockIdx.x >> 1;
-  Work wk = load_work(p, pair);
+  Work wk = load_pair_work(p, blockIdx.x);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = warp & 3;  // TMEM lane quarter this warp may access
   uint8_t* wst = rstage + q * 2 * kResidChunk;
   uint32_t sbuf = 0;
   int it = 0;
-  for (int t = pair; t < wk.n; t += npairs) {
-    TileInfo ti = get_tile(p, wk, t, npairs);
-    if (!ti.valid) continue;
-    ti.m0 += static_cast<int>(rank) * kBM;  // this CTA's rows
+  for (int t = blockIdx.x; t < wk.n; t += gridDim.x) {
+    const TileInfo ti = get_tile(p, wk, t, gridDim.x);
     const int acc = it & 1;
     const uint32_t aph = (it >> 1) & 1;
     const bool staged = p.stage_tma && (ti.ncols & 63) == 0 && (ti.n0 & 7) == 0 && ti.m0 + q * 32 + 32 <= ti.m_end;

@@ -133,10 +133,11 @@ struct GemmParams {
 cudaError_t launch_gemm(EpiKind kind, const GemmParams& p, int grid, cudaStream_t stream, bool e4m3 = false,
                         bool thin = false);
 
-// The gated QKV / gate-up GEMM on 256-row tiles by clusters of two CTAs
-// (tcgen05 cta_group::2): `pairs` clusters walk the tile list (tiles of up to
-// 256 rows), mapA has 128-row boxes, mapB b_box_rows (0: 128; 64 where tiles may
-// have 128 columns or fewer).
+// The gated QKV / gate-up GEMM on clusters of two CTAs (tcgen05 cta_group::2):
+// `pairs` clusters walk a list whose entries 2i and 2i + 1 are the pair's tiles,
+// of the same columns and up to 128 rows each (the second may have none). mapA
+// has 128-row boxes, mapB b_box_rows (0: 128; 64 where tiles may have 128
+// columns or fewer).
 cudaError_t launch_gemm_pair(EpiKind kind, const GemmParams& p, int pairs, cudaStream_t stream, bool e4m3 = false);
 // Clusters of two of the pair kernel that can be resident at once (0 if the
 // query fails).

@@ -199,10 +199,10 @@ enum ListKind : int { kListQkv = 0, kListO = 1, kListDown = 2, kListGateUp = 3, 
 struct ScheduleArgs {
   int B, L, G, P;
   int num_sms;              // CTAs of the persistent GEMM (one wave of tiles)
-  int nsparse_rows;         // rows per tile of the QKV and gate/up lists (128, or 256 for CTA pairs)
+  int pairs;                // QKV and gate/up run on CTA pairs: their lists hold two entries per pair
   int qkv_step;             // columns per QKV tile (256; 128 for THIN launches)
-  int nsparse_wave;         // tiles of those lists that run at once (CTAs, or CTA pairs)
-  int mband;                // m-tiles per raster band of those lists (see kMBandBytes)
+  int nsparse_wave;         // entries of those lists that run at once (the CTAs, in pairs or not)
+  int mband;                // m-tiles per raster band of those lists (see kMBandBytes; even for pairs)
   int A, Akv, dh, D, Di;
   const int* cu_seqlens;
   const uint8_t* layer_gate;

@@ -281,3 +281,41 @@ def test_pack_of_many_samples(B):
     assert torch.equal(out["X"][:T][~visual], w["embed"][b["text_ids"].long()])
     assert svl.svl_get_device_status(m.handle) == 0
     m.close()
+
+
+PAIR_DIMS = {"llava": LLAVA.dims, "qwen": synth.WORKLOADS["qwen"].dims, "head64": TINY.dims}
+
+
+@pytest.mark.parametrize("fmt", [svl.SVL_GEMM_BF16, svl.SVL_GEMM_E4M3], ids=["bf16", "e4m3"])
+@pytest.mark.parametrize("lengths", [[1, 129, 255, 257, 40, 3, 128, 300], [33], [384], [60] * 16, [500] * 7],
+                         ids=["ragged", "one", "odd", "short", "long"])
+@pytest.mark.parametrize("name", list(PAIR_DIMS))
+def test_cta_pairs_with_masks(name, lengths, fmt, monkeypatch):
+    """Pairs against single CTAs where each sample has group masks of its own (one sample skips the layer): runs that end
+    inside a pair, tiles of different runs in one pair, an odd tile without a partner, K and V tiles of one KV head
+    (128 or 64 columns). Outputs start as NaN: exactly the active columns are written, with the same bits."""
+    dims = synth.reduced(PAIR_DIMS[name], n_layers=1, vocab=512)
+    T, B, G = sum(lengths), len(lengths), dims.n_groups
+    g = torch.Generator().manual_seed(B + T)
+    gg = (torch.rand(B, 1, G, generator=g) < 0.6).to(torch.uint8)
+    gg[0] = 1
+    if B > 2:
+        gg[2] = 0
+    on = torch.repeat_interleave(gg[:, 0].bool(), torch.tensor(lengths), 0).cuda()  # [T, G]
+    got = []
+    for env in ("0", "1"):
+        monkeypatch.setenv("SVL_PAIR_GEMM", env)
+        s = _Stage(dims, lengths, 65, gemm_format=fmt)
+        s.gg = gg.cuda()
+        X = _rand(T, dims.d_model, seed=66)
+        nan = lambda *shape: torch.full(shape, float("nan"), dtype=torch.bfloat16, device="cuda")  # noqa: E731
+        q, k, h = nan(T, dims.n_heads * dims.d_head), nan(T, dims.d_kv), nan(T, dims.d_ffn)
+        vt = nan(dims.d_kv, (T + 7) // 8 * 8)
+        s.run(svl.SVL_LAYER_QKV, X, q=q, k=k, vt=vt)
+        s.run(svl.SVL_LAYER_GATEUP, X, h=h)
+        got.append((q, k, vt[:, :T].T, h))
+        assert bool(vt[:, T:].isnan().all())
+        s.m.close()
+    for a, b in zip(*got):
+        assert torch.equal(a.contiguous().view(torch.int16), b.contiguous().view(torch.int16))
+        assert torch.equal(~b.isnan(), torch.repeat_interleave(on, b.shape[1] // G, 1))
