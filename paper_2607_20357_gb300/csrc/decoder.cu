@@ -343,13 +343,18 @@ __device__ void build_list(const ScheduleArgs& a, int l, int kind, int* dyn) {
     // Attention items: per active sample and active head, blocks of kAttnQ
     // queries, head by head and latest block first: the kernel takes units from
     // the front of the list, so one head's blocks run at about the same time
-    // and share its keys in L2. A block's work grows with its index, and with a
-    // sample of over kAttnLong rows the largest units of the last heads would
-    // start last (40 us units of 2,300 rows; the CTAs ended 30 us apart): then
-    // the latest blocks of all heads come first, in chunks of samples whose keys
-    // and values stay in L2. Two samples of 2.3k rows: 91.5 us head by head,
-    // 88.3 by size; 16 of up to 640 rows: 43.2 and 44.9. Beyond kAttnSorted
-    // samples the units are many and the order does not matter.
+    // and share its keys in L2. A block's work grows with its index, so with few
+    // long samples the largest units of the last heads would start last and the
+    // CTAs end far apart: then the latest blocks of all heads come first, in
+    // chunks of samples whose keys and values stay in L2. With many units the
+    // spread at the end is small and the shared keys count for more.
+    // Stage calls at LLaVA-7B / Qwen2-VL-7B widths, head by head's time over by
+    // size: one sample of 2,300 rows 1.23 / 1.25, two of 3,000 1.08 / 1.12, four of
+    // 2,300 1.03 / 1.09, six of 1,500 1.02 / 1.06, eight of 1,024 to 3,000 1.00 to 1.02,
+    // one of 2,300 among seven short ones 1.09 / 1.06. The other way round: ten of
+    // 1,024 0.99, sixteen of 769 0.96, of 2,500 0.99, one of 2,300 among 15 short
+    // ones 0.95 / 0.97, 64 of 1,024 0.91; eight of 900 0.97, four of 800 0.95 / 1.00,
+    // one of 900 0.91 / 0.98 (the short ones within the timer's 1 us).
     int4* items = a.attn_items + static_cast<size_t>(l) * a.attn_cap;
     const int hpg = a.A / G;
     const int total = prefix_offsets(sh, sh.n, s_scan, [&](int i) {

@@ -24,8 +24,8 @@ constexpr int kNBandO = 16;       // O list (16 n-tiles of 256 x 4,096 weights: 
 // On CTA pairs bands of 20, 27 and 60 MB were no faster (four layers, 10,240
 // rows: 10.99, 11.02 and 11.24 ms against 10.95 to 10.98).
 constexpr long long kMBandBytes = 40ll << 20;
-constexpr int kAttnSorted = 64;                    // samples up to which attention items may be ordered by size ...
-constexpr int kAttnLong = 768;                     // ... which they are when one has more rows than this
+constexpr int kAttnSorted = 8;    // attention items are ordered by size for at most this many samples ...
+constexpr int kAttnLong = 1000;   // ... of which one has more rows than this (measured: see build_list)
 constexpr long long kAttnChunkBytes = 40ll << 20;  // keys and values of the samples ordered together
 constexpr int kBM_SCHED = 128;    // tile rows (the GEMM's M)
 

@@ -319,3 +319,8 @@ def test_cta_pairs_with_masks(name, lengths, fmt, monkeypatch):
     for a, b in zip(*got):
         assert torch.equal(a.contiguous().view(torch.int16), b.contiguous().view(torch.int16))
         assert torch.equal(~b.isnan(), torch.repeat_interleave(on, b.shape[1] // G, 1))
+
+@pytest.mark.parametrize("lengths", [[1000, 1000], [1001, 20], [1001] + [30] * 7, [1001] + [30] * 8])
+def test_attention_order_at_the_edges_of_its_rule(lengths):
+    """At most eight samples, one of over 1,000 rows: by size; one row fewer or one sample more: head by head."""
+    test_attention_items_by_size_and_head_by_head(lengths)
