@@ -398,8 +398,7 @@ class GatedPrefill:
                             opt("kap_w2"), opt("gate_w"), opt("gate_c"))
         self.handle = svl_model_create(self.desc, self._wts)
         self._ws = None
-        self._ws_key = None
-        self._ws_need = 0
+        self._ws_size = None
 
     def close(self):
         if self.handle:
@@ -414,12 +413,13 @@ class GatedPrefill:
 
     def workspace(self, B, n_vis, n_text, device="cuda", stages=("select", "pack", "prefill")):
         key = (B, n_vis, n_text, tuple(stages))
-        if key != self._ws_key:  # the sizes of the last call
-            self._ws_key, self._ws_need = key, svl_workspace_size_for(self.handle, stages, B, n_vis, n_text)
-        need = self._ws_need
-        if self._ws is None or self._ws.numel() < need:
-            self._ws = torch.empty(need, dtype=torch.uint8, device=device)
-        return self._ws, self._ws.numel()
+        size = self._ws_size  # (sizes, bytes) of the last call: one object, so that threads see either as a whole
+        if size is None or size[0] != key:
+            size = self._ws_size = (key, svl_workspace_size_for(self.handle, stages, B, n_vis, n_text))
+        ws = self._ws
+        if ws is None or ws.numel() < size[1]:
+            ws = self._ws = torch.empty(size[1], dtype=torch.uint8, device=device)
+        return ws, ws.numel()
 
     def alloc_outputs(self, batch: dict, logits_mode: int = SVL_LOGITS_LAST):
         d = self.dims

@@ -130,3 +130,26 @@ def test_ksplit_plan_launch_rule(svl_lib):
                         want = sp if sp >= 2 else 1
                     assert plan(tiles, cap, n, 1, units) == want, (n, tiles, units, cap)
                     assert plan(tiles, cap, n, 0, units) == 1
+
+
+def test_workspace_is_sized_for_its_own_call(monkeypatch):
+    """Another thread's call may come between any two steps of a call: here one runs when the bytes of a call have been
+    stored on the model. Every call must still get a workspace of its own size."""
+    monkeypatch.setattr(svl, "svl_workspace_size_for", lambda h, stages, B, nv, nt: 1000 * B)
+
+    class Model(svl.GatedPrefill):
+        def __init__(self):
+            self.handle = None
+            self._ws = self._ws_size = None
+            self.calls = []
+
+        def __setattr__(self, name, value):
+            super().__setattr__(name, value)
+            if name == "_ws_size" and getattr(self, "calls", None):
+                self.workspace(self.calls.pop(), 0, 0, "cpu")
+
+    for B, between in ((7, [2]), (7, [2, 3]), (2, [7]), (5, [5, 1])):
+        m = Model()
+        m.calls = between
+        ws, n = m.workspace(B, 0, 0, "cpu")
+        assert n == ws.numel() >= 1000 * B
