@@ -350,10 +350,9 @@ svl_status svl_decode_step(svl_model* model, int32_t B, const int32_t* tokens, v
  *  for a workspace -- code running during CUDA stream capture (where
  *  cudaMalloc is not permitted), plugins whose host framework keeps all
  *  device memory for its own allocator, real-time paths that must not wait
- *  in an allocator. It allocates nothing; its scratch (budget embeddings and
- *  per-sample kept lists) lives in one fixed 512 KiB device array inside the
- *  library, present on every GPU that loads the library until the process
- *  exits. Limits: B <= 256, n_vis_total <= 65536, h_ctrl <= 256; larger
+ *  in an allocator. It allocates nothing; its scratch (budget embeddings)
+ *  lives in one fixed 256 KiB device array inside the library, present on
+ *  every GPU that loads the library until the process exits. Limits: B <= 256, n_vis_total <= 65536, h_ctrl <= 256; larger
  *  calls return SVL_ERR_SHAPE and launch nothing. Outputs and their meaning
  *  are those of svl_score_select. The first call on a device looks up the
  *  array's device address (cudaGetSymbolAddress, once per device, with that

@@ -1347,7 +1347,6 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
 
   // final norm + LM head
   na.gain = static_cast<const __nv_bfloat16*>(m->w.final_norm);
-  na.act = nullptr;
   GemmParams p = base_params(m);
   if (logits_mode == SVL_LOGITS_LAST) {
     const int n_pad = ((B + 15) / 16) * 16;
@@ -1730,17 +1729,16 @@ svl_status svl_get_device_status(svl_model* m, void* stream, uint32_t* code) {
 // not allowed there), plugins whose host framework has already reserved the
 // device's memory for its own allocator and gives them none, or real-time
 // paths that must not block in the allocator. For them this entry point keeps
-// its scratch -- the budget embeddings e_b and the per-sample kept lists -- in
-// one fixed array in device memory that is part of the library image. Every
-// GPU that loads the library holds the array until the process exits.
+// its scratch -- the budget embeddings e_b (with gates given, the selection
+// writes its indices to their final place) -- in one fixed array in device
+// memory that is part of the library image. Every GPU that loads the library
+// holds the array until the process exits.
 namespace {
 
 constexpr int kNoAllocMaxBatch = 256;     // samples per call
 constexpr int kNoAllocMaxHctrl = 256;     // token-controller hidden width
-constexpr int kNoAllocMaxVis = 65536;     // visual tokens per call (all samples)
-constexpr size_t kNoAllocEbBytes = sizeof(float) * kNoAllocMaxBatch * kNoAllocMaxHctrl;   // 256 KiB
-constexpr size_t kNoAllocListBytes = sizeof(int) * kNoAllocMaxVis;                        // 256 KiB
-constexpr size_t kNoAllocScratchBytes = kNoAllocEbBytes + kNoAllocListBytes;              // 512 KiB
+constexpr int kNoAllocMaxVis = 65536;     // visual tokens per call (all samples; a limit of the interface, no scratch)
+constexpr size_t kNoAllocScratchBytes = sizeof(float) * kNoAllocMaxBatch * kNoAllocMaxHctrl;  // 256 KiB
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
 
@@ -1777,14 +1775,12 @@ extern "C" svl_status svl_score_select_noalloc(svl_model* m, int32_t B, int32_t 
   svl_status st = check_select(m, c);
   if (st != SVL_OK) return st;
   if (B > kNoAllocMaxBatch || n_vis_total > kNoAllocMaxVis || m->d.h_ctrl > kNoAllocMaxHctrl)
-    return SVL_ERR_SHAPE;  // beyond the fixed scratch array
+    return SVL_ERR_SHAPE;  // beyond the stated limits
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev != m->device) return SVL_ERR_INVALID_ARG;
   void* scratch = nullptr;
   if ((st = noalloc_scratch(&scratch)) != SVL_OK) return st;
   // Every scratch element read is written earlier in the same call, so nothing
   // has to be cleared first.
-  return run_select(m, c, static_cast<float*>(scratch),
-                    reinterpret_cast<int*>(static_cast<unsigned char*>(scratch) + kNoAllocEbBytes),
-                    static_cast<cudaStream_t>(stream));
+  return run_select(m, c, static_cast<float*>(scratch), nullptr, static_cast<cudaStream_t>(stream));
 }

@@ -660,7 +660,6 @@ __global__ void rmsnorm_kernel(NormArgs a) {
   const int r = blockIdx.x * (blockDim.x >> 5) + warp;
   const int T = a.cu_seqlens[a.B];
   if (r >= T || r >= a.t_cap) return;
-  if (a.act && !a.act[find_sample(a.cu_seqlens, a.B, r)]) return;
   norm_row(a.X + static_cast<size_t>(r) * a.D, a.gain, a.Y + static_cast<size_t>(r) * a.D, a.D, a.eps, lane);
 }
 

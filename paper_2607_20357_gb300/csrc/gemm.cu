@@ -1279,10 +1279,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
 // set-up and before the tensor memory is released) are reached by every thread
 // of both CTAs on every path; each producer first waits for the release of its
 // last stages, so no MMA completion can arrive after its CTA has exited.
-#ifndef SVL_PAIR_STAGES
-#define SVL_PAIR_STAGES 6
-#endif
-constexpr int kPairStages = SVL_PAIR_STAGES;
+constexpr int kPairStages = 6;
 constexpr int kPairBBytes = kBHalf * kBK * 2;        // up to 128 B rows per CTA
 constexpr int kPairStageBytes = kABytes + kPairBBytes;
 constexpr int kPairSmem = kPairStages * kPairStageBytes + 1024 + 1024 + kResidStageBytes;

@@ -24,7 +24,6 @@ constexpr int kGemmThreads = 224;  // warp 0 TMA of B, warp 1 MMA + TMEM, warps 
 constexpr int kPairThreads = 224;  // CTA pairs: the same roles
 constexpr int kAccCols = 256;      // fp32 columns per accumulator
 constexpr int kTmemCols = 512;     // two accumulators (epilogue overlaps the next tile)
-constexpr int kGemmSmem = kStages * kStageBytes + 1024 /*align*/ + 256 /*barriers*/;
 constexpr int kResidChunk = 32 * 128;             // one warp's 32 rows x 64 columns of bf16 (staged epilogues)
 constexpr int kResidStageBytes = 4 * 2 * kResidChunk;  // two chunk buffers per epilogue warp
 

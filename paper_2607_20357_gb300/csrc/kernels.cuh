@@ -294,7 +294,6 @@ struct NormArgs {
   const __nv_bfloat16* gain;
   __nv_bfloat16* Y;
   const int* cu_seqlens;
-  const uint8_t* act;     // [B] or nullptr (every row)
 };
 void launch_rmsnorm(const NormArgs& a, cudaStream_t s);
 
