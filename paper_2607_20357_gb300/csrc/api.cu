@@ -1227,6 +1227,7 @@ svl_status prefill_impl(svl_model* m, int32_t B, int32_t t_cap, void* X, const i
       da.out = ao;
       Launch L1(m, SVL_TAG_ATTENTION, s);
       da.late = !f8;
+      da.num_sms = m->num_sms;
       next_launch(da.late);
       if (launch_decode_attn(da, s) != cudaSuccess) return SVL_ERR_CUDA;
     } else {

@@ -70,9 +70,10 @@ void launch_kv_store(const KvArgs& a, int t_cap, cudaStream_t s) {
 //  - one query head per KV head: a block per head, a warp per run, and the V
 //    rows are requested into registers before the scores are formed;
 //  - several (GQA): a cluster of kRuns blocks per KV head, a block per run, a
-//    warp per query head, so the cache is read once for all of them; 128
-//    positions at a time (the score chains of four tiles side by side) while
-//    the next 128 load, and the runs meet through distributed shared memory.
+//    warp per query head, so the cache is read once for all of them; 32 or 128
+//    positions at a time (the score chains of four tiles side by side; the rule
+//    is at launch_dec) while the next ones load, and the runs meet through
+//    distributed shared memory.
 constexpr int kRuns = 8;
 constexpr int kDecThreads = kRuns * 32;
 
@@ -317,14 +318,13 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(DecAttnArgs
   }
 }
 
-constexpr int kGqaTiles = 4;  // tiles per step (16 KB each at d_head 128); two steps in shared memory
-
 // Several query heads per KV head: cluster of kRuns blocks, block = run, warp
-// = query head; blockIdx.y = KV head times passes of kRuns query heads.
-template <int DH>
-__global__ void __launch_bounds__(kDecThreads, 1) decode_attn_gqa_kernel(DecAttnArgs a) {
+// = query head; blockIdx.y = KV head times passes of kRuns query heads. A step is
+// KT tiles of 32 positions (16 KB each at d_head 128); two steps in shared memory.
+template <int DH, int KT>
+__global__ void __launch_bounds__(kDecThreads, KT == 1 ? 3 : 1) decode_attn_gqa_kernel(DecAttnArgs a) {
   constexpr int PER = DH / 32, CH = DH / 8, TB = 32 * DH * 2;
-  extern __shared__ __align__(128) uint8_t dec_smem[];  // [2][kGqaTiles] of 32 K rows and 32 V rows
+  extern __shared__ __align__(128) uint8_t dec_smem[];  // [2][KT] of 32 K rows and 32 V rows
   __shared__ __align__(16) float sq[kRuns][DH];
   __shared__ float sm_m[kRuns], sm_l[kRuns];  // per query head, read by the cluster
   __shared__ float sm_o[kRuns][DH];
@@ -348,8 +348,8 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_attn_gqa_kernel(DecAttn
   const int n = len + 1, per_run = (n + kRuns - 1) / kRuns;
   const int p_begin = run * per_run, p_end = min(n, p_begin + per_run);
   auto request = [&](int p0, int buf) {  // the tiles of one step into half `buf` of the ring
-    uint8_t* tiles = dec_smem + buf * kGqaTiles * 2 * TB;
-    for (int idx = tid; idx < 32 * kGqaTiles * CH; idx += kDecThreads) {
+    uint8_t* tiles = dec_smem + buf * KT * 2 * TB;
+    for (int idx = tid; idx < 32 * KT * CH; idx += kDecThreads) {
       const int row = idx / CH, c = idx % CH, p = p0 + row;
       if (p >= p_end) break;  // rows only grow
       uint8_t* kt = tiles + (row >> 5) * 2 * TB + (row & 31) * DH * 2;
@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_attn_gqa_kernel(DecAttn
     }
     cp_async_commit();
     const int jn = len - p0;  // the new token's V row (transposed in this step's V^T)
-    if (jn >= 0 && jn < 32 * kGqaTiles && len < p_end && tid < DH)
+    if (jn >= 0 && jn < 32 * KT && len < p_end && tid < DH)
       reinterpret_cast<__nv_bfloat16*>(tiles + (jn >> 5) * 2 * TB + TB)[(jn & 31) * DH + tid] =
           vnew[static_cast<size_t>(tid) * a.t_pad];
   };
@@ -375,21 +375,21 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_attn_gqa_kernel(DecAttn
 #pragma unroll
   for (int i = 0; i < PER; ++i) r.o[i] = 0.f;
   int buf = 0;
-  for (int p0 = p_begin; p0 < p_end; p0 += 32 * kGqaTiles) {
+  for (int p0 = p_begin; p0 < p_end; p0 += 32 * KT) {
     cp_async_wait<0>();
     __syncthreads();  // this step's tiles have landed, and the previous step's are read
-    request(p0 + 32 * kGqaTiles, buf ^ 1);
+    request(p0 + 32 * KT, buf ^ 1);
     if (warp < nh) {
-      const uint8_t* kt = dec_smem + buf * kGqaTiles * 2 * TB;
-      float sc[kGqaTiles], mx[kGqaTiles];
-      tile_scores<DH, kGqaTiles>(kt, 2 * TB, sq[warp], lane, sc);
+      const uint8_t* kt = dec_smem + buf * KT * 2 * TB;
+      float sc[KT], mx[KT];
+      tile_scores<DH, KT>(kt, 2 * TB, sq[warp], lane, sc);
 #pragma unroll
-      for (int t = 0; t < kGqaTiles; ++t) {
+      for (int t = 0; t < KT; ++t) {
         if (p0 + 32 * t + lane >= p_end) sc[t] = -INFINITY;
         mx[t] = warp_max(sc[t]);
       }
 #pragma unroll
-      for (int t = 0; t < kGqaTiles; ++t) {
+      for (int t = 0; t < KT; ++t) {
         const int n = p_end - (p0 + 32 * t);
         if (n <= 0) break;
         const float e = fold_scores<PER>(r, sc[t], mx[t], lane < n);
@@ -432,16 +432,31 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_attn_gqa_kernel(DecAttn
   cluster_sync();  // the others have read this block's run
 }
 
+template <int DH, int KT>
+static cudaError_t launch_gqa(const DecAttnArgs& a, int kv_blocks, cudaStream_t s) {
+  constexpr int ring = 2 * KT * 2 * 32 * DH * 2;
+  const cudaError_t e =
+      cudaFuncSetAttribute(decode_attn_gqa_kernel<DH, KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, ring);
+  if (e != cudaSuccess) return e;
+  return launch_pdl_cluster(decode_attn_gqa_kernel<DH, KT>, dim3(kRuns, kv_blocks, a.B), kDecThreads, ring, kRuns, s,
+                            a);
+}
+
+// Steps of four tiles while the rings of all blocks find room at once in 128 KB
+// per SM: every block has its SM (nearly) to itself then, and what counts is how
+// much of its run is in flight. With more blocks, steps of one tile: four blocks
+// fit on an SM and cover each other's latency. A decode step of four layers at
+// Qwen2-VL-7B widths (four KV heads), one tile / four: 1 sample of 2,000 rows
+// 579 / 522 us, 4 of 1,000 542 / 536, 8 of 30 475 / 520 and of 2,000 622 / 656, 64 of
+// 200 669 / 1,018, 256 of 30 1,012 / 2,244 (two tiles: 542, 507, 479, 561, 756, 1,334).
 template <int DH>
 static cudaError_t launch_dec(const DecAttnArgs& a, cudaStream_t s) {
   const int grp = a.A / a.Akv;
   if (grp > 1) {
-    constexpr int ring = 2 * kGqaTiles * 2 * 32 * DH * 2;
-    const cudaError_t e =
-        cudaFuncSetAttribute(decode_attn_gqa_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, ring);
-    if (e != cudaSuccess) return e;
-    return launch_pdl_cluster(decode_attn_gqa_kernel<DH>, dim3(kRuns, a.Akv * ((grp + kRuns - 1) / kRuns), a.B),
-                              kDecThreads, ring, kRuns, s, a);
+    const int kv_blocks = a.Akv * ((grp + kRuns - 1) / kRuns);
+    const int64_t rings = static_cast<int64_t>(kRuns) * kv_blocks * a.B * (4 * 2 * 2 * 32 * DH * 2);
+    return rings <= static_cast<int64_t>(a.num_sms) * (128 << 10) ? launch_gqa<DH, 4>(a, kv_blocks, s)
+                                                                  : launch_gqa<DH, 1>(a, kv_blocks, s);
   }
   constexpr int smem = kRuns * 32 * DH * 2;
   const cudaError_t e =

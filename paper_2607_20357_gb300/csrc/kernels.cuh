@@ -187,6 +187,7 @@ struct DecAttnArgs {
   __nv_bfloat16* v_cache;
   __nv_bfloat16* out;       // [B, A*dh]
   bool late;                // see QuantArgs
+  int num_sms;
 };
 cudaError_t launch_decode_attn(const DecAttnArgs& a, cudaStream_t s);
 cudaError_t launch_decode_finish(int B, int V, const float* logits, int* next_token, int* cache_len, int max_len,

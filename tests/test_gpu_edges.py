@@ -324,3 +324,33 @@ def test_cta_pairs_with_masks(name, lengths, fmt, monkeypatch):
 def test_attention_order_at_the_edges_of_its_rule(lengths):
     """At most eight samples, one of over 1,000 rows: by size; one row fewer or one sample more: head by head."""
     test_attention_items_by_size_and_head_by_head(lengths)
+
+
+@pytest.mark.parametrize("heads,kv_heads,head_dim", [(28, 4, 128), (32, 4, 64), (20, 2, 64)])
+def test_decode_step_of_many_samples_equals_its_samples_alone(heads, kv_heads, head_dim):
+    """Grouped KV heads: a batch whose blocks share SMs walks its caches 32 positions a step, a single sample 128; the
+    order of every sum is the same, so are the bits. Caches around the eight runs' and the steps' lengths."""
+    dims = synth.reduced(synth.WORKLOADS["qwen"].dims, n_layers=1, vocab=512, d_model=heads * head_dim, n_heads=heads,
+                         n_kv_heads=kv_heads, d_ffn=1024, c_vis=heads * head_dim, n_groups=2)
+    m, _ = _model(dims, 101, max_seq=2048)
+    lens = [0, 1, 7, 8, 31, 32, 255, 256, 257, 300, 511, 513, 1023, 1024, 1025, 1500] * 2
+    B, max_len, i32 = len(lens), 1600, dict(dtype=torch.int32, device="cuda")
+    kv = _rand(2, 1, B, max_len, dims.d_kv, seed=102)
+
+    def step(rows):
+        n = len(rows)
+        cache = kv[:, :, rows].contiguous()
+        tok, length = torch.tensor(rows, **i32), torch.tensor([lens[r] for r in rows], **i32)
+        lg = torch.ones(n, 1, dtype=torch.uint8, device="cuda")
+        gg = torch.ones(n, 1, dims.n_groups, dtype=torch.uint8, device="cuda")
+        logits, nxt = torch.empty(n, dims.vocab, device="cuda"), torch.empty(n, **i32)
+        ws = torch.empty(svl.svl_decode_workspace_size(m.handle, n), dtype=torch.uint8, device="cuda")
+        svl.svl_decode_step(m.handle, n, tok, cache, max_len, length, lg, gg, logits, nxt, ws, ws.numel())
+        assert svl.svl_get_device_status(m.handle) == 0
+        return logits, nxt, cache
+
+    whole = step(list(range(B)))
+    for r in range(B):
+        one = step([r])
+        assert torch.equal(whole[0][r], one[0][0]) and torch.equal(whole[2][:, :, r], one[2][:, :, 0]), lens[r]
+    m.close()
