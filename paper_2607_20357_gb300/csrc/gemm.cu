@@ -156,7 +156,7 @@ SVL_DEVINL void set_abort(volatile int* abort, uint32_t* status) {
 
 // Stage geometry per epilogue: the token-score GEMM streams the features
 // once and reads a B box of only H rows per stage (H <= 64: 24 KB stages,
-// nine deep; H <= 128: 32 KB, six deep), keeping more feature bytes in flight.
+// eight deep; H <= 128: 32 KB, six deep), keeping more feature bytes in flight.
 // THIN launches (at most kThinRows rows of A, e.g. one row per sample in
 // decode) are weight-streaming: their A box is kThinRows rows, so a stage is
 // 36 KB and six of them keep 192 KB of weights in flight per SM. The MMA
@@ -203,12 +203,18 @@ struct StageCfg<EPI_GELU, true> {
 };
 template <>
 struct StageCfg<EPI_ROWMAP, true> : StageCfg<EPI_GELU, true> {};
+// Token scores: eight stages, not the nine that fit, so that the CTAs of the
+// selection behind it (18 KB of shared memory) start beside this kernel's and
+// wait there. With nine they started as its CTAs left one by one: 40 samples of
+// 576 tokens under the paper's rule 48.8 us (36.5 with eight), 16 of 3,000 116 (67).
 template <>
 struct StageCfg<EPI_SCORE, false> {
-  static constexpr int stages = 9;
+  static constexpr int stages = 8;
   static constexpr int abytes = kABytes;
   static constexpr int bytes = kABytes + kBHalfBytes / 2;
 };
+static_assert(StageCfg<EPI_SCORE, false>::stages * StageCfg<EPI_SCORE, false>::bytes <= (228 - 28) * 1024,
+              "room for a CTA of the selection");
 template <>
 struct StageCfg<EPI_SCORE_WIDE, false> {
   static constexpr int stages = 6;
