@@ -695,13 +695,14 @@ svl_status run_select(svl_model* m, const CtlCall& c, float* e_b, int* kept_loca
     const svl_status st = launch(d.h_ctrl <= 64 ? EPI_SCORE : EPI_SCORE_WIDE, m, SVL_TAG_SCORE, p, p.grid_m, s);
     if (st != SVL_OK) return st;
   }
-  Launch L1(m, SVL_TAG_SELECT, s);
-  if (c.rule == 0) {
-    launch_topk(c.B, c.scores, c.vis_off, c.k, c.kept_off, c.kept_idx, s);
-    return last_error();
-  }
-  launch_select(a, c.B, s);
   {
+    Launch L1(m, SVL_TAG_SELECT, s);
+    if (c.rule == 0)
+      launch_topk(c.B, c.scores, c.vis_off, c.k, c.kept_off, c.kept_idx, s);
+    else
+      launch_select(a, c.B, s);
+  }
+  if (c.rule != 0) {
     Launch L2(m, SVL_TAG_SELECT, s);
     launch_compact(c.B, c.vis_off, c.k, kept_local, c.kept_idx, c.kept_off, s);
   }
@@ -799,9 +800,11 @@ svl_status pack_impl(svl_model* m, int32_t B, int32_t n_vis_total, int32_t n_tex
   if (d.proj_hidden && n_vis_total > 0) {
     // 128-column tiles (six stages of 32 KB) while at most two thirds of the
     // SMs would have a 256-column one: a tile then takes half the time, and
-    // even every token kept makes no more than two waves of them (one request of
-    // 576 tokens, 5 x 16 wide tiles, over four layers: 828 us; 801 with these tiles and the
-    // controller's and the gather's launches merged)
+    // even with every token kept there are no more than two waves of them (the
+    // host knows the tokens given, not those kept; fewer rows make fewer tiles of
+    // either kind, and load_work halves wide ones that fill half a wave). One
+    // request of 576 tokens, 5 x 16 wide tiles, over four layers: 828 us; 801 with
+    // these tiles and the controller's and the gather's launches merged
     const int64_t wide = static_cast<int64_t>((n_vis_total + kBM - 1) / kBM) * ((d.d_model + 255) / 256);
     const bool narrow = 3 * wide <= 2 * m->num_sms;
     GemmParams p = base_params(m);

@@ -182,3 +182,35 @@ def test_packs_chained_through_their_rows():
         assert torch.equal(got["X"][:96], want)
     m.close()
     first.close()
+
+
+@pytest.mark.parametrize("gates", ["paper", "later"])
+def test_recorded_launch_times_do_not_overlap(gates):
+    """Each record covers its own launch: together they take no longer than the call. One sample that keeps all of its
+    60,000 tokens makes the compaction far longer than the gaps between launches."""
+    n = 60000
+    m = svl.GatedPrefill(TINY.dims, synth.make_weights(TINY.dims, 103, device="cuda"), max_seq=64)
+    b = synth.make_batch(TINY, 104, n_vis_list=[n], s_text_list=[1], keep_list=[n], device="cuda")
+    out = m.alloc_outputs(b)
+    ws, wsb = m.workspace(1, n, 1, stages=("select",))
+    logits = torch.ones(1, TINY.dims.n_layers, TINY.dims.n_groups, device="cuda")
+    lg, gg = (out["layer_gate"], out["group_gate"]) if gates == "paper" else (None, None)
+
+    def call():
+        svl.svl_score_select_paper(m.handle, 1, n, b["vis"], b["vis_off"], out["text_len"], b["budget"],
+                                   b["keep_count"], logits if gates == "paper" else None, out["scores"], out["k"],
+                                   out["kept_idx"], out["kept_off"], out["flags"], lg, gg, None, ws, wsb)
+
+    call()
+    for _ in range(5):
+        start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        svl.svl_profile_start(m.handle)
+        start.record()
+        call()
+        end.record()
+        svl.svl_profile_stop(m.handle)
+        end.synchronize()
+        launches = svl.svl_profile_launches(m.handle)
+        assert [t for t, _ in launches] == ["budget_embed", "score", "select", "select"]
+        assert sum(ms for _, ms in launches) <= start.elapsed_time(end), launches
+    m.close()
