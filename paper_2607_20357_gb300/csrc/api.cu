@@ -113,12 +113,12 @@ constexpr int kMaxPrefillBatch = 4096;  // samples per prefill call
 // a third less per MMA. The host knows the capacity only; the rows are what the
 // budgets leave of it. Forwards of four layers with room for 3,200 to 10,240 rows
 // at LLaVA-7B and Qwen2-VL-7B widths, single CTAs' time over pairs', every share of
-// the rows from 0.1 to 1: all groups on 1.01 to 1.10 but 0.98 at 5 and 7 row tiles
+// the rows from 0.1 to 1: all groups on 1.01 to 1.10, but 0.98 at 5 and 7 row tiles
 // (an odd tile has no partner) and 0.91 at 3 (a tenth of 3,200 rows); gates scaled
-// with the budget 1.00 to 1.07, but 0.97 at a tenth; 64 samples with budgets and
-// gates of their own 1.08 to 1.11. e4m3 models 0.91, 0.95 to 1.08 and 1.08. With
-// room for 1,024 to 2,048 rows, one layer's MLP and QKV + O gained -2 to +6 %; at
-// 320 the MLP lost 4 %.
+// with the budget 0.99 to 1.08, but 0.97 at a tenth; 64 samples with budgets and
+// gates of their own 1.08 to 1.11. e4m3 models 0.92 at 3 row tiles, 0.95 to 1.08
+// and 1.08. With room for 1,024 to 2,048 rows, one layer's MLP and QKV + O gained
+// -2 to +6 %; at 320 the MLP lost 4 %.
 constexpr int kPairRows = 3072;
 
 // Each call keeps its scratch at the start of the workspace: no data flows
