@@ -840,6 +840,7 @@ svl_status pack_impl(svl_model* m, int32_t B, int32_t n_vis_total, int32_t n_tex
     q.out[0] = X;
     q.ld[0] = d.d_model;
     q.row_map = a.row_map;
+    q.out_rows = a.t_cap;
     st = launch(EPI_ROWMAP, m, SVL_TAG_PROJECTOR, q, static_cast<int64_t>(q.grid_m) * q.grid_n, s, false, narrow);
     if (st != SVL_OK) return st;
   }

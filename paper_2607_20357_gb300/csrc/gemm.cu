@@ -518,6 +518,8 @@ SVL_DEVINL void epilogue_tile(const GemmParams& p, const TileInfo& ti, int row, 
     __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(p.out[0]);
     const size_t ld = static_cast<size_t>(p.ld[0]);
     const int orow = (KIND == EPI_ROWMAP && rv) ? p.row_map[row] : row;
+    // (rows of samples that the packing cut off have no entry in the map)
+    if (KIND == EPI_ROWMAP && static_cast<unsigned>(orow) >= static_cast<unsigned>(p.out_rows)) rv = false;
     for (int c = 0; c < ti.ncols; c += 32) {
       tmem_ld32(taddr + c, v);
       if (rv) {

@@ -66,7 +66,8 @@ struct GemmParams {
   // epilogue operands
   void* out[3];
   int ld[3];
-  const int* row_map;
+  const int* row_map;  // EPI_ROWMAP: row of out per row, skipped unless in [0, out_rows)
+  int out_rows;
   const int* pos;
   const float2* rope_cs;  // [d_head/2, rope_rows] (cos, sin), position fastest
   int rope_rows;

@@ -214,3 +214,26 @@ def test_recorded_launch_times_do_not_overlap(gates):
         assert [t for t, _ in launches] == ["budget_embed", "score", "select", "select"]
         assert sum(ms for _, ms in launches) <= start.elapsed_time(end), launches
     m.close()
+
+
+def test_pack_cuts_off_and_reports_rows_past_its_capacity():
+    """text_off that promises more rows than n_text_total: the rows past the capacity are cut off (kept visual rows of
+    the second sample among them, which the projector then has no place for), the others are as without the cut, and
+    the status word says so. Nothing past the capacity is written."""
+    dims = synth.reduced(LLAVA.dims, n_layers=1, vocab=512)
+    m = svl.GatedPrefill(dims, synth.make_weights(dims, 105, device="cuda"), max_seq=1024)
+    b = synth.make_batch(LLAVA, 106, n_vis_list=[100, 140], s_text_list=[200, 40], keep_list=[100, 140], dims=dims,
+                         device="cuda")
+    out = m.run(b, stages=("select", "pack"))
+    assert svl.svl_get_device_status(m.handle) == 0
+    want, D, n_text = out["X"].clone(), dims.d_model, 100  # 240 + 100 rows of 480
+    cap = 240 + n_text
+    ws = torch.full((svl.svl_workspace_size_for(m.handle, ("pack",), 2, 240, n_text),), 0x7F, dtype=torch.uint8,
+                    device="cuda")
+    X = torch.full((cap + 64, D), 7.0, dtype=torch.bfloat16, device="cuda")
+    svl.svl_pack(m.handle, 2, 240, n_text, b["vis"], b["vis_off"], out["kept_idx"], out["kept_off"], b["text_ids"],
+                 b["text_off"], X, out["cu_seqlens"], out["pos"], ws, ws.numel())
+    assert svl.svl_get_device_status(m.handle) == svl.SVL_DEV_BAD_INDEX
+    assert out["cu_seqlens"].tolist() == [0, 300, cap]
+    assert torch.equal(X[:cap], want[:cap]) and bool((X[cap:] == 7).all())
+    m.close()
